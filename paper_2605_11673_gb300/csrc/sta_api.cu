@@ -59,7 +59,7 @@ static void free_ctx(sta_ctx *x) {
     if (x->h_count) cudaFreeHost(x->h_count);
     if (x->c.h_count_mapped) cudaFreeHost(x->c.h_count_mapped);
     if (x->h2d_done) cudaEventDestroy(x->h2d_done);
-    if (x->c.g_cg) cudaGraphExecDestroy(x->c.g_cg);
+    if (x->c.h_cg) cudaFreeHost(x->c.h_cg);
     graph_release(&x->c);
     delete x;
 }

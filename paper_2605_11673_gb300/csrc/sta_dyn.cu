@@ -10,15 +10,9 @@
 // a streaming frame re-folds the nodes of its edited tetrahedra after the mask update; a
 // rebuild re-folds every node.
 //
-// Solve: conjugate gradients with the Jacobi preconditioner (the paper's solver: CG with
-// diagonal preconditioning), on the free DOFs -- not clamped, of a node with mass; a clamped
-// DOF stays 0, a DOF of a node without mass keeps its displacement with velocity 0.  Start:
-// x = u_t.  Stop: ||r|| <= tol ||b|| or max_iter.  A x = m x + h^2 (K x) is applied without
-// forming the matrix, one thread per node over its three rows (they share their columns).
-// Every dot product is a fixed-order reduction (warp tree, warps in order, CTAs in order by the
-// last CTA to arrive), so a solve is deterministic for a given context.  Iterations run in
-// captured chunks of CG_CHUNK (2 launches each: the SpMV of z also forms p = z + beta p and
-// q = A z + beta q = A p, then the update); the host reads the state between chunks.
+// Solve: conjugate gradients with the Jacobi preconditioner (sta_cg.cu) on the free DOFs -- not
+// clamped, of a node with mass; a clamped DOF stays 0, a DOF of a node without mass keeps its
+// displacement with velocity 0.  Start: x = u_t.  Stop: ||r|| <= tol ||b|| or max_iter.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -29,15 +23,6 @@ namespace sta {
 namespace {
 
 constexpr int DYN_TPB = 256;
-constexpr int DYN_WARPS = DYN_TPB / 32;
-constexpr int CG_CHUNK = 8;
-
-// Device state of one step's solve.
-struct CgState {
-    double rz, pq, rr, bb, alpha, beta, tol2, pad0;
-    int32_t iters, max_iter, done, pad1;
-    unsigned int arrive[4];  // last-CTA counters: spmv, r0, update, spare
-};
 
 // -------------------------------------------------------------------------------- mass
 
@@ -103,41 +88,6 @@ __global__ void k_dyn_mass_edited(const int32_t *__restrict__ edited, int64_t m,
 
 // -------------------------------------------------------------------------------- CG
 
-// Sum over the CTA in a fixed order; the result is valid in thread 0.
-__device__ __forceinline__ double cta_sum(double v, double *sh) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-    __syncthreads();
-    return t;
-}
-
-// Thread 0 has stored this CTA's partials; true (in every thread) in the last CTA to arrive,
-// once all partials are visible.  The last CTA resets the counter for the next use.
-__device__ __forceinline__ bool last_cta(unsigned int *arrive) {
-    __shared__ bool last;
-    __threadfence();
-    if (threadIdx.x == 0) last = atomicAdd(arrive, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (last) __threadfence();
-    return last;
-}
-
-// In the last CTA (every thread calls it): the sum of the n per-CTA partials, each thread over
-// a fixed stride of them, then the CTA tree; valid in thread 0.
-__device__ __forceinline__ double sum_parts(const double *part, int n, double *sh) {
-    double t = 0.0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) t += __ldcg(part + i);
-    return cta_sum(t, sh);
-}
-
-__device__ __forceinline__ bool cg_stopped(const CgState *st) {
-    return st->done || st->iters >= st->max_iter;
-}
-
 // b, x0 = u, Jacobi inverse diagonal and the free flags, per DOF.
 __global__ void k_cg_init(int64_t n3, const int32_t *__restrict__ adj_ptr,
                           const int32_t *__restrict__ adj, const int32_t *__restrict__ row_ptr,
@@ -177,21 +127,15 @@ __global__ void k_cg_init(int64_t n3, const int32_t *__restrict__ adj_ptr,
 // instruction for a whole warp whatever its active lanes, and the FP64 pipe is the scarce unit
 // here, so every lane works on its own entries and the only cross-lane adds are the two quad
 // levels.  The nodes are taken in the order `perm` (ascending row length), so that the eight
-// nodes of a warp have rows of nearly one length.  With `dots`, the last CTA forms p.q and
-// alpha = rz / pq.
+// nodes of a warp have rows of nearly one length.
 __global__ void __launch_bounds__(DYN_TPB)
-k_cg_spmv(int64_t n, const int32_t *__restrict__ perm, const int32_t *__restrict__ row_ptr,
-          const int32_t *__restrict__ col, const double *__restrict__ val,
-          const double *__restrict__ mass, double h2, const uint8_t *__restrict__ fr,
-          const double *__restrict__ xin, double *__restrict__ qout, double *__restrict__ part,
-          CgState *st, bool dots, double *__restrict__ p) {
-    __shared__ double sh[DYN_WARPS];
-    if (dots && cg_stopped(st)) return;
-    const double beta = p ? st->beta : 0.0;
+k_dyn_spmv(int64_t n, const int32_t *__restrict__ perm, const int32_t *__restrict__ row_ptr,
+           const int32_t *__restrict__ col, const double *__restrict__ val,
+           const double *__restrict__ mass, double h2, const uint8_t *__restrict__ fr,
+           const double *__restrict__ xin, double *__restrict__ qout) {
     const int lane = threadIdx.x & 31, qd = lane & 3;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    double pq = 0.0;
     for (int64_t base = 8 * warp; base < n; base += 8 * nwarps) {  // warp-uniform
         const int64_t j = base + (lane >> 2);
         double s0 = 0.0, s1 = 0.0, s2 = 0.0;
@@ -234,112 +178,11 @@ k_cg_spmv(int64_t n, const int32_t *__restrict__ perm, const int32_t *__restrict
         }
         if (a >= 0 && qd < 3) {
             const int64_t d = 3 * a + qd;
-            const double xd = xin[d];
             const double sd = qd == 0 ? s0 : (qd == 1 ? s1 : s2);
-            double q = fr[d] ? __fma_rn(mass[a], xd, h2 * sd) : 0.0;
-            if (p) {  // CG step: xin = z, p = z + beta p, q = A z + beta q = A p
-                const double pd = __fma_rn(beta, p[d], xd);
-                q = __fma_rn(beta, qout[d], q);
-                p[d] = pd;
-                qout[d] = q;
-                pq = __fma_rn(pd, q, pq);
-            } else {
-                qout[d] = q;
-                pq = __fma_rn(xd, q, pq);
-            }
-        }
-    }
-    if (!dots) return;
-    const double t = cta_sum(pq, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-    if (last_cta(&st->arrive[0])) {
-        const double s = sum_parts(part, gridDim.x, sh);
-        if (threadIdx.x == 0) {
-            st->pq = s;
-            if (s > 0.0) st->alpha = st->rz / s;
-            else st->done = 1;  // breakdown: p = 0 (already converged) or A not positive definite
-            st->arrive[0] = 0u;
+            qout[d] = fr[d] ? __fma_rn(mass[a], xin[d], h2 * sd) : 0.0;
         }
     }
 }
-
-// r = b - q, z = D^-1 r, p = q = 0; rz, rr, bb; the convergence test.
-__global__ void __launch_bounds__(DYN_TPB)
-k_cg_r0(int64_t n3, const double *__restrict__ b, double *__restrict__ q,
-        const double *__restrict__ dinv, double *__restrict__ r, double *__restrict__ z,
-        double *__restrict__ p, double *__restrict__ part, CgState *st) {
-    __shared__ double sh[DYN_WARPS];
-    double rz = 0.0, rr = 0.0, bb = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const double ri = b[i] - q[i], zi = dinv[i] * ri;
-        r[i] = ri;
-        z[i] = zi;
-        p[i] = 0.0;  // with beta = 0 the first step forms p = z and q = A z
-        q[i] = 0.0;
-        rz = __fma_rn(ri, zi, rz);
-        rr = __fma_rn(ri, ri, rr);
-        bb = __fma_rn(b[i], b[i], bb);
-    }
-    const double a0 = cta_sum(rz, sh), a1 = cta_sum(rr, sh), a2 = cta_sum(bb, sh);
-    if (threadIdx.x == 0) {
-        part[blockIdx.x] = a0;
-        part[gridDim.x + blockIdx.x] = a1;
-        part[2 * gridDim.x + blockIdx.x] = a2;
-    }
-    if (last_cta(&st->arrive[1])) {
-        const double s0 = sum_parts(part, gridDim.x, sh);
-        const double s1 = sum_parts(part + gridDim.x, gridDim.x, sh);
-        const double s2 = sum_parts(part + 2 * gridDim.x, gridDim.x, sh);
-        if (threadIdx.x == 0) {
-            st->rz = s0;
-            st->rr = s1;
-            st->bb = s2;
-            st->beta = 0.0;
-            st->iters = 0;
-            st->done = s1 <= st->tol2 * s2 ? 1 : 0;
-            st->arrive[1] = 0u;
-        }
-    }
-}
-
-// x += alpha p, r -= alpha q, z = D^-1 r; rz, rr; beta, the iteration count, the test.
-__global__ void __launch_bounds__(DYN_TPB)
-k_cg_update(int64_t n3, double *__restrict__ x, double *__restrict__ r, double *__restrict__ z,
-            const double *__restrict__ p, const double *__restrict__ q,
-            const double *__restrict__ dinv, double *__restrict__ part, CgState *st) {
-    __shared__ double sh[DYN_WARPS];
-    if (cg_stopped(st)) return;
-    const double alpha = st->alpha;
-    double rz = 0.0, rr = 0.0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        x[i] = __fma_rn(alpha, p[i], x[i]);
-        const double ri = __fma_rn(-alpha, q[i], r[i]), zi = dinv[i] * ri;
-        r[i] = ri;
-        z[i] = zi;
-        rz = __fma_rn(ri, zi, rz);
-        rr = __fma_rn(ri, ri, rr);
-    }
-    const double a0 = cta_sum(rz, sh), a1 = cta_sum(rr, sh);
-    if (threadIdx.x == 0) {
-        part[blockIdx.x] = a0;
-        part[gridDim.x + blockIdx.x] = a1;
-    }
-    if (last_cta(&st->arrive[2])) {
-        const double rzn = sum_parts(part, gridDim.x, sh);
-        const double rrn = sum_parts(part + gridDim.x, gridDim.x, sh);
-        if (threadIdx.x == 0) {
-            st->rr = rrn;
-            st->beta = st->rz != 0.0 ? rzn / st->rz : 0.0;
-            st->rz = rzn;
-            st->iters += 1;
-            if (rrn <= st->tol2 * st->bb) st->done = 1;
-            st->arrive[2] = 0u;
-        }
-    }
-}
-
 
 // Static solve (sta_solve): b, x0 and the Jacobi inverse diagonal on the caller's free DOFs.
 __global__ void k_cg_init_static(int64_t n3, const int32_t *__restrict__ adj_ptr,
@@ -387,61 +230,6 @@ __global__ void k_cg_init_scalar(int64_t n, const int32_t *__restrict__ pdiag,
     }
 }
 
-// q = A x on the free rows of a scalar operator, four lanes per row (rows in the order `perm`,
-// ascending length), each row's lanes adding their partial sums as (s0 + s1) + (s2 + s3).
-// With `dots`, the last CTA forms p.q and alpha = rz / pq.
-__global__ void __launch_bounds__(DYN_TPB)
-k_cg_spmv_scalar(int64_t n, const int32_t *__restrict__ perm, const int32_t *__restrict__ row_ptr,
-                 const int32_t *__restrict__ col, const double *__restrict__ val,
-                 const uint8_t *__restrict__ fr, const double *__restrict__ xin,
-                 double *__restrict__ qout, double *__restrict__ part, CgState *st, bool dots,
-                 double *__restrict__ p) {
-    __shared__ double sh[DYN_WARPS];
-    if (dots && cg_stopped(st)) return;
-    const double beta = p ? st->beta : 0.0;
-    const int lane = threadIdx.x & 31, qd = lane & 3;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    double pq = 0.0;
-    for (int64_t base = 8 * warp; base < n; base += 8 * nwarps) {  // warp-uniform
-        const int64_t j = base + (lane >> 2);
-        double acc = 0.0;
-        int64_t a = -1;
-        if (j < n) {
-            a = perm[j];
-            const int32_t r0 = row_ptr[a], r1 = row_ptr[a + 1];
-            for (int32_t k = r0 + qd; k < r1; k += 4) acc = __fma_rn(val[k], xin[col[k]], acc);
-        }
-        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-        if (a >= 0 && qd == 0) {
-            double q = fr[a] ? acc : 0.0;
-            if (p) {  // CG step: xin = z, p = z + beta p, q = A z + beta q = A p
-                const double pa = __fma_rn(beta, p[a], xin[a]);
-                q = __fma_rn(beta, qout[a], q);
-                p[a] = pa;
-                qout[a] = q;
-                pq = __fma_rn(pa, q, pq);
-            } else {
-                qout[a] = q;
-                pq = __fma_rn(xin[a], q, pq);
-            }
-        }
-    }
-    if (!dots) return;
-    const double t = cta_sum(pq, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = t;
-    if (last_cta(&st->arrive[0])) {
-        const double s = sum_parts(part, gridDim.x, sh);
-        if (threadIdx.x == 0) {
-            st->pq = s;
-            if (s > 0.0) st->alpha = st->rz / s;
-            else st->done = 1;
-            st->arrive[0] = 0u;
-        }
-    }
-}
-
 // The adjoint rule of a solve (A_ff u_f = f_f): dL/dA_ij = -lam_i u_j on entries between free
 // DOFs, 0 elsewhere.  One thread per row.
 __global__ void k_outer_grad(int64_t nrows, const int32_t *__restrict__ row_ptr,
@@ -469,22 +257,6 @@ __global__ void k_dyn_restrict(int64_t n3, const double *__restrict__ mass,
         const bool free = !clamped[a] && mass[a] > 0.0;
         fr[i] = free ? 1 : 0;
         xf[i] = free ? x[i] : 0.0;
-    }
-}
-
-// u, v from the solution.
-__global__ void k_dyn_advance(int64_t n3, double *__restrict__ u, double *__restrict__ v,
-                              const double *__restrict__ x, const uint8_t *__restrict__ fr,
-                              const uint8_t *__restrict__ clamped, double h) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        if (fr[i]) {
-            v[i] = (x[i] - u[i]) / h;
-            u[i] = x[i];
-        } else {
-            v[i] = 0.0;
-            if (clamped[i / 3]) u[i] = 0.0;
-        }
     }
 }
 
@@ -523,140 +295,18 @@ int launch_dyn_qmass(Ctx *c, cudaStream_t s) {
     return STA_OK;
 }
 
-namespace {
-
-// One chunk of CG_CHUNK iterations (2 launches each) of A = diag(mass) + h2 K(val), launched
-// or captured on s.
-int cg_chunk(Ctx *c, const double *val, const double *mass, double h2, cudaStream_t s) {
-    const int64_t n3 = c->nrows;  // DOFs: 3 per node, or 1 for the scalar proxy operator
-    const unsigned gv = c->cg_grid;
-    double *x = c->cg, *b = x + n3, *r = b + n3, *z = r + n3, *p = z + n3, *q = p + n3;
-    double *dinv = q + n3;
-    CgState *st = reinterpret_cast<CgState *>(c->cg_state);
-    for (int it = 0; it < CG_CHUNK; ++it) {
-        if (c->op == STA_OP_PROXY)
-            k_cg_spmv_scalar<<<gv, DYN_TPB, 0, s>>>(c->n, c->dyn_perm, c->row_ptr, c->col, val,
-                                                    c->cg_free, z, q, c->cg_part, st, true, p);
-        else
-            k_cg_spmv<<<gv, DYN_TPB, 0, s>>>(c->n, c->dyn_perm, c->row_ptr, c->col, val, mass, h2,
-                                            c->cg_free, z, q, c->cg_part, st, true, p);
-        k_cg_update<<<gv, DYN_TPB, 0, s>>>(n3, x, r, z, p, q, dinv, c->cg_part, st);
-    }
-    STA_CUDA_TRY(cudaGetLastError());
-    return STA_OK;
-}
-
-}  // namespace
-
-namespace {
-
-// CG iterations in chunks until converged or max_iter: the captured chunk `g` if given, else
-// direct launches of the chunk for (val, mass, h2).  The host reads the state between chunks;
-// with `stagnate`, it also stops once the residual has not halved for 1000 iterations (the
-// attainable accuracy reached).
-int cg_iterate(Ctx *c, cudaGraphExec_t g, const double *val, const double *mass, double h2,
-               int32_t max_iter, bool stagnate, cudaStream_t s, CgState *hs) {
-    CgState *st = reinterpret_cast<CgState *>(c->cg_state);
-    double best = -1.0;
-    int32_t best_it = 0;
-    // the first chunk goes out with the initial residual (its kernels return at once if that is
-    // already converged or max_iter is 0): one host round trip fewer per solve
-    if (c->n > 0) {
-        if (g) STA_CUDA_TRY(cudaGraphLaunch(g, s));
-        else STA_TRY(cg_chunk(c, val, mass, h2, s));
-    }
-    for (;;) {
-        if (c->n > 0) {
-            STA_CUDA_TRY(cudaMemcpyAsync(hs, st, sizeof *hs, cudaMemcpyDeviceToHost, s));
-            STA_CUDA_TRY(cudaStreamSynchronize(s));
-        }
-        if (c->n == 0 || hs->done || hs->iters >= max_iter) break;
-        if (stagnate) {
-            if (best < 0.0 || hs->rr < 0.25 * best) {
-                best = hs->rr;
-                best_it = hs->iters;
-            } else if (hs->iters - best_it > 1000) {
-                break;
-            }
-        }
-        if (g) STA_CUDA_TRY(cudaGraphLaunch(g, s));
-        else STA_TRY(cg_chunk(c, val, mass, h2, s));
-    }
-    return STA_OK;
-}
-
-}  // namespace
-
-// The CG buffers shared by the implicit-Euler step and the static solve, allocated once.
-int cg_alloc(Ctx *c) {
-    if (c->cg) return STA_OK;
-    const int64_t n = c->n, n3 = c->nrows;  // DOFs
-    const int rows = c->op == STA_OP_PROXY ? 1 : 3;  // rows per node
-    c->cg_grid = (int)dyn_grid(c, n3 > 0 ? n3 : 1);
-    STA_TRY(dev_alloc(c, &c->cg, 7 * n3));
-    STA_TRY(dev_alloc(c, &c->cg_free, n3));
-    STA_TRY(dev_alloc(c, &c->cg_part, 3 * (int64_t)c->cg_grid));
-    STA_TRY(dev_alloc(c, &c->cg_state, (int64_t)sizeof(CgState)));
-    STA_TRY(dev_alloc(c, &c->cg_zero, n));
-    STA_CUDA_TRY(cudaMemset(c->cg_zero, 0, sizeof(double) * (size_t)(n > 0 ? n : 1)));
-    // the SpMV's node order: ascending row length (ties by node id)
+// sta_dyn_apply's node order: ascending row length (ties by node id).
+static int dyn_order(Ctx *c) {
+    if (c->dyn_perm) return STA_OK;
+    const int64_t n = c->n;
     STA_TRY(dev_alloc(c, &c->dyn_perm, n));
-    std::vector<int32_t> rp(rows * n + 1), perm(n);
-    STA_CUDA_TRY(cudaMemcpy(rp.data(), c->row_ptr, sizeof(int32_t) * (rows * n + 1),
-                            cudaMemcpyDeviceToHost));
+    std::vector<int32_t> rp(3 * n + 1), perm(n);
+    STA_CUDA_TRY(cudaMemcpy(rp.data(), c->row_ptr, sizeof(int32_t) * (3 * n + 1), cudaMemcpyDeviceToHost));
     for (int64_t a = 0; a < n; ++a) perm[a] = (int32_t)a;
     std::stable_sort(perm.begin(), perm.end(), [&](int32_t p, int32_t q) {
-        return rp[rows * p + rows] - rp[rows * p] < rp[rows * q + rows] - rp[rows * q];
+        return rp[3 * p + 3] - rp[3 * p] < rp[3 * q + 3] - rp[3 * q];
     });
     STA_CUDA_TRY(cudaMemcpy(c->dyn_perm, perm.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice));
-    return STA_OK;
-}
-
-int launch_dyn_step(Ctx *c, double tol, int32_t max_iter, int32_t *iters, double *rel_res,
-                    cudaStream_t s) {
-    const int64_t n3 = 3 * c->n;
-    const unsigned gv = c->cg_grid;
-    double *x = c->cg, *b = x + n3, *r = b + n3, *z = r + n3, *p = z + n3, *q = p + n3;
-    double *dinv = q + n3;
-    CgState *st = reinterpret_cast<CgState *>(c->cg_state);
-    CgState h0 = {};
-    h0.tol2 = tol * tol;
-    h0.max_iter = max_iter;
-    STA_CUDA_TRY(cudaMemcpyAsync(st, &h0, sizeof h0, cudaMemcpyHostToDevice, s));
-    if (n3 > 0) {
-        k_cg_init<<<gv, DYN_TPB, 0, s>>>(n3, c->adj_ptr, c->adj, c->row_ptr, c->val, c->mass,
-                                         c->clamped, c->du, c->dv, c->df, c->dyn_h, x, b, dinv,
-                                         c->cg_free);
-        k_cg_spmv<<<gv, DYN_TPB, 0, s>>>(c->n, c->dyn_perm, c->row_ptr, c->col, c->val, c->mass,
-                                        c->dyn_h * c->dyn_h, c->cg_free, x, q, c->cg_part, st, false, nullptr);
-        k_cg_r0<<<gv, DYN_TPB, 0, s>>>(n3, b, q, dinv, r, z, p, c->cg_part, st);
-        STA_CUDA_TRY(cudaGetLastError());
-    }
-    if (!c->g_cg) {  // capture the chunk once (the context's buffers never move)
-        cudaStream_t cs = nullptr;
-        STA_CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-        cudaGraph_t g = nullptr;
-        cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-        int rc = e == cudaSuccess ? cg_chunk(c, c->val, c->mass, c->dyn_h * c->dyn_h, cs) : STA_ECUDA;
-        cudaError_t e2 = cudaStreamEndCapture(cs, &g);
-        if (rc == STA_OK && e == cudaSuccess && e2 == cudaSuccess)
-            e2 = cudaGraphInstantiate(&c->g_cg, g, 0);
-        if (g) cudaGraphDestroy(g);
-        cudaStreamDestroy(cs);
-        if (rc != STA_OK || e != cudaSuccess || e2 != cudaSuccess) {
-            c->g_cg = nullptr;
-            return fail(STA_ECUDA, "CG chunk capture failed");
-        }
-    }
-    CgState hs = {};
-    STA_TRY(cg_iterate(c, c->g_cg, nullptr, nullptr, 0.0, max_iter, false, s, &hs));
-    if (n3 > 0) {
-        k_dyn_advance<<<gv, DYN_TPB, 0, s>>>(n3, c->du, c->dv, x, c->cg_free, c->clamped, c->dyn_h);
-        STA_CUDA_TRY(cudaGetLastError());
-        STA_CUDA_TRY(cudaStreamSynchronize(s));
-    }
-    if (iters) *iters = hs.iters;
-    if (rel_res) *rel_res = hs.bb > 0.0 ? std::sqrt(hs.rr / hs.bb) : 0.0;
     return STA_OK;
 }
 
@@ -683,6 +333,7 @@ extern "C" int sta_dyn_setup(sta_ctx *x, double rho, double h, const double *f,
         STA_TRY(dev_alloc(c, &c->clamped, n));
     }
     STA_TRY(cg_alloc(c));
+    STA_TRY(dyn_order(c));
     std::vector<double> hf(n3 > 0 ? n3 : 1, 0.0);
     std::vector<uint8_t> hc(n > 0 ? n : 1, 0);
     if (f) std::copy(f, f + n3, hf.begin());
@@ -692,10 +343,6 @@ extern "C" int sta_dyn_setup(sta_ctx *x, double rho, double h, const double *f,
     STA_CUDA_TRY(cudaMemcpyAsync(c->clamped, hc.data(), (size_t)n, cudaMemcpyHostToDevice, s));
     STA_CUDA_TRY(cudaMemsetAsync(c->du, 0, sizeof(double) * (size_t)(n3 > 0 ? n3 : 1), s));
     STA_CUDA_TRY(cudaMemsetAsync(c->dv, 0, sizeof(double) * (size_t)(n3 > 0 ? n3 : 1), s));
-    if (c->g_cg) {  // the captured CG chunk holds h^2: capture again on the next step
-        cudaGraphExecDestroy(c->g_cg);
-        c->g_cg = nullptr;
-    }
     c->dyn = true;
     c->dyn_rho = rho;
     c->dyn_h = h;
@@ -711,7 +358,20 @@ extern "C" int sta_dyn_step(sta_ctx *x, double tol, int32_t max_iter, int32_t *i
     Ctx *c = &x->c;
     if (!c->dyn) return fail(STA_ESTATE, "call sta_dyn_setup first");
     if (!(tol >= 0.0) || max_iter < 0) return fail(STA_EINVAL, "tol and max_iter must be >= 0");
-    return launch_dyn_step(c, tol, max_iter, iters, rel_res, (cudaStream_t)stream);
+    cudaStream_t s = (cudaStream_t)stream;
+    const int64_t n3 = 3 * c->n;
+    CgResult res{};
+    if (n3 > 0) {
+        k_cg_init<<<dyn_grid(c, n3), DYN_TPB, 0, s>>>(n3, c->adj_ptr, c->adj, c->row_ptr, c->val, c->mass,
+                                                      c->clamped, c->du, c->dv, c->df, c->dyn_h, c->cg,
+                                                      c->cg + n3, c->cg + 2 * n3, c->cg_free);
+        STA_CUDA_TRY(cudaGetLastError());
+        STA_TRY(launch_cg_solve(c, c->val, c->mass, c->dyn_h * c->dyn_h, tol, max_iter, false, nullptr,
+                                true, s, &res));
+    }
+    if (iters) *iters = res.iters;
+    if (rel_res) *rel_res = res.bb > 0.0 ? std::sqrt(res.rr / res.bb) : 0.0;
+    return STA_OK;
 }
 
 extern "C" int sta_dyn_apply(sta_ctx *x, const double *xv, double *y, void *stream) {
@@ -722,12 +382,11 @@ extern "C" int sta_dyn_apply(sta_ctx *x, const double *xv, double *y, void *stre
     if (n3 == 0) return STA_OK;
     if (!xv || !y) return fail(STA_EINVAL, "NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
-    double *xf = c->cg + 4 * n3;  // the CG's p buffer (free between steps)
-    const unsigned gv = (unsigned)c->cg_grid;
+    double *xf = c->cg + 3 * n3;  // the solve's z buffer (free between steps)
+    const unsigned gv = dyn_grid(c, n3);
     k_dyn_restrict<<<gv, DYN_TPB, 0, s>>>(n3, c->mass, c->clamped, xv, xf, c->cg_free);
-    k_cg_spmv<<<gv, DYN_TPB, 0, s>>>(c->n, c->dyn_perm, c->row_ptr, c->col, c->val, c->mass,
-                                    c->dyn_h * c->dyn_h, c->cg_free, xf, y, c->cg_part,
-                                    reinterpret_cast<CgState *>(c->cg_state), false, nullptr);
+    k_dyn_spmv<<<gv, DYN_TPB, 0, s>>>(c->n, c->dyn_perm, c->row_ptr, c->col, c->val, c->mass,
+                                     c->dyn_h * c->dyn_h, c->cg_free, xf, y);
     STA_CUDA_TRY(cudaGetLastError());
     return STA_OK;
 }
@@ -743,35 +402,21 @@ extern "C" int sta_solve(sta_ctx *x, const double *val, const double *b, const u
     cudaStream_t s = (cudaStream_t)stream;
     STA_TRY(cg_alloc(c));
     const double *A = val ? val : c->val;
-    double *xw = c->cg, *bw = xw + n3, *r = bw + n3, *z = r + n3, *p = z + n3, *q = p + n3;
-    double *dinv = q + n3;
-    CgState *st = reinterpret_cast<CgState *>(c->cg_state);
-    CgState h0 = {};
-    h0.tol2 = tol * tol;
-    h0.max_iter = max_iter;
-    STA_CUDA_TRY(cudaMemcpyAsync(st, &h0, sizeof h0, cudaMemcpyHostToDevice, s));
-    CgState hs = {};
+    CgResult res{};
     if (n3 > 0) {
-        const unsigned gv = (unsigned)c->cg_grid;
-        if (c->op == STA_OP_PROXY) {
+        const unsigned gv = dyn_grid(c, n3);
+        double *xw = c->cg, *bw = xw + n3, *dinv = bw + n3;
+        if (c->op == STA_OP_PROXY)
             k_cg_init_scalar<<<gv, DYN_TPB, 0, s>>>(n3, c->pdiag, A, free, b, xv, xw, bw, dinv,
                                                     c->cg_free);
-            k_cg_spmv_scalar<<<gv, DYN_TPB, 0, s>>>(c->n, c->dyn_perm, c->row_ptr, c->col, A,
-                                                    c->cg_free, xw, q, c->cg_part, st, false, nullptr);
-        } else {
+        else
             k_cg_init_static<<<gv, DYN_TPB, 0, s>>>(n3, c->adj_ptr, c->adj, c->row_ptr, A, free, b,
                                                     xv, xw, bw, dinv, c->cg_free);
-            k_cg_spmv<<<gv, DYN_TPB, 0, s>>>(c->n, c->dyn_perm, c->row_ptr, c->col, A, c->cg_zero,
-                                            1.0, c->cg_free, xw, q, c->cg_part, st, false, nullptr);
-        }
-        k_cg_r0<<<gv, DYN_TPB, 0, s>>>(n3, bw, q, dinv, r, z, p, c->cg_part, st);
         STA_CUDA_TRY(cudaGetLastError());
-        STA_TRY(cg_iterate(c, nullptr, A, c->cg_zero, 1.0, max_iter, true, s, &hs));
-        STA_CUDA_TRY(cudaMemcpyAsync(xv, xw, sizeof(double) * n3, cudaMemcpyDeviceToDevice, s));
-        STA_CUDA_TRY(cudaStreamSynchronize(s));
+        STA_TRY(launch_cg_solve(c, A, nullptr, 1.0, tol, max_iter, true, xv, false, s, &res));
     }
-    if (iters) *iters = hs.iters;
-    if (rel_res) *rel_res = hs.bb > 0.0 ? std::sqrt(hs.rr / hs.bb) : 0.0;
+    if (iters) *iters = res.iters;
+    if (rel_res) *rel_res = res.bb > 0.0 ? std::sqrt(res.rr / res.bb) : 0.0;
     return STA_OK;
 }
 

@@ -130,6 +130,12 @@ inline size_t frame_bytes(int64_t m) { return sizeof(FrameHeader) + sizeof(int32
 constexpr int STA_OP_ELASTICITY = 0;
 constexpr int STA_OP_PROXY = 1;
 
+// What a solve leaves for the host.
+struct CgResult {
+    double rr, bb;       // ||r||^2 at exit, ||b||^2
+    int32_t iters, failed;
+};
+
 struct Ctx {
     int op = STA_OP_ELASTICITY;
     int64_t n = 0, T = 0, nblocks = 0, nnz = 0, nrows = 0;
@@ -221,14 +227,21 @@ struct Ctx {
     double *mass = nullptr;     // n: lumped mass per node, maintained with the mask
     double *du = nullptr, *dv = nullptr, *df = nullptr;  // 3n: displacement, velocity, load
     uint8_t *clamped = nullptr; // n
-    double *cg = nullptr;       // 7 x 3n: x, b, r, z, p, q, D^-1
-    uint8_t *cg_free = nullptr; // 3n: DOF solved for
-    double *cg_part = nullptr;  // 3 x cg_grid: per-CTA partial sums
-    unsigned char *cg_state = nullptr;  // the solve's device scalars
-    int32_t *dyn_perm = nullptr;  // n: the CG SpMV's node order (ascending row length)
-    double *cg_zero = nullptr;    // n zeros: the mass term of a static solve (sta_solve)
-    int cg_grid = 0;
-    cudaGraphExec_t g_cg = nullptr;     // one captured chunk of CG iterations
+    int32_t *dyn_perm = nullptr;  // n: sta_dyn_apply's node order (ascending row length)
+
+    // conjugate gradients (sta_cg.cu), allocated by the first sta_dyn_setup or sta_solve
+    double *cg = nullptr;       // 4 x nrows: x, b, D^-1, z
+    uint8_t *cg_free = nullptr; // nrows: DOF solved for
+    int32_t *cg_snode = nullptr, *cg_sbase = nullptr, *cg_cta = nullptr, *cg_col = nullptr;  // slice plan
+    double *cg_val = nullptr;   // the matrix of a solve in slice order
+    double *cg_vec = nullptr;   // vectors in slice order when shared memory does not hold them
+    void *cg_slots = nullptr;   // words of the grid-wide sums
+    unsigned long long cg_epoch = 0;  // number of the last grid-wide sum given out
+    int cg_grid = 0, cg_S = 1, cg_warps = 1;
+    int64_t cg_slices = 0, cg_steps = 0;
+    bool cg_resident = false;   // the matrix is kept in shared memory
+    size_t cg_smem = 0;
+    CgResult *h_cg = nullptr, *d_cg = nullptr;  // host-mapped: a solve's result
 
     // CUDA-graph mode (sta_graph_enable): captured frame sequences and fixed staging
     bool graph_on = false;
@@ -315,8 +328,10 @@ int launch_dyn_qmass(Ctx *c, cudaStream_t s);     // sta_dyn.cu (no-ops unless s
 int launch_dyn_mass_all(Ctx *c, cudaStream_t s);
 int launch_dyn_mass_edited(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_dev,
                            int64_t cap, cudaStream_t s);
-int launch_dyn_step(Ctx *c, double tol, int32_t max_iter, int32_t *iters, double *rel_res,
-                    cudaStream_t s);
+int cg_alloc(Ctx *c);                              // sta_cg.cu
+int launch_cg_solve(Ctx *c, const double *val, const double *mass, double h2, double tol,
+                    int32_t max_iter, bool stagnate, double *xout, bool advance, cudaStream_t s,
+                    CgResult *res);
 int build_proxy_maps(Ctx *c, const int32_t *tblk, cudaStream_t s);  // sta_proxy.cu
 int launch_proxy_rebuild(Ctx *c, cudaStream_t s);
 int launch_proxy_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_dev,
