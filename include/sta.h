@@ -229,8 +229,8 @@ int sta_element_matrices(sta_ctx *ctx, const int32_t *tet_ids, int64_t n, double
  *   dX  (n_nodes x 3 doubles)  dL/dx_v, summed over the active tetrahedra incident to v in
  *       ascending id (deterministic).
  * Element matrices are recomputed from positions and materials (not read from the cache).
- * The first call allocates a per-element scratch of 96 bytes per tetrahedron held by the
- * context.  All pointers are device memory.
+ * The first call allocates a scratch of 112 bytes per tetrahedron and 80 per node pair held by
+ * the context.  All pointers are device memory.
  */
 int sta_adjoint(sta_ctx *ctx, const double *grad_val, double *dE, double *dnu, double *dX,
                 void *stream);

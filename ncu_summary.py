@@ -42,7 +42,7 @@ CSRC = ROOT / "paper_2605_11673_gb300" / "csrc"
 KERNEL_SOURCES = {
     "rebuild": ("sta_rebuild.cu", "sta_fold.cuh", "sta_create.cu", "sta_internal.cuh"),
     "k_elements": ("sta_element.cu", "sta_internal.cuh"),
-    "k_adjoint": ("sta_element.cu", "sta_internal.cuh"),
+    "k_adjoint": ("sta_adjoint.cu", "sta_internal.cuh"),
 }
 # FP64 thread instructions (predicated on), when a capture collected them
 FP64_INST = ("smsp__sass_thread_inst_executed_op_dadd_pred_on.sum",

@@ -182,6 +182,8 @@ struct Ctx {
     int32_t *nt_ptr = nullptr;     // n + 1: node -> incident tetrahedra
     int32_t *nt_list = nullptr;    // 4 T: incident tetrahedra, ascending id
     double *dXe = nullptr;         // T x 12: per-element position gradients (adjoint, lazily)
+    double *gunit = nullptr;       // nunits x 10: parts of each unit's gradient (adjoint, lazily)
+    int32_t *nt_run = nullptr;     // 4 T: offset in dXe of each nt_list entry (adjoint, lazily)
     int32_t *act_list = nullptr;   // T: active tets, unordered (element / adjoint kernels, lazily)
     unsigned long long *act_count = nullptr;
 
@@ -305,7 +307,8 @@ int persistent_grid(const Ctx *c, const void *kernel, int threads, int64_t items
 int build_pattern(Ctx *c, cudaStream_t s);                       // sta_create.cu
 int launch_elements(Ctx *c, bool active_only, cudaStream_t s);   // sta_element.cu
 int launch_expand_elements(Ctx *c, const int32_t *ids, int64_t n, double *out, cudaStream_t s);
-int launch_adjoint(Ctx *c, const double *gval, double *dE, double *dnu, double *dX, cudaStream_t s);
+int launch_active_list(Ctx *c, double *dE, double *dnu, double *dXe, cudaStream_t s);
+int launch_adjoint(Ctx *c, const double *gval, double *dE, double *dnu, double *dX, cudaStream_t s);  // sta_adjoint.cu
 int launch_spmv(Ctx *c, const double *val, const double *x, double *y, cudaStream_t s);
 int launch_rebuild(Ctx *c, cudaStream_t s);                      // sta_rebuild.cu
 int rebuild_form_of(const Ctx *c);  // the form the next rebuild takes (AUTO resolved)
