@@ -183,7 +183,7 @@ int sta::create_impl(const double *nodes, int64_t n_nodes, const int32_t *tets, 
     c->tstate.assign((size_t)n_tets, 0);
     c->seen.assign((size_t)n_tets, 0);
     c->last_counters = c->counters;
-    if (cudaMallocHost((void **)&x->h_count, sizeof(unsigned long long)) != cudaSuccess ||
+    if (cudaMallocHost((void **)&x->h_count, 4 * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMallocHost((void **)&x->h_mask, (size_t)(n_tets > 0 ? n_tets : 1)) != cudaSuccess ||
         cudaHostAlloc((void **)&c->h_count_mapped, sizeof(unsigned long long),
                       cudaHostAllocMapped) != cudaSuccess ||
@@ -246,7 +246,7 @@ extern "C" int sta_proxy_create(int64_t n_nodes, const int32_t *tets, int64_t n_
     c->tstate.assign((size_t)n_tets, 0);
     c->seen.assign((size_t)n_tets, 0);
     c->last_counters = c->counters;
-    if (cudaMallocHost((void **)&x->h_count, sizeof(unsigned long long)) != cudaSuccess ||
+    if (cudaMallocHost((void **)&x->h_count, 4 * sizeof(unsigned long long)) != cudaSuccess ||
         cudaMallocHost((void **)&x->h_mask, (size_t)(n_tets > 0 ? n_tets : 1)) != cudaSuccess)
         return bail(fail(STA_ENOMEM, "pinned mask buffer"));
     *out = x;
@@ -553,12 +553,10 @@ int sta_set_params(sta_ctx *x, const double *nodes, const double *young, const d
     if (x->c.op != STA_OP_ELASTICITY) return fail(STA_ESTATE, "not an elasticity context");
     Ctx *c = &x->c;
     cudaStream_t s = (cudaStream_t)stream;
-    if (nodes) {
-        if (on_device) {
-            STA_CUDA_TRY(cudaMemcpy2DAsync(c->X, sizeof(double4_32a), nodes, 3 * sizeof(double),
-                                           3 * sizeof(double), (size_t)c->n,
-                                           cudaMemcpyDeviceToDevice, s));
-        } else {
+    if (on_device) {
+        STA_TRY(launch_pack_params(c, nodes, young, poisson, s));
+    } else {
+        if (nodes) {
             std::vector<double> X4(4 * (size_t)(c->n > 0 ? c->n : 1), 0.0);
             for (int64_t v = 0; v < c->n; ++v)
                 for (int k = 0; k < 3; ++k) X4[4 * v + k] = nodes[3 * v + k];
@@ -566,21 +564,18 @@ int sta_set_params(sta_ctx *x, const double *nodes, const double *young, const d
                                          cudaMemcpyHostToDevice, s));
             STA_CUDA_TRY(cudaStreamSynchronize(s));
         }
+        if (young)
+            STA_CUDA_TRY(cudaMemcpy2DAsync(c->mat, sizeof(double2), young, sizeof(double),
+                                           sizeof(double), (size_t)c->T, cudaMemcpyHostToDevice, s));
+        if (poisson)
+            STA_CUDA_TRY(cudaMemcpy2DAsync((double *)c->mat + 1, sizeof(double2), poisson,
+                                           sizeof(double), sizeof(double), (size_t)c->T,
+                                           cudaMemcpyHostToDevice, s));
+        STA_TRY(launch_pack_params(c, nullptr, nullptr, nullptr, s));  // the counters
     }
-    cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
-    if (young)
-        STA_CUDA_TRY(cudaMemcpy2DAsync(c->mat, sizeof(double2), young, sizeof(double),
-                                       sizeof(double), (size_t)c->T, kind, s));
-    if (poisson)
-        STA_CUDA_TRY(cudaMemcpy2DAsync((double *)c->mat + 1, sizeof(double2), poisson,
-                                       sizeof(double), sizeof(double), (size_t)c->T, kind, s));
-    unsigned long long init[2] = {0ull, 0ull};
-    STA_CUDA_TRY(cudaMemcpyAsync(c->counters, init, sizeof init, cudaMemcpyHostToDevice, s));
-    unsigned long long mx = ~0ull;
-    STA_CUDA_TRY(cudaMemcpyAsync(c->counters + 2, &mx, sizeof mx, cudaMemcpyHostToDevice, s));
     STA_TRY(launch_elements(c, false, s));
-    unsigned long long back[4];
-    STA_CUDA_TRY(cudaMemcpyAsync(back, c->counters, sizeof back, cudaMemcpyDeviceToHost, s));
+    unsigned long long *back = x->h_count;  // pinned: a pageable target is staged, and slower
+    STA_CUDA_TRY(cudaMemcpyAsync(back, c->counters, 4 * sizeof *back, cudaMemcpyDeviceToHost, s));
     STA_CUDA_TRY(cudaStreamSynchronize(s));
     if (back[0] != 0)
         return fail(STA_EINVAL, std::to_string(back[0]) + " tetrahedra have det <= 0 (first: tet " +

