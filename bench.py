@@ -280,21 +280,16 @@ class SupersetStats:
         the per-entry byte model (1200 B per active tet + 12 B per pattern entry)."""
         L = self.live(mask)
         ta = L["T_act"]
-        tiles = (6 * self.Ud + 9 * self.Up) / 32.0
         if form == "fused":
-            # 78 operands (624 B) per active tet, 10 contributor words per superset tet, unit
-            # records (16 B, + 8 B mirror record off the diagonal) and tile records (16 B) of
-            # every unit and tile, 8 B per value
-            b = 624.0 * ta + 40.0 * self.T + 16.0 * (self.Ud + self.Up) + 8.0 * self.Up \
-                + 16.0 * tiles + 8.0 * self.nnz
+            # 78 operands (624 B) per active tet; record, mirror record and activity (40 B) of
+            # every unit, 8 B per value
+            b = 624.0 * ta + 40.0 * (self.Ud + self.Up) + 8.0 * self.nnz
         else:
-            # fill: 8 B per value; flags: the mask, 10 unit and 10 tile words per active tet,
-            # 2 B per tile; fold of the flagged tiles: their records, unit records and contributor
-            # words, 624 B per active tet, 8 B per value of a unit with an active contributor
-            tl = (6 * L["Ud"] + 9 * L["Up"]) / 32.0
-            b = 8.0 * self.nnz + self.T + 80.0 * ta + 2.0 * tiles + 16.0 * tl \
-                + 16.0 * (L["Ud"] + L["Up"]) + 8.0 * L["Up"] + 4.0 * L["C_live"] + 624.0 * ta \
-                + 8.0 * L["nnz_live"]
+            # fill: 8 B per value, the activity of every unit; fold: records, mirror records and
+            # activity of the units with an active contributor, 624 B per active tet, 8 B per
+            # value of those units
+            b = 8.0 * self.nnz + 16.0 * (self.Ud + self.Up) + 40.0 * (L["Ud"] + L["Up"]) \
+                + 624.0 * ta + 8.0 * L["nnz_live"]
         if fixed:  # integer sum written and exponent read per fold entry (+ the sums' fill)
             b += 10.0 * (6 * self.Ud + 9 * self.Up) + (8.0 * self.nnz if form != "fused" else 0.0)
         return {"algorithmic_bytes": b, "per_entry_model_bytes": 1200.0 * ta + 12.0 * self.nnz,
@@ -1177,7 +1172,7 @@ def roofline_of(runs, r_ms_mean: float, wkey: str, policy: str) -> dict:
     roof = {"bound": "hbm", "achieved": per_entry / t / 1e9, "peak": hbm_peak, "unit": "GB/s",
             "frac": per_entry / t / 1e9 / hbm_peak, "traffic": traffic, "peak_kind": peak_kind,
             "kernel": f"sta_refold ({runs[0].form} form: "
-                      + ("k_fold_flat" if runs[0].form == "fused" else "k_tile_flags + k_fold_flat")
+                      + ("k_fold_flat" if runs[0].form == "fused" else "k_zero_fill + k_fold_flat")
                       + (", fixed point)" if policy == "fixed" else ")"),
             "algorithmic_bytes": per_entry, "byte_model": "1200 B per active tet + 12 B per entry",
             "own_model_bytes": alg, "frac_own_model": alg / t / 1e9 / hbm_peak,

@@ -63,7 +63,8 @@ typedef struct {
 
 typedef struct {
     double eps;             /* eps of Eq. 4 / Eq. 8, added to diagonal entries; default 0 */
-    int32_t block_threads;  /* threads per CTA of the rebuild fold: 64, 128 or 256; 0 = 128 */
+    int32_t block_threads;  /* 64, 128 or 256; 0 = 128.  Kept for callers that set it: the rebuild
+                             * fold's CTAs have one shape */
     int32_t blocks_per_sm;  /* CTAs per SM of the persistent rebuild grid; 0 = occupancy max */
 } sta_options;
 
@@ -117,11 +118,9 @@ int sta_refold(sta_ctx *ctx, void *stream);
  * graph mode is on (STA_ESTATE). */
 int sta_set_launch(sta_ctx *ctx, int32_t block_threads, int32_t blocks_per_sm);
 
-/* Operand loads each lane of the rebuild fold keeps in flight: 4 (default; the fold kernel
- * then fits 64 registers a thread, 32 resident warps per SM) or 6 (80 registers, 24 warps).
- * The fold is bound by load latency and which choice hides it better depends on the mesh and
- * mask; results do not depend on it.  A launch choice of the library with no counterpart in
- * the paper.  Not allowed while graph mode is on (STA_ESTATE); STA_EINVAL for another value. */
+/* 4 (default) or 6.  Kept for callers that set it: how many operand loads a lane of the rebuild
+ * fold kept in flight, before the fold took its operands from shared memory; it has no effect.
+ * Not allowed while graph mode is on (STA_ESTATE); STA_EINVAL for another value. */
 int sta_set_fold_depth(sta_ctx *ctx, int32_t operands_in_flight);
 
 /*
@@ -129,12 +128,11 @@ int sta_set_fold_depth(sta_ctx *ctx, int32_t operands_in_flight);
  * the values; the values are the same bits in every form.
  *  STA_REBUILD_FUSED:     one fold kernel writes every value, +0.0 for the entries without an
  *                         active contributor.  Suits a superset that is mostly active.
- *  STA_REBUILD_ZERO_FILL: a coalesced fill sets every value to +0.0 while the tiles of fold
- *                         units with an active contributor are flagged from the mask; the fold
- *                         then visits only the flagged tiles (and, when eps != 0, the diagonal
- *                         ones).  Suits a superset that is mostly inactive (preallocated
- *                         refinement children, split copies).  Takes 4 more bytes of device
- *                         memory per fold unit and 2 per tile of 32 fold entries (at create).
+ *  STA_REBUILD_ZERO_FILL: a coalesced fill sets every value to +0.0 while the chunks of fold
+ *                         units with an active contributor are flagged; the fold then visits only
+ *                         the flagged chunks (and, when eps != 0, the diagonal ones).  Suits a
+ *                         superset that is mostly inactive (preallocated refinement children,
+ *                         split copies).
  *  STA_REBUILD_AUTO:      (default) ZERO_FILL while fewer than 40% of the tetrahedra are
  *                         active, else FUSED; decided when the rebuild is issued (in graph mode:
  *                         when sta_graph_enable captures it).

@@ -10,7 +10,7 @@ program those captures run.  Measurement tooling beside bench.py, not part of th
     python ncu_summary.py record <report.ncu-rep> <key> <workload> <out.json> \
             --kernels <regex> [--units N] [--command "..."]
         counters summed over the captured launches of the kernels matching <regex> -- one
-        launch sequence, e.g. a rebuild's k_tile_flags + k_fold_flat (DRAM bytes, duration and,
+        launch sequence, e.g. a rebuild's k_zero_fill + k_fold_flat (DRAM bytes, duration and,
         when captured, the FP64 thread instructions; --units: the work items it processed,
         e.g. active tetrahedra, for per-unit figures) -- recorded as <key>_<workload> with the
         hash of the sources the kernels and their data layout are built from
@@ -38,9 +38,9 @@ ROOT = Path(__file__).resolve().parent
 CSRC = ROOT / "paper_2605_11673_gb300" / "csrc"
 # the sources each recorded kernel and the data layout it reads are built from: a record is
 # current only while these hash to the value it was taken with (the rebuild's traffic also
-# depends on the unit order and tiles that create builds)
+# depends on the unit order and chunks that create builds)
 KERNEL_SOURCES = {
-    "rebuild": ("sta_rebuild.cu", "sta_fold.cuh", "sta_create.cu", "sta_internal.cuh"),
+    "rebuild": ("sta_rebuild.cu", "sta_fold.cuh", "sta_bulk.cuh", "sta_create.cu", "sta_internal.cuh"),
     "k_elements": ("sta_element.cu", "sta_internal.cuh"),
     "k_adjoint": ("sta_adjoint.cu", "sta_internal.cuh"),
 }
@@ -154,7 +154,7 @@ def _bytes(value, unit: str) -> float:
 def record(rep: str, key: str, workload: str, out_json: str, kernels: str, units: float = 0.0,
            command: str = "") -> dict:
     """Sum the counters of every captured launch whose kernel name matches `kernels` (the
-    capture holds one launch sequence, e.g. the rebuild's k_tile_flags + k_fold_flat) and write
+    capture holds one launch sequence, e.g. the rebuild's k_zero_fill + k_fold_flat) and write
     the record <key>_<workload>.json, tied to the hash of KERNEL_SOURCES[key]."""
     hdr, unit_row, rows = _raw(rep)
     ki = hdr.index("Kernel Name")

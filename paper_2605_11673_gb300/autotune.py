@@ -1,11 +1,12 @@
 """Launch autotuner for the full rebuild.
 
-Sweeps the rebuild form (fused, or zero fill + fold of the flagged tiles; sta_set_rebuild_form),
-the fold's CTA size (64, 128, 256 threads), CTAs per SM (0 = occupancy maximum, or a fixed
-count) and the operand loads each lane keeps in flight (4 at 32 resident warps per SM, or 6 at
-24; sta_set_fold_depth) on a given context, timing the full refold with CUDA events after an L2
-flush, and keeps the fastest choice in a JSON cache keyed by GPU name, the context's sizes and
-its active fraction (in tenths: the best form depends on how much of the superset is active).
+Sweeps the rebuild form (fused, or zero fill + fold of the flagged chunks; sta_set_rebuild_form)
+and the fold's CTAs per SM (0 = occupancy maximum, or a fixed count) on a given context, timing
+the full refold with CUDA events after an L2 flush, and keeps the fastest choice in a JSON cache
+keyed by GPU name, the context's sizes and its active fraction (in tenths: the best form depends
+on how much of the superset is active).  A choice also names a CTA size and a fold depth, which
+the library accepts but which no longer change the schedule: of the shapes that differ only in
+those, the first is measured.
 The choice changes only the schedule: values are identical for every form and shape.
 """
 from __future__ import annotations
@@ -20,6 +21,8 @@ FUSED, ZERO_FILL = 1, 2  # sta.h STA_REBUILD_FUSED, STA_REBUILD_ZERO_FILL
 # (rebuild form, threads per CTA, CTAs per SM, operand loads in flight)
 SHAPES = [(f, t, b, d) for f in (FUSED, ZERO_FILL) for d in (4, 6) for t in (64, 128, 256)
           for b in (0, 1, 2, 3, 4, 6, 8)]
+# one shape per schedule: the fold runs at most 3 CTAs per SM
+DISTINCT = [(f, 64, b, 4) for f in (FUSED, ZERO_FILL) for b in (0, 1, 2)]
 
 
 def key_for(gpu_name: str, sizes: dict, active_tenths: int = 10) -> str:
@@ -89,7 +92,7 @@ def tune(asm, repeats: int = 11, use_cache: bool = True, path: Path = CACHE,
     if use_cache and key in cache and len(cache[key].get("shape", ())) == len(SHAPES[0]):
         shape = tuple(cache[key]["shape"])
     else:
-        timings = {s: measure(asm, s, repeats) for s in (shapes or SHAPES)}
+        timings = {s: measure(asm, s, repeats) for s in (shapes or DISTINCT)}
         shape = pick_best(timings)
         cache[key] = {"shape": list(shape), "ms": timings[shape],
                       "all": {f"{f}:{t}x{b}:d{d}": ms for (f, t, b, d), ms in timings.items()}}

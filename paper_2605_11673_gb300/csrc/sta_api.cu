@@ -41,6 +41,13 @@ static int64_t set_host_mask(Ctx *c, const uint8_t *__restrict__ mask, uint8_t *
     return na;
 }
 
+// A bounded wait of an earlier rebuild ran out: its values are incomplete.
+static int check_fault(const Ctx *c) {
+    if (c->h_fault && *reinterpret_cast<volatile unsigned int *>(c->h_fault))
+        return fail(STA_ECUDA, "an earlier rebuild did not complete");
+    return STA_OK;
+}
+
 static int wait_staging(sta_ctx *x) {
     if (x->h2d_pending) {
         STA_CUDA_TRY(cudaEventSynchronize(x->h2d_done));
@@ -58,6 +65,7 @@ static void free_ctx(sta_ctx *x) {
     if (x->h_mask) cudaFreeHost(x->h_mask);
     if (x->h_count) cudaFreeHost(x->h_count);
     if (x->c.h_count_mapped) cudaFreeHost(x->c.h_count_mapped);
+    if (x->c.h_fault) cudaFreeHost(x->c.h_fault);
     if (x->h2d_done) cudaEventDestroy(x->h2d_done);
     if (x->c.h_cg) cudaFreeHost(x->c.h_cg);
     graph_release(&x->c);
@@ -162,7 +170,7 @@ int sta::create_impl(const double *nodes, int64_t n_nodes, const int32_t *tets, 
 
     if ((rc = build_pattern(c, s))) return bail(rc);
 
-    if ((rc = dev_alloc(c, &c->Ke, KE_STRIDE * n_tets)) || (rc = dev_alloc(c, &c->mask, n_tets)) ||
+    if ((rc = dev_alloc(c, &c->Ke, c->ke_len)) || (rc = dev_alloc(c, &c->mask, n_tets)) ||
         (rc = dev_alloc(c, &c->val, c->nnz)))
         return bail(rc);
     unsigned long long init[4] = {0ull, 0ull, ~0ull, 0ull};
@@ -187,8 +195,11 @@ int sta::create_impl(const double *nodes, int64_t n_nodes, const int32_t *tets, 
         cudaMallocHost((void **)&x->h_mask, (size_t)(n_tets > 0 ? n_tets : 1)) != cudaSuccess ||
         cudaHostAlloc((void **)&c->h_count_mapped, sizeof(unsigned long long),
                       cudaHostAllocMapped) != cudaSuccess ||
-        cudaHostGetDevicePointer((void **)&c->d_count_mapped, c->h_count_mapped, 0) != cudaSuccess)
+        cudaHostGetDevicePointer((void **)&c->d_count_mapped, c->h_count_mapped, 0) != cudaSuccess ||
+        cudaHostAlloc((void **)&c->h_fault, sizeof(unsigned int), cudaHostAllocMapped) != cudaSuccess ||
+        cudaHostGetDevicePointer((void **)&c->d_fault, c->h_fault, 0) != cudaSuccess)
         return bail(fail(STA_ENOMEM, "pinned host buffers"));
+    *c->h_fault = 0u;
     *out = x;
     return STA_OK;
 }
@@ -267,6 +278,7 @@ int sta_full_rebuild(sta_ctx *x, const uint8_t *mask, int mask_on_device, void *
     Ctx *c = &x->c;
     if (c->T > 0 && !mask) return fail(STA_EINVAL, "mask is NULL");
     cudaStream_t s = (cudaStream_t)stream;
+    STA_TRY(check_fault(c));
     if (c->T > 0) {
         STA_TRY(wait_staging(x));
         if (mask_on_device) {  // read back for the host mirror; the device copy is the 0/1 one
@@ -326,6 +338,7 @@ int sta_get_rebuild_form(const sta_ctx *x, int32_t *form) {
 
 int sta_refold(sta_ctx *x, void *stream) {
     if (!x) return fail(STA_EINVAL, "ctx is NULL");
+    STA_TRY(check_fault(&x->c));
     if (x->c.graph_on) {
         STA_CUDA_TRY(cudaGraphLaunch(x->c.g_refold, (cudaStream_t)stream));
         return STA_OK;

@@ -1,4 +1,5 @@
-// Append counting shared by the claim kernels of the fixed-point and proxy frames: each warp's
+// What the claim kernels of the streaming frames share: the claim of a fold unit, and append
+// counting of the fixed-point and proxy frames: each warp's
 // winners are counted in one CTA-wide step, so a frame issues one atomic per CTA on each
 // counter word instead of one per warp (a large frame's warps all appending to one word
 // serialise at the L2).
@@ -8,6 +9,24 @@
 
 namespace sta {
 namespace {
+
+// Contributor j of unit u becomes active (`on`) or inactive: moves its bit (which holds the other
+// state: edits are validated) and counts a claim of the unit, for j < 32 in one atomic; true for
+// the thread that claims the unit first in its frame.
+__device__ __forceinline__ bool claim_unit(UnitState *__restrict__ ustate, uint32_t *__restrict__ uext,
+                                           int32_t u, int32_t j, bool on) {
+    unsigned long long step = 1ull << 32;  // one claim
+    if (j < 32) {
+        const unsigned long long bit = 1ull << j;
+        step = on ? step + bit : step - bit;
+    } else {
+        uint32_t *w = j < 64 ? &ustate[u].w1 : uext + ustate[u].xoff + (j / 32 - 2);
+        const uint32_t bit = 1u << (j & 31);
+        if (on) atomicOr(w, bit);
+        else atomicAnd(w, ~bit);
+    }
+    return (atomicAdd(reinterpret_cast<unsigned long long *>(ustate + u), step) >> 32) == 0ull;
+}
 
 // Called by every thread of a CTA of THREADS threads, the same number of times.  Lane 0 of
 // each warp brings its warp's counts c1 (for counters[1]) and c3 (for counters[3]); returns,

@@ -9,7 +9,7 @@
 //   tet -> block of each local node pair              tblk   (T x 16)
 //   tet -> CSR index of each local entry              scat   (T x 144)
 //   fold units (node pairs a <= b) with their contributors in ascending tet id, and each
-//   tetrahedron's 10 unit slots                      bmeta / bmirror / ccode / cslot / tunit
+//   tetrahedron's 10 unit slots                      bmeta / bmirror / ctet / tpos / tunit
 // Lists filled with atomics are sorted afterwards, so every array is deterministic.
 #include <algorithm>
 #include <climits>
@@ -350,37 +350,37 @@ __global__ void k_unit_fill(const int4 *tets, const int32_t *tunit, int64_t T, c
     }
 }
 
-// cslot[10 t + s] = position of tetrahedron t's slot-s contribution in its unit's list
-__global__ void k_unit_slots(const int32_t *ccode, int64_t T, int32_t *cslot) {
+// From the sorted contributor codes: the contributors' tetrahedra, and for each tetrahedron's slots
+// its place among the unit's contributors and the offset of its run.
+__global__ void k_unit_slots(const int32_t *__restrict__ ccode, int64_t T,
+                             const int32_t *__restrict__ tunit, const int64_t *__restrict__ uptr,
+                             const int32_t *__restrict__ koff, int32_t *__restrict__ ctet,
+                             int32_t *__restrict__ tpos, int32_t *__restrict__ krun) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < 10 * T;
          k += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t code = ccode[k];
-        cslot[10 * (int64_t)code_tet(code) + slot_of((code >> 2) & 3, code & 3)] = (int32_t)k;
+        const int32_t code = ccode[k], t = code_tet(code);
+        const int s = slot_of((code >> 2) & 3, code & 3);
+        const int64_t i = 10 * (int64_t)t + s;
+        const int32_t u = tunit[i], j = (int32_t)(k - uptr[u]);
+        ctet[k] = t;
+        tpos[i] = j;
+        krun[i] = koff[u] + (s < 4 ? RUN_DIAG : RUN_PAIR) * j;
     }
 }
 
-// contributor codes (t, la, lb) -> contributor words: offset of the element-cache run the
-// contributor supplies to its unit (word_offset), active bit clear
-__global__ void k_code_words(int32_t *ccode, int64_t n, int64_t T) {
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t code = ccode[k];
-        const int la = (code >> 2) & 3, lb = code & 3;
-        ccode[k] = (int32_t)ke_slot_at(T, code_tet(code), slot_of(la, lb));
-    }
-}
-
-// unit records: value offset and row stride of (a, b) and of its mirror (b, a), contributors
+// unit records: value offset and row stride of (a, b) and of its mirror (b, a), the offset of the
+// runs, the number of contributors
 __global__ void k_unit_meta(int64_t nblocks, const int32_t *block_node, const int32_t *adj,
                             const int32_t *adj_ptr, const int2 *boff, const int64_t *uid,
-                            const int32_t *upper, const int64_t *uptr, int4 *umeta, int2 *umirror) {
+                            const int32_t *upper, const int64_t *uptr, const int32_t *koff,
+                            int4 *umeta, int2 *umirror) {
     for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < nblocks;
          g += (int64_t)gridDim.x * blockDim.x) {
         if (!upper[g]) continue;
         const int32_t a = block_node[g], b = adj[g];
         const int64_t u = uid[g];
         const int2 o = boff[g], m = boff[find_block(adj_ptr, adj, b, a)];
-        umeta[u] = make_int4(o.x, o.y << 1 | (a == b ? 1 : 0), (int32_t)uptr[u], (int32_t)uptr[u + 1]);
+        umeta[u] = make_int4(o.x, o.y << 1 | (a == b ? 1 : 0), koff[u], (int32_t)(uptr[u + 1] - uptr[u]));
         umirror[u] = m;
     }
 }
@@ -413,28 +413,27 @@ struct Scratch {
     }
 };
 
-// Unit order and fold tiles.  The units (node order) are cut into windows of UNIT_WINDOW;
+// Unit order and fold chunks.  The units (node order) are cut into windows of UNIT_WINDOW;
 // inside a window the diagonal units come first, then the off-diagonal ones, each group with
 // the longest contributor lists first.  The rebuild (k_fold_flat) gives every fold entry a
-// lane -- 6 entries per diagonal unit, 9 per off-diagonal unit -- and takes 32 consecutive
-// entries of one group per warp tile, so tiles never mix the two kinds, neighbouring units
-// have lists of equal length (the tile waits for its longest), and a window's values are
-// written close together in time.  Any order gives the same values: each unit folds its own
-// list in its own order.
-// Tile record: {first unit, entry offset in it | diagonal << 4 | entries in the tile << 5,
-// first code of the tile's units, end of their codes}.
+// lane -- 6 entries per diagonal unit, 9 per off-diagonal unit -- and takes chunks of consecutive
+// units of one group, so the entries of a warp's round are of one kind and fold lists of equal
+// length (the round waits for its longest), and a window's values are written close together in
+// time.  Any order gives the same values: each unit folds its own list in its own order.
+// Chunk record: {first unit, units | diagonal << 8}.
 #ifndef STA_UNIT_WINDOW
 #define STA_UNIT_WINDOW 2048
 #endif
 
 void unit_order(const std::vector<int32_t> &cnt, const std::vector<int32_t> &umin,
-                const std::vector<uint8_t> &diag, std::vector<int32_t> &rn, std::vector<int4> &tiles) {
+                const std::vector<uint8_t> &diag, std::vector<int32_t> &rn, std::vector<int32_t> &order,
+                std::vector<int2> &chunks) {
     const int64_t m = (int64_t)cnt.size();
     const int64_t W = STA_UNIT_WINDOW > 1 ? STA_UNIT_WINDOW : 1;
-    std::vector<int32_t> order;
+    order.clear();
     order.reserve(m);
     rn.assign(m, 0);
-    tiles.clear();
+    chunks.clear();
     for (int64_t w0 = 0; w0 < m; w0 += W) {
         const int64_t w1 = std::min(m, w0 + W);
         for (int cls = 1; cls >= 0; --cls) {
@@ -444,26 +443,21 @@ void unit_order(const std::vector<int32_t> &cnt, const std::vector<int32_t> &umi
             std::stable_sort(order.begin() + first, order.end(), [&](int32_t a, int32_t b) {
                 return cnt[a] != cnt[b] ? cnt[a] > cnt[b] : umin[a] < umin[b];
             });
-            const int64_t per = cls ? FOLD_TASKS_DIAG : FOLD_TASKS_PAIR;
-            const int64_t nent = per * (int64_t)(order.size() - first);
-            for (int64_t e = 0; e < nent; e += 32) {
-                const int64_t k = std::min<int64_t>(32, nent - e);
-                // code range filled in below, once every unit's list position is known
-                tiles.push_back(make_int4((int32_t)(first + e / per),
-                                          (int32_t)(e % per) | cls << 4 | (int32_t)k << 5,
-                                          (int32_t)(first + (e + k - 1) / per), 0));
+            const int32_t most = cls ? CHUNK_DIAG : CHUNK_PAIR;
+            for (size_t k = first; k < order.size();) {  // as many units as fit; a long one alone
+                const size_t k0 = k;
+                int64_t bytes = 0;
+                int32_t n = 0;
+                for (; k < order.size() && n < most; ++k, ++n) {
+                    const int64_t c = cnt[order[k]], b = 8 * (((cls ? RUN_DIAG : RUN_PAIR) * c + 1) & ~1LL);
+                    if (n > 0 && (c > 64 || cnt[order[k - 1]] > 64 || bytes + b > CHUNK_BYTES)) break;
+                    bytes += b;
+                }
+                chunks.push_back(make_int2((int32_t)k0, n | cls << 8));
             }
         }
     }
     for (int64_t k = 0; k < m; ++k) rn[order[k]] = (int32_t)k;
-    // lists are stored in new-id order: unit k's codes start at the sum of the earlier counts
-    std::vector<int64_t> cs(m + 1, 0);
-    for (int64_t k = 0; k < m; ++k) cs[k + 1] = cs[k] + cnt[order[k]];
-    for (auto &t : tiles) {
-        const int64_t last = t.z;
-        t.z = (int32_t)cs[t.x];
-        t.w = (int32_t)cs[last + 1];
-    }
 }
 
 }  // namespace
@@ -563,15 +557,21 @@ int build_pattern(Ctx *c, cudaStream_t s) {
     c->nunits = nunits;
     STA_TRY(dev_alloc(c, &c->bmeta, nunits));
     STA_TRY(dev_alloc(c, &c->bmirror, nunits));
-    STA_TRY(dev_alloc(c, &c->ccode, 10 * T));
-    STA_TRY(dev_alloc(c, &c->cslot, 10 * T));
+    STA_TRY(dev_alloc(c, &c->ustate, nunits));
+    STA_TRY(dev_alloc(c, &c->uc0, nunits + 1));
+    STA_TRY(dev_alloc(c, &c->ctet, 10 * T));
+    STA_TRY(dev_alloc(c, &c->tpos, 10 * T));
+    STA_TRY(dev_alloc(c, &c->krun, 10 * T));
     STA_TRY(dev_alloc(c, &c->tunit, 10 * T));
-    STA_TRY(dev_alloc(c, &c->owner, nunits));
     STA_TRY(dev_alloc(c, &c->touched, nunits));
     k_unit_of_block<<<grid_for(nblocks), TPB, 0, s>>>(nblocks, c->block_node, c->adj, c->adj_ptr,
                                                       uid, ublk);
     int64_t *uptr = nullptr;
+    int32_t *koff = nullptr, *ccode = nullptr;
     STA_TRY(sc.get(&uptr, nunits + 1));
+    STA_TRY(sc.get(&koff, nunits));
+    STA_TRY(sc.get(&ccode, 10 * T));
+    int64_t next_words = 0;
     STA_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (nunits > 0 ? nunits : 1), s));
     k_unit_count<<<grid_for(10 * T), TPB, 0, s>>>(c->tblk, ublk, T, c->tunit, cnt);
     if (nunits > 0) {  // renumber (windows: diagonal units first, longest lists first)
@@ -581,9 +581,9 @@ int build_pattern(Ctx *c, cudaStream_t s) {
         STA_TRY(sc.get(&rn_dev, nunits));
         k_unit_diag<<<grid_for(nblocks), TPB, 0, s>>>(nblocks, c->block_node, c->adj, upper, uid,
                                                       udiag);
-        std::vector<int32_t> hcnt(nunits), hmin(nunits), rn;
+        std::vector<int32_t> hcnt(nunits), hmin(nunits), rn, order;
         std::vector<uint8_t> hdiag(nunits);
-        std::vector<int4> htiles;
+        std::vector<int2> hchunks;
         k_fill_i32<<<grid_for(nunits), TPB, 0, s>>>(rn_dev, nunits, INT32_MAX);
         k_unit_min_tet<<<grid_for(10 * T), TPB, 0, s>>>(c->tunit, T, rn_dev);
         STA_CUDA_TRY(cudaMemcpyAsync(hmin.data(), rn_dev, sizeof(int32_t) * nunits,
@@ -592,34 +592,29 @@ int build_pattern(Ctx *c, cudaStream_t s) {
                                      cudaMemcpyDeviceToHost, s));
         STA_CUDA_TRY(cudaMemcpyAsync(hdiag.data(), udiag, nunits, cudaMemcpyDeviceToHost, s));
         STA_CUDA_TRY(cudaStreamSynchronize(s));
-        unit_order(hcnt, hmin, hdiag, rn, htiles);
-        c->ntiles = (int64_t)htiles.size();
-        STA_TRY(dev_alloc(c, &c->ftile, c->ntiles));
-        // per unit (new ids) its first tile | (it also reaches the next tile) << 31, and per
-        // tile whether it is of diagonal units: the zero-fill rebuild's tile flags
-        {
-            std::vector<int32_t> hut(nunits, -1);
-            std::vector<uint8_t> htd(c->ntiles);
-            for (int64_t ti = 0; ti < c->ntiles; ++ti) {
-                const int4 t = htiles[ti];
-                const int per = (t.y >> 4) & 1 ? FOLD_TASKS_DIAG : FOLD_TASKS_PAIR;
-                const int64_t ulast = t.x + ((t.y & 15) + (t.y >> 5) - 1) / per;
-                htd[ti] = (uint8_t)((t.y >> 4) & 1);
-                for (int64_t u = t.x; u <= ulast; ++u)
-                    hut[u] = hut[u] < 0 ? (int32_t)ti : (int32_t)(hut[u] | INT32_MIN);
-            }
-            STA_TRY(dev_alloc(c, &c->utile, nunits));
-            STA_TRY(dev_alloc(c, &c->tdiag, c->ntiles));
-            STA_TRY(dev_alloc(c, &c->tflag, c->ntiles));
-            STA_CUDA_TRY(cudaMemcpyAsync(c->utile, hut.data(), sizeof(int32_t) * nunits,
-                                         cudaMemcpyHostToDevice, s));
-            STA_CUDA_TRY(cudaMemcpyAsync(c->tdiag, htd.data(), (size_t)c->ntiles,
-                                         cudaMemcpyHostToDevice, s));
-            // zero between rebuilds (the zero-fill fold clears each flag it reads)
-            STA_CUDA_TRY(cudaMemsetAsync(c->tflag, 0, (size_t)c->ntiles, s));
-            STA_CUDA_TRY(cudaStreamSynchronize(s));  // host vectors go out of scope
+        unit_order(hcnt, hmin, hdiag, rn, order, hchunks);
+        // where each unit's runs start in the element cache (an even offset), and its activity
+        // words past the first two
+        std::vector<int32_t> hko(nunits);
+        std::vector<UnitState> hus(nunits);
+        int64_t ke = 0;
+        for (int64_t k = 0; k < nunits; ++k) {
+            const int64_t cnt_k = hcnt[order[k]];
+            hko[k] = (int32_t)ke;
+            ke += (hdiag[order[k]] ? RUN_DIAG : RUN_PAIR) * cnt_k;
+            ke += ke & 1;
+            hus[k] = UnitState{0u, 0u, 0u, cnt_k > 64 ? (uint32_t)next_words : UNIT_NARROW};
+            if (cnt_k > 64) next_words += (cnt_k + 31) / 32 - 2;
         }
-        STA_CUDA_TRY(cudaMemcpyAsync(c->ftile, htiles.data(), sizeof(int4) * c->ntiles,
+        c->ke_len = ke;
+        STA_CUDA_TRY(cudaMemcpyAsync(koff, hko.data(), sizeof(int32_t) * nunits,
+                                     cudaMemcpyHostToDevice, s));
+        STA_CUDA_TRY(cudaMemcpyAsync(c->ustate, hus.data(), sizeof(UnitState) * nunits,
+                                     cudaMemcpyHostToDevice, s));
+        c->nchunks = (int64_t)hchunks.size();
+        STA_TRY(dev_alloc(c, &c->chunks, c->nchunks));
+        STA_TRY(dev_alloc(c, &c->cflag, c->nchunks));
+        STA_CUDA_TRY(cudaMemcpyAsync(c->chunks, hchunks.data(), sizeof(int2) * c->nchunks,
                                      cudaMemcpyHostToDevice, s));
         STA_CUDA_TRY(cudaMemcpyAsync(rn_dev, rn.data(), sizeof(int32_t) * nunits,
                                      cudaMemcpyHostToDevice, s));
@@ -630,13 +625,16 @@ int build_pattern(Ctx *c, cudaStream_t s) {
     }
     STA_TRY(exclusive_scan(c, cnt, nunits, uptr, tiles, s));
     STA_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (nunits > 0 ? nunits : 1), s));
-    k_unit_fill<<<grid_for(10 * T), TPB, 0, s>>>(c->tets, c->tunit, T, uptr, cnt, c->ccode);
-    k_sort_segments<<<grid_for(nunits), TPB, 0, s>>>(uptr, nunits, c->ccode);
-    k_unit_slots<<<grid_for(10 * T), TPB, 0, s>>>(c->ccode, T, c->cslot);
-    k_code_words<<<grid_for(10 * T), TPB, 0, s>>>(c->ccode, 10 * T, T);
+    k_unit_fill<<<grid_for(10 * T), TPB, 0, s>>>(c->tets, c->tunit, T, uptr, cnt, ccode);
+    k_sort_segments<<<grid_for(nunits), TPB, 0, s>>>(uptr, nunits, ccode);
+    k_unit_slots<<<grid_for(10 * T), TPB, 0, s>>>(ccode, T, c->tunit, uptr, koff, c->ctet, c->tpos,
+                                                  c->krun);
+    k_to_i32<<<grid_for(nunits + 1), TPB, 0, s>>>(uptr, nunits + 1, c->uc0);
     k_unit_meta<<<grid_for(nblocks), TPB, 0, s>>>(nblocks, c->block_node, c->adj, c->adj_ptr,
-                                                  c->boff, uid, upper, uptr, c->bmeta, c->bmirror);
-    k_fill_i32<<<grid_for(nunits), TPB, 0, s>>>(c->owner, nunits, INT32_MAX);
+                                                  c->boff, uid, upper, uptr, koff, c->bmeta,
+                                                  c->bmirror);
+    STA_TRY(dev_alloc(c, &c->uext, next_words));
+    STA_CUDA_TRY(cudaMemsetAsync(c->uext, 0, sizeof(uint32_t) * (size_t)(next_words > 0 ? next_words : 1), s));
     STA_CUDA_TRY(cudaGetLastError());
     STA_CUDA_TRY(cudaStreamSynchronize(s));
     return STA_OK;

@@ -1,6 +1,6 @@
 // Element stiffness kernel: the 12x12 linear-tetrahedron elasticity matrix K^(tau)
 // (STA-FEM Sec. 3.4 and Sec. 5.2; the standard P1 isotropic small-strain element,
-// K = V B^T D B), 78 unique entries per tetrahedron written to the element cache.
+// K = V B^T D B), 78 unique entries per tetrahedron written to the element cache as 10 runs.
 //
 // The evaluation order is fixed (see include/sta.h, sta_recompute_elements) and this file
 // is compiled with --fmad=false: every fma below is an explicit __fma_rn, every other
@@ -30,74 +30,63 @@ __device__ __forceinline__ V3 cross_fma(const V3 &u, const V3 &v) {
 
 __device__ __forceinline__ double gc(const V3 &g, int i) { return i == 0 ? g.x : (i == 1 ? g.y : g.z); }
 
-// Computes the 78-entry record of one tetrahedron (node ids q) into rec[] (registers or shared
-// memory).  Returns false when det <= 0 (record filled with zeros).
-__device__ __forceinline__ bool element_record(double4_32a x0, double4_32a x1, double4_32a x2, double4_32a x3,
-                                               double E, double nu, int4 q, double *rec) {
-    const int gid[4] = {q.x, q.y, q.z, q.w};
+// What the entries of one element matrix are formed from: barycentric gradients g, P = V lam g,
+// Q = V mu g, V mu.
+struct Element {
+    V3 g[4], P[4], Q[4];
+    double Vm;
+};
+
+// Returns false when det <= 0 (everything zero: a zero matrix).
+__device__ __forceinline__ bool element(double4_32a x0, double4_32a x1, double4_32a x2,
+                                        double4_32a x3, double E, double nu, Element &e) {
     V3 d1 = sub(x1, x0), d2 = sub(x2, x0), d3 = sub(x3, x0);
     V3 c1 = cross_fma(d2, d3), c2 = cross_fma(d3, d1), c3 = cross_fma(d1, d2);
     double det = __fma_rn(d1.z, c1.z, __fma_rn(d1.y, c1.y, d1.x * c1.x));
     if (!(det > 0.0)) {
 #pragma unroll
-        for (int k = 0; k < KE_STRIDE; ++k) rec[k] = 0.0;
+        for (int a = 0; a < 4; ++a) e.g[a] = e.P[a] = e.Q[a] = {0.0, 0.0, 0.0};
+        e.Vm = 0.0;
         return false;
     }
     double r = 1.0 / det;
-    V3 g[4];
-    g[1] = {c1.x * r, c1.y * r, c1.z * r};
-    g[2] = {c2.x * r, c2.y * r, c2.z * r};
-    g[3] = {c3.x * r, c3.y * r, c3.z * r};
-    g[0] = {-((g[1].x + g[2].x) + g[3].x), -((g[1].y + g[2].y) + g[3].y),
-            -((g[1].z + g[2].z) + g[3].z)};
+    e.g[1] = {c1.x * r, c1.y * r, c1.z * r};
+    e.g[2] = {c2.x * r, c2.y * r, c2.z * r};
+    e.g[3] = {c3.x * r, c3.y * r, c3.z * r};
+    e.g[0] = {-((e.g[1].x + e.g[2].x) + e.g[3].x), -((e.g[1].y + e.g[2].y) + e.g[3].y),
+              -((e.g[1].z + e.g[2].z) + e.g[3].z)};
     double V = det / 6.0;
     double onu = 1.0 + nu;
     double lam = (E * nu) / (onu * (1.0 - (nu + nu)));
     double mu = E / (onu + onu);
-    double Vl = V * lam, Vm = V * mu;
-    double P[4][3], Q[4][3];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-            P[a][i] = Vl * gc(g[a], i);
-            Q[a][i] = Vm * gc(g[a], i);
-        }
-    // diagonal blocks (a, a), entries i <= j
+    double Vl = V * lam;
+    e.Vm = V * mu;
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
-        double D = Vm * __fma_rn(g[a].z, g[a].z, __fma_rn(g[a].y, g[a].y, g[a].x * g[a].x));
-        double *o = rec + ke_diag_off(a);
-#pragma unroll
-        for (int i = 0; i < 3; ++i)
-#pragma unroll
-            for (int j = i; j < 3; ++j) {
-                double v = (i != j)
-                               ? __fma_rn(P[a][i], gc(g[a], j), Q[a][j] * gc(g[a], i))
-                               : __fma_rn(P[a][i], gc(g[a], i), __fma_rn(Q[a][i], gc(g[a], i), D));
-                o[ke_tri(i, j)] = v;
-            }
+        e.P[a] = {Vl * e.g[a].x, Vl * e.g[a].y, Vl * e.g[a].z};
+        e.Q[a] = {e.Vm * e.g[a].x, e.Vm * e.g[a].y, e.Vm * e.g[a].z};
     }
-    // off-diagonal blocks (a, b), a < b, all (i, j)
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = a + 1; b < 4; ++b) {
-            double D = Vm * __fma_rn(g[a].z, g[b].z, __fma_rn(g[a].y, g[b].y, g[a].x * g[b].x));
-            double *o = rec + ke_off_off(a, b);
-            const bool tr = gid[a] > gid[b];  // run stored with the lower node id's rows
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    double v = (i != j)
-                                   ? __fma_rn(P[a][i], gc(g[b], j), Q[a][j] * gc(g[b], i))
-                                   : __fma_rn(P[a][i], gc(g[b], i), __fma_rn(Q[a][i], gc(g[b], i), D));
-                    o[tr ? 3 * j + i : 3 * i + j] = v;
-                }
-            o[9] = 0.0;  // pad to a 16-byte aligned run
-        }
     return true;
+}
+
+// Entries of the block (a, b): a == b the 6 entries i <= j, else all 9, row-major, transposed when
+// `tr` (a run is stored with the lower node id's rows).
+template <int a, int b>
+__device__ __forceinline__ void element_run(const Element &e, bool tr, double *o) {
+    const V3 &ga = e.g[a], &gb = e.g[b];
+    const double D = e.Vm * __fma_rn(ga.z, gb.z, __fma_rn(ga.y, gb.y, ga.x * gb.x));
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = a == b ? i : 0; j < 3; ++j) {
+            const double v =
+                i != j ? __fma_rn(gc(e.P[a], i), gc(gb, j), gc(e.Q[a], j) * gc(gb, i))
+                       : __fma_rn(gc(e.P[a], i), gc(gb, i), __fma_rn(gc(e.Q[a], i), gc(gb, i), D));
+            if (a == b)
+                o[ke_tri(i, j)] = v;
+            else
+                o[tr ? 3 * j + i : 3 * i + j] = v;
+        }
 }
 
 // New positions and materials (device arrays, null: kept) into the context's padded layout, and
@@ -193,53 +182,80 @@ k_active_list(const uint8_t *__restrict__ mask, int64_t T, int32_t *__restrict__
     }
 }
 
-// Element records of tets list[0 .. *count) (or of all tets 0 .. T-1 when list is null), one
-// per thread, staged per warp in shared memory and written out as contiguous records.
-__global__ void __launch_bounds__(EL_TPB)
+// The warp's 32 runs of one slot from its buffer to the element cache: consecutive lanes write
+// consecutive doubles of a run.
+template <int N>
+__device__ __forceinline__ void write_runs(const double *buf, int32_t off, double *__restrict__ Ke,
+                                           int lane) {
+    __syncwarp();
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int e = 32 * k + lane, r = e / N;
+        const int32_t o = __shfl_sync(0xffffffffu, off, r);
+        if (o >= 0) Ke[o + (e - N * r)] = buf[e];
+    }
+    __syncwarp();
+}
+
+// Element matrices of tets list[0 .. *count) (or of all tets 0 .. T-1 when list is null), one per
+// thread, written to the cache run by run.  Bound by the FP64 pipe: 307 instructions a tetrahedron.
+// One run at a time is staged (2.3 KB a warp), so registers alone limit the CTAs of an SM and the
+// quadrant's other warps compute while one writes; staging whole records (84 KB a CTA of 4 warps,
+// 2 warps a quadrant) left the pipe idle a quarter of the time: 384,000 tetrahedra 257 -> 225 us
+// (FP64 floor 190 us; with 3 CTAs an SM instead of 4, without the 64 spilled bytes: 236 us).
+__global__ void __launch_bounds__(EL_TPB, 4)
 k_elements(const double4_32a *__restrict__ X, const int4 *__restrict__ tets,
            const double2 *__restrict__ mat, const int32_t *__restrict__ list,
-           const unsigned long long *__restrict__ count, int64_t T, double *__restrict__ Ke,
-           unsigned long long *bad) {
-    extern __shared__ double smem[];
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double *wrec = smem + (size_t)wid * 32 * KE_STRIDE;
+           const unsigned long long *__restrict__ count, int64_t T,
+           const int32_t *__restrict__ krun, double *__restrict__ Ke, unsigned long long *bad) {
+    __shared__ double bufs[EL_TPB / 32][32 * RUN_PAIR];
+    const int lane = threadIdx.x & 31;
+    double *buf = bufs[threadIdx.x >> 5];
     const int64_t n = list ? (int64_t)*count : T;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n;
          base += (int64_t)gridDim.x * blockDim.x) {  // block-uniform
         const int64_t i = base + threadIdx.x;
         const bool doit = i < n;
-        const int32_t t = doit ? (list ? list[i] : (int32_t)i) : 0;
+        int32_t off[10];  // of the tet's runs; -1: none
+        Element e;
+        bool t01 = false, t02 = false, t03 = false, t12 = false, t13 = false, t23 = false;
         if (doit) {
+            const int32_t t = list ? list[i] : (int32_t)i;
             const int4 q = tets[t];
             const double2 m = mat[t];
-            const bool ok = element_record(X[q.x], X[q.y], X[q.z], X[q.w], m.x, m.y, q,
-                                           wrec + (size_t)lane * KE_STRIDE);
-            if (!ok) {
+            const int2 *kr = reinterpret_cast<const int2 *>(krun + 10 * (int64_t)t);
+#pragma unroll
+            for (int h = 0; h < 5; ++h) {
+                const int2 v = __ldg(kr + h);
+                off[2 * h] = v.x;
+                off[2 * h + 1] = v.y;
+            }
+            if (!element(X[q.x], X[q.y], X[q.z], X[q.w], m.x, m.y, e)) {
                 atomicAdd(&bad[0], 1ull);
                 atomicMin(&bad[2], (unsigned long long)t);
             }
+            t01 = q.x > q.y; t02 = q.x > q.z; t03 = q.x > q.w;
+            t12 = q.y > q.z; t13 = q.y > q.w; t23 = q.z > q.w;
+        } else {
+#pragma unroll
+            for (int h = 0; h < 10; ++h) off[h] = -1;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) e.g[a] = e.P[a] = e.Q[a] = {0.0, 0.0, 0.0};
+            e.Vm = 0.0;
         }
-        unsigned todo = __ballot_sync(FULL, doit);
-        __syncwarp();
-        while (todo) {  // coalesced copy-out, one record at a time, to its diagonal and pair rows
-            const int r = __ffs(todo) - 1;
-            todo &= todo - 1;
-            const int32_t tr = __shfl_sync(FULL, t, r);
-            const double2 *src = reinterpret_cast<const double2 *>(wrec + (size_t)r * KE_STRIDE);
-            double2 *dd = reinterpret_cast<double2 *>(Ke + ke_diag_at(T, tr, 0));
-            double2 *dp = reinterpret_cast<double2 *>(Ke + ke_pair_at(T, tr, 0));
-            for (int k = lane; k < KE_STRIDE / 2; k += 32) {
-                if (k < KE_DIAG / 2)
-                    dd[k] = src[k];
-                else
-                    dp[k - KE_DIAG / 2] = src[k];
-            }
-        }
-        __syncwarp();
+        double *d = buf + RUN_DIAG * lane, *p = buf + RUN_PAIR * lane;
+        element_run<0, 0>(e, false, d); write_runs<RUN_DIAG>(buf, off[0], Ke, lane);
+        element_run<1, 1>(e, false, d); write_runs<RUN_DIAG>(buf, off[1], Ke, lane);
+        element_run<2, 2>(e, false, d); write_runs<RUN_DIAG>(buf, off[2], Ke, lane);
+        element_run<3, 3>(e, false, d); write_runs<RUN_DIAG>(buf, off[3], Ke, lane);
+        element_run<0, 1>(e, t01, p); write_runs<RUN_PAIR>(buf, off[4], Ke, lane);
+        element_run<0, 2>(e, t02, p); write_runs<RUN_PAIR>(buf, off[5], Ke, lane);
+        element_run<0, 3>(e, t03, p); write_runs<RUN_PAIR>(buf, off[6], Ke, lane);
+        element_run<1, 2>(e, t12, p); write_runs<RUN_PAIR>(buf, off[7], Ke, lane);
+        element_run<1, 3>(e, t13, p); write_runs<RUN_PAIR>(buf, off[8], Ke, lane);
+        element_run<2, 3>(e, t23, p); write_runs<RUN_PAIR>(buf, off[9], Ke, lane);
     }
 }
-
 
 // y = A x over the context's CSR (one thread per row, ascending columns).
 __global__ void k_spmv(const int32_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
@@ -254,8 +270,9 @@ __global__ void k_spmv(const int32_t *__restrict__ row_ptr, const int32_t *__res
 }
 
 // Expand cached records of selected tetrahedra to full 12x12 row-major matrices.
-__global__ void k_expand(const double *__restrict__ Ke, const int4 *__restrict__ tets, int64_t T,
-                         const int32_t *ids, int64_t n, double *out) {
+__global__ void k_expand(const double *__restrict__ Ke, const int32_t *__restrict__ krun,
+                         const int4 *__restrict__ tets, int64_t T, const int32_t *ids, int64_t n,
+                         double *out) {
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < 144 * n;
          k += (int64_t)gridDim.x * blockDim.x) {
         int64_t e = k / 144;
@@ -272,10 +289,8 @@ __global__ void k_expand(const double *__restrict__ Ke, const int4 *__restrict__
         }
         const int4 tq = tets[t];
         const int gid[4] = {tq.x, tq.y, tq.z, tq.w};
-        const double *dg = Ke + ke_diag_at(T, t, a), *pr = Ke + ke_pair_at(T, t, ke_pair(a, b));
-        out[k] = (a == b)             ? dg[ke_tri(i, j)]
-                 : gid[a] < gid[b] ? pr[3 * i + j]
-                                   : pr[3 * j + i];
+        const double *run = Ke + krun[10 * (int64_t)t + slot_of(a, b)];
+        out[k] = run[a == b ? ke_tri(i, j) : (gid[a] < gid[b] ? 3 * i + j : 3 * j + i)];
     }
 }
 
@@ -311,20 +326,17 @@ int launch_active_list(Ctx *c, double *dE, double *dnu, double *dXe, cudaStream_
 
 int launch_elements(Ctx *c, bool active_only, cudaStream_t s) {
     if (c->T == 0) return STA_OK;
-    size_t smem = (size_t)EL_TPB * KE_STRIDE * sizeof(double);  // 84 KB
-    STA_CUDA_TRY(cudaFuncSetAttribute(k_elements, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)smem));
     if (active_only) STA_TRY(launch_active_list(c, nullptr, nullptr, nullptr, s));
     int64_t blocks = (c->T + EL_TPB - 1) / EL_TPB;
     int per_sm = 0;
-    STA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_elements, EL_TPB, smem));
+    STA_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_elements, EL_TPB, 0));
     if (per_sm < 1) per_sm = 1;
     int64_t cap = (int64_t)per_sm * c->num_sms;
     if (blocks > cap) blocks = cap;
-    k_elements<<<(unsigned)blocks, EL_TPB, smem, s>>>(c->X, c->tets, c->mat,
-                                                      active_only ? c->act_list : nullptr,
-                                                      active_only ? c->act_count : nullptr, c->T,
-                                                      c->Ke, c->counters);
+    k_elements<<<(unsigned)blocks, EL_TPB, 0, s>>>(c->X, c->tets, c->mat,
+                                                   active_only ? c->act_list : nullptr,
+                                                   active_only ? c->act_count : nullptr, c->T,
+                                                   c->krun, c->Ke, c->counters);
     STA_CUDA_TRY(cudaGetLastError());
     return STA_OK;
 }
@@ -344,7 +356,7 @@ int launch_expand_elements(Ctx *c, const int32_t *ids, int64_t n, double *out, c
     int64_t items = 144 * n;
     int64_t blocks = (items + 255) / 256;
     if (blocks > 65535LL * 16) blocks = 65535LL * 16;
-    k_expand<<<(unsigned)blocks, 256, 0, s>>>(c->Ke, c->tets, c->T, ids, n, out);
+    k_expand<<<(unsigned)blocks, 256, 0, s>>>(c->Ke, c->krun, c->tets, c->T, ids, n, out);
     STA_CUDA_TRY(cudaGetLastError());
     return STA_OK;
 }

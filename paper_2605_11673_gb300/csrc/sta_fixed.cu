@@ -46,14 +46,14 @@ __device__ __forceinline__ int32_t unit_key(int4 bm, bool diag, int q) {
 // m_k: maximum exponent field over the superset contributions of every entry.
 // One thread per (tet, unit slot).
 __global__ void k_fx_emax(int64_t T, const int32_t *__restrict__ tunit, const int4 *__restrict__ bmeta,
-                          const double *__restrict__ Ke, int32_t *__restrict__ emax) {
+                          const int32_t *__restrict__ krun, const double *__restrict__ Ke,
+                          int32_t *__restrict__ emax) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 10 * T;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = i / 10;
         const int s = (int)(i % 10);
         const int4 bm = __ldg(bmeta + __ldg(tunit + i));
         const bool diag = s < 4;
-        const double *run = Ke + ke_slot_at(T, t, s);
+        const double *run = Ke + __ldg(krun + i);
         for (int q = 0; q < (diag ? 6 : 9); ++q) atomicMax(&emax[unit_key(bm, diag, q)], exp_field(run[q]));
     }
 }
@@ -65,7 +65,7 @@ __global__ void k_fx_exponents(int64_t nunits, const int4 *__restrict__ bmeta,
          u += (int64_t)gridDim.x * blockDim.x) {
         const int4 bm = bmeta[u];
         const bool diag = bm.y & 1;
-        const int L = ceil_log2(bm.w - bm.z > 0 ? bm.w - bm.z : 1);
+        const int L = ceil_log2(bm.w > 0 ? bm.w : 1);
         for (int q = 0; q < (diag ? 6 : 9); ++q) {
             const int32_t k = unit_key(bm, diag, q);
             const int m = emax[k];
@@ -79,15 +79,14 @@ __global__ void k_fx_exponents(int64_t nunits, const int4 *__restrict__ bmeta,
 // q of every superset contribution, at the element-cache offsets of Ke.  One thread per
 // (tet, unit slot).
 __global__ void k_fx_quantize(int64_t T, const int32_t *__restrict__ tunit,
-                              const int4 *__restrict__ bmeta, const double *__restrict__ Ke,
-                              const int16_t *__restrict__ e, long long *__restrict__ Kq) {
+                              const int4 *__restrict__ bmeta, const int32_t *__restrict__ krun,
+                              const double *__restrict__ Ke, const int16_t *__restrict__ e, long long *__restrict__ Kq) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 10 * T;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = i / 10;
         const int s = (int)(i % 10);
         const int4 bm = __ldg(bmeta + __ldg(tunit + i));
         const bool diag = s < 4;
-        const int64_t off = ke_slot_at(T, t, s);
+        const int64_t off = __ldg(krun + i);
         for (int q = 0; q < (diag ? 6 : 9); ++q)
             Kq[off + q] = __double2ll_rn(Ke[off + q] * pow2i(-e[unit_key(bm, diag, q)]));
     }
@@ -118,10 +117,11 @@ constexpr int FX_CLAIM_THREADS = 256;
 
 __global__ void __launch_bounds__(FX_CLAIM_THREADS)
 k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
-                           const int64_t *__restrict__ m_dev, int64_t T,
-                           const int32_t *__restrict__ tunit, const int32_t *__restrict__ cslot,
-                           int32_t *__restrict__ ccode, uint8_t *__restrict__ mask,
-                           int32_t *__restrict__ owner, int32_t *__restrict__ list,
+                           const int64_t *__restrict__ m_dev,
+                           const int32_t *__restrict__ tunit, const int32_t *__restrict__ tpos,
+                           const int32_t *__restrict__ krun, UnitState *__restrict__ ustate,
+                           uint32_t *__restrict__ uext, uint8_t *__restrict__ mask,
+                           int32_t *__restrict__ list,
                            unsigned long long *counters, const int4 *__restrict__ bmeta,
                            const long long *__restrict__ Kq, long long *__restrict__ S) {
     const int64_t n = 10 * (m_dev ? *m_dev : m);
@@ -137,10 +137,8 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
             const uint32_t on = w >> 31;
             const int s = (int)(i % 10);
             if (s == 0) mask[t] = (uint8_t)on;
-            const int32_t slot = cslot[10 * (int64_t)t + s];
             u = tunit[10 * (int64_t)t + s];
-            const int64_t off = ke_slot_at(T, t, s);
-            ccode[slot] = (int32_t)((uint32_t)off | (on << 31));
+            const int64_t off = krun[10 * (int64_t)t + s];
             diag = s < 4;
             const int4 bm = __ldg(bmeta + u);
             for (int q = 0; q < (diag ? 6 : 9); ++q) {
@@ -148,7 +146,7 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
                 atomicAdd(reinterpret_cast<unsigned long long *>(&S[unit_key(bm, diag, q)]),
                           (unsigned long long)(on ? v : -v));
             }
-            won = atomicCAS(&owner[u], INT32_MAX, 0) == INT32_MAX;
+            won = claim_unit(ustate, uext, u, tpos[10 * (int64_t)t + s], on != 0u);
         }
         const unsigned ball = __ballot_sync(0xffffffffu, won);
         const unsigned dball = __ballot_sync(0xffffffffu, won && diag);
@@ -164,7 +162,7 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
 __global__ void k_fx_convert(FoldArgs A, const int32_t *__restrict__ list,
                              const unsigned long long *__restrict__ count,
                              const int16_t *__restrict__ e, const long long *__restrict__ S,
-                             int32_t *__restrict__ owner, unsigned long long *next_count) {
+                             UnitState *__restrict__ ustate, unsigned long long *next_count) {
     if (next_count && blockIdx.x == 0 && threadIdx.x == 0) {
         next_count[0] = 0;
         next_count[2] = 0;
@@ -183,7 +181,7 @@ __global__ void k_fx_convert(FoldArgs A, const int32_t *__restrict__ list,
         if (diag && q >= 6) continue;
         const int2 mir = diag ? make_int2(0, 0) : __ldg(A.bmirror + u);
         fx_write(A, e, bm, mir, diag, q, S[unit_key(bm, diag, q)]);
-        if (q == 0) owner[u] = INT32_MAX;
+        if (q == 0) ustate[u].claims = 0;
     }
 }
 
@@ -199,7 +197,7 @@ int grid_cap(const Ctx *c, int64_t items, int threads) {
 // fixed-point arrays on first use).
 int launch_fx_prepare(Ctx *c, cudaStream_t s) {
     if (!c->fx_q) {
-        STA_TRY(dev_alloc(c, &c->fx_q, KE_STRIDE * (c->T > 0 ? c->T : 1)));
+        STA_TRY(dev_alloc(c, &c->fx_q, c->ke_len));
         STA_TRY(dev_alloc(c, &c->fx_e, c->nnz > 0 ? c->nnz : 1));
         STA_TRY(dev_alloc(c, &c->fx_s, c->nnz > 0 ? c->nnz : 1));
     }
@@ -207,11 +205,11 @@ int launch_fx_prepare(Ctx *c, cudaStream_t s) {
     // m_k in the integer-sum array (rebuilt afterwards), as int32 starting very negative
     int32_t *emax = reinterpret_cast<int32_t *>(c->fx_s);
     STA_CUDA_TRY(cudaMemsetAsync(emax, 0x80, sizeof(int32_t) * c->nnz, s));
-    k_fx_emax<<<grid_cap(c, 10 * c->T, 256), 256, 0, s>>>(c->T, c->tunit, c->bmeta, c->Ke, emax);
+    k_fx_emax<<<grid_cap(c, 10 * c->T, 256), 256, 0, s>>>(c->T, c->tunit, c->bmeta, c->krun, c->Ke, emax);
     STA_CUDA_TRY(cudaMemsetAsync(c->fx_e, 0, sizeof(int16_t) * c->nnz, s));
     k_fx_exponents<<<grid_cap(c, c->nunits, 256), 256, 0, s>>>(c->nunits, c->bmeta, emax, c->fx_e);
-    STA_CUDA_TRY(cudaMemsetAsync(c->fx_q, 0, sizeof(long long) * KE_STRIDE * c->T, s));
-    k_fx_quantize<<<grid_cap(c, 10 * c->T, 256), 256, 0, s>>>(c->T, c->tunit, c->bmeta, c->Ke,
+    STA_CUDA_TRY(cudaMemsetAsync(c->fx_q, 0, sizeof(long long) * c->ke_len, s));
+    k_fx_quantize<<<grid_cap(c, 10 * c->T, 256), 256, 0, s>>>(c->T, c->tunit, c->bmeta, c->krun, c->Ke,
                                                              c->fx_e, c->fx_q);
     STA_CUDA_TRY(cudaGetLastError());
     return STA_OK;
@@ -222,10 +220,10 @@ int launch_fx_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_d
                     unsigned long long *next_cnt) {
     const int threads = FX_CLAIM_THREADS;
     k_fx_claim<<<grid_cap(c, 10 * cap, threads), threads, 0, s>>>(
-        edited, m, m_dev, c->T, c->tunit, c->cslot, c->ccode, c->mask, c->owner, touched,
+        edited, m, m_dev, c->tunit, c->tpos, c->krun, c->ustate, c->uext, c->mask, touched,
         counters, c->bmeta, c->fx_q, c->fx_s);
     k_fx_convert<<<grid_cap(c, (10 * (cap > 0 ? cap : 1) + 2) / 3 * 32, 128), 128, 0, s>>>(
-        fold_args(c), touched, counters + 1, c->fx_e, c->fx_s, c->owner,
+        fold_args(c), touched, counters + 1, c->fx_e, c->fx_s, c->ustate,
         next_cnt ? next_cnt + 1 : nullptr);
     STA_CUDA_TRY(cudaGetLastError());
     return STA_OK;

@@ -34,60 +34,41 @@ int fail(int code, const std::string &msg);
 
 // ------------------------------------------------------------------------------------
 // Element cache: the 78 unique entries of each symmetric 12x12 element matrix, grouped by 3x3
-// node-pair block into runs, stored as two row arrays in one allocation of 84 T doubles:
-//   Kd = Ke[0 .. 24T):   row 4t + a (6 doubles, 48 B): diagonal block (a, a), entries i <= j
-//                        row-major: (0,0) (0,1) (0,2) (1,1) (1,2) (2,2)
-//   Kp = Ke[24T .. 84T): row 6t + pair(a, b) (10 doubles, 80 B: 9 entries + a +0.0 pad), a < b
-//                        local indices: the block row-major over the node with the LOWER global
-//                        id, i.e. K[3a+i][3b+j] at 3i+j if id(a) < id(b), else at 3j+i
-// with pair(0,1..3) = 0..2, pair(1,2..3) = 3..4, pair(2,3) = 5.  Every run starts on a 16-byte
-// boundary.  Oriented this way, the contribution of any tetrahedron to the node-pair block
-// (a, b), id(a) < id(b), is one row read as is (the folds never transpose), and the rows of
-// one kind have one width (whole-row gathers).  A tet's record is computed in the order
-// diagonal runs then pair runs (84 doubles, KE_STRIDE), then split between the two arrays.
+// node-pair block into runs
+//   diagonal block (a, a): 6 doubles, entries i <= j row-major (0,0) (0,1) (0,2) (1,1) (1,2) (2,2)
+//   pair block (a, b), a < b local indices: 9 doubles, the block row-major over the node with the
+//                          LOWER global id, i.e. K[3a+i][3b+j] at 3i+j if id(a) < id(b), else at 3j+i
+// and stored by fold unit (node pair), not by tetrahedron: unit u's runs follow one another from
+// Ke[bmeta[u].z] in ascending tetrahedron id, the order in which a fold adds them, every unit from
+// an even offset (16 bytes).  So a fold needs no list of addresses -- its j-th contributor's run
+// is at a fixed stride -- and reads its operands as one contiguous piece; which contributors are
+// active is a bit each (UnitState).  Oriented by node id, a run is read as is (the folds never
+// transpose).  krun[10 t + s] is the offset of tet t's run of unit slot s.
 // ------------------------------------------------------------------------------------
-constexpr int KE_STRIDE = 84;
-constexpr int KE_DIAG = 24;   // doubles of a tet's 4 diagonal runs (Kd)
-constexpr int KE_PAIR = 60;   // doubles of a tet's 6 pair runs (Kp)
+constexpr int KE_STRIDE = 84;  // doubles of the cache per tetrahedron at most (4 x 6 + 6 x (9 + pad))
+constexpr int RUN_DIAG = 6, RUN_PAIR = 9;
 
-__host__ __device__ inline int ke_diag_off(int a) { return 6 * a; }
-__host__ __device__ inline int ke_pair(int a, int b) {  // a < b
-    return a == 0 ? b - 1 : (a == 1 ? b + 1 : 5);
-}
-__host__ __device__ inline int ke_off_off(int a, int b) { return 24 + 10 * ke_pair(a, b); }
-// Ke offset of tet t's diagonal run a, and of its pair run p
-__host__ __device__ inline int64_t ke_diag_at(int64_t T, int64_t t, int a) {
-    (void)T;
-    return KE_DIAG * t + 6 * a;
-}
-__host__ __device__ inline int64_t ke_pair_at(int64_t T, int64_t t, int p) {
-    return KE_DIAG * T + KE_PAIR * t + 10 * p;
-}
 // index of (i, j), i <= j, inside a diagonal 6-run
 __host__ __device__ inline int ke_tri(int i, int j) {
     return i == 0 ? j : (i == 1 ? 2 + j : 5);
 }
 
-// Contributor code of a fold unit (node pair a <= b): tetrahedron id and the local indices of
-// the unit's nodes a (la) and b (lb) inside that tetrahedron; bit 31 holds the tetrahedron's
-// current activity (kept equal to the mask by every call that changes it).
-constexpr uint32_t CODE_ACTIVE = 0x80000000u;
+// Contributor code of a fold unit (node pair a <= b) while the lists are built: tetrahedron id and
+// the local indices of the unit's nodes a (la) and b (lb) inside that tetrahedron.
 __host__ __device__ inline int32_t contrib_code(int32_t t, int la, int lb) {
     return (t << 4) | (la << 2) | lb;
 }
 __host__ __device__ inline int32_t code_tet(int32_t code) { return (code >> 4) & 0x07ffffff; }
 
-// Contributor word of a unit list (ccode after create): the element-cache offset of the
-// contributor's run for the unit (ke_diag_at / ke_pair_at) | active << 31.
-__host__ __device__ inline uint32_t word_offset(uint32_t w) { return w & 0x7fffffffu; }
-__host__ __device__ inline int32_t word_tet(uint32_t w, int64_t T) {
-    const int64_t off = word_offset(w);
-    return (int32_t)(off < KE_DIAG * T ? off / KE_DIAG : (off - KE_DIAG * T) / KE_PAIR);
-}
-// the run of tet t for unit slot s (0..3 diagonal, 4..9 pairs)
-__host__ __device__ inline int64_t ke_slot_at(int64_t T, int64_t t, int s) {
-    return s < 4 ? ke_diag_at(T, t, s) : ke_pair_at(T, t, s - 4);
-}
+// Activity of a unit's contributors, kept equal to the mask by every call that changes it, and the
+// claims of the streaming frame in progress.  Contributor j's bit: w0 bit j (j < 32), w1 bit j - 32
+// (j < 64), else bit j % 32 of uext[xoff + j / 32 - 2].  w0 and claims are one 64-bit word to the
+// claim kernels: one atomic sets or clears the bit (by adding or subtracting it) and counts the
+// claim, and the thread that finds no claim yet has won the unit.  claims is 0 between frames.
+struct __align__(16) UnitState {
+    uint32_t w0, claims, w1, xoff;  // xoff: UNIT_NARROW for at most 64 contributors
+};
+constexpr uint32_t UNIT_NARROW = 0xffffffffu;
 
 // The 10 unit slots of a tetrahedron: 0..3 diagonal (la, la), 4..9 the pairs (0,1) (0,2) (0,3)
 // (1,2) (1,3) (2,3).
@@ -101,10 +82,9 @@ __host__ __device__ inline int slot_of(int la, int lb) {  // unordered local pai
     return 4 + (lo == 0 ? hi - 1 : (lo == 1 ? hi + 1 : 5));
 }
 
-// Lanes of the rebuild fold per unit (one fold entry each): a diagonal unit folds its 6
-// distinct entries, an off-diagonal unit its 9.
-constexpr int FOLD_TASKS_DIAG = 6;
-constexpr int FOLD_TASKS_PAIR = 9;
+// Units of one chunk of the rebuild fold -- their entries (9 per pair unit, 6 per diagonal unit) are
+// whole rounds of 32 lanes, the last one nearly -- and the bytes of their runs.
+constexpr int CHUNK_PAIR = 28, CHUNK_DIAG = 16, CHUNK_BYTES = 12 * 1024;
 
 // Frame block: what one streaming frame moves to the device in a single transfer -- the
 // edited count, the frame's counters (zeroed by the host) and the edited list (tet id | new
@@ -166,18 +146,20 @@ struct Ctx {
     // (3b+j, 3a+i) fold the same operands in the same order (the element matrices are exactly
     // symmetric), so one fold per unit writes both blocks.
     int64_t nunits = 0;
-    int64_t ntiles = 0;
-    int4 *ftile = nullptr;         // ntiles: rebuild fold tiles {first unit, q0 | diag << 4 |
-                                   //   entries << 5, code range of the tile's units}
-    // zero-fill rebuild (sta_rebuild.cu): per unit its first tile | reaches the next << 31;
-    // per tile whether its units are diagonal, and its flag "fold this tile"
-    int32_t *utile = nullptr;      // nunits
-    uint8_t *tdiag = nullptr;      // ntiles
-    uint8_t *tflag = nullptr;      // ntiles: zero-fill flags, all zero between rebuilds
-    int4 *bmeta = nullptr;         // nunits: {value offset of (a,b), rs_a << 1 | diagonal, c0, c1}
+    int64_t nchunks = 0;
+    int2 *chunks = nullptr;        // nchunks: rebuild fold chunks {first unit, units | diagonal << 8}
+    uint8_t *cflag = nullptr;      // nchunks: the zero-fill rebuild's "fold this chunk"
+    unsigned int *d_fault = nullptr;  // host-mapped word: a fold's bounded wait ran out
+    unsigned int *h_fault = nullptr;
+    int4 *bmeta = nullptr;         // nunits: {value offset of (a,b), rs_a << 1 | diagonal, offset of
+                                   //   the unit's first run, contributors}
     int2 *bmirror = nullptr;       // nunits: {value offset of (b,a), rs_b}
-    int32_t *ccode = nullptr;      // 10 T: unit contributor words (word_offset), ascending tet id
-    int32_t *cslot = nullptr;      // T x 10: position in ccode of tet t's unit slot
+    UnitState *ustate = nullptr;   // nunits: contributor activity and claims
+    uint32_t *uext = nullptr;      // activity words of contributors 64 and up
+    int32_t *uc0 = nullptr;        // nunits + 1: first position of each unit's contributors in ctet
+    int32_t *ctet = nullptr;       // 10 T: contributors of every unit, ascending tet id
+    int32_t *tpos = nullptr;       // T x 10: tet t's place among the contributors of its slot's unit
+    int32_t *krun = nullptr;       // T x 10: offset of tet t's run of a slot in Ke
     int32_t *tunit = nullptr;      // T x 10: unit of tet t's slot (4 diagonal, 6 pairs)
     int32_t *nt_ptr = nullptr;     // n + 1: node -> incident tetrahedra
     int32_t *nt_list = nullptr;    // 4 T: incident tetrahedra, ascending id
@@ -188,15 +170,15 @@ struct Ctx {
     unsigned long long *act_count = nullptr;
 
     // state
-    double *Ke = nullptr;       // 84 T: element cache, diagonal runs then pair runs (KE_DIAG, KE_PAIR)
+    int64_t ke_len = 0;         // doubles of the element cache (<= 84 T)
+    double *Ke = nullptr;       // ke_len: element cache
     // update policy (STA_POLICY_*) and the fixed-point state (sta_fixed.cu), allocated on first use
     int policy = STA_POLICY_REFOLD;
-    long long *fx_q = nullptr;  // 84 T: quantised contributions at the element-cache offsets
+    long long *fx_q = nullptr;  // ke_len: quantised contributions at the element-cache offsets
     int16_t *fx_e = nullptr;    // nnz: exponent of each entry (keyed by its upper-block index)
     long long *fx_s = nullptr;  // nnz: exact integer sum of each entry's active contributions
     uint8_t *mask = nullptr;    // T
     double *val = nullptr;      // nnz
-    int32_t *owner = nullptr;   // nunits: streaming dedupe slot, INT32_MAX when free
     int32_t *touched = nullptr; // nunits: list of units touched by the current frame
     // [0] bad elements, [1] touched units, [2] first bad element, [3] touched CSR entries
     unsigned long long *counters = nullptr;
@@ -327,7 +309,7 @@ int launch_fx_prepare(Ctx *c, cudaStream_t s);                   // sta_fixed.cu
 int launch_fx_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_dev, int64_t cap,
                     int32_t *touched, unsigned long long *counters, cudaStream_t s,
                     unsigned long long *next_cnt);
-int launch_mask_bits(Ctx *c, cudaStream_t s);                    // codes <- mask
+int launch_mask_bits(Ctx *c, cudaStream_t s);                    // activity bits <- mask
 int launch_values(Ctx *c, cudaStream_t s);  // the operator's rebuild (elasticity or proxy)
 int launch_dyn_qmass(Ctx *c, cudaStream_t s);     // sta_dyn.cu (no-ops unless set up)
 int launch_dyn_mass_all(Ctx *c, cudaStream_t s);

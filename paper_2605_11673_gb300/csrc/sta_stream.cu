@@ -3,6 +3,8 @@
 // exactly those with the rebuild's operands, order and operations.  Also the mask-to-activity
 // pass of a full rebuild with a new mask.  Fold definition and shared device code:
 // sta_fold.cuh.
+#include "sta_bulk.cuh"
+#include "sta_claim.cuh"
 #include "sta_fold.cuh"
 
 namespace sta {
@@ -18,147 +20,70 @@ namespace {
 // 9 entries (i, j)).  A warp's step count is its longest fold, and on GB300 an FP64 warp
 // instruction holds the SM's FP64 pipe for about 16 cycles: mixing a ~24-contribution diagonal
 // unit with ~6-contribution pair units would leave most of those steps idle.
-// The unit's active codes are compacted (in list order) into shared memory first, three codes
-// per lane and step.  Then the element-cache runs of the active contributors (48 B for a
-// diagonal unit, 80 B for a pair; 16-byte aligned) are copied into shared memory with 16-byte
-// cp.async copies, all in flight at once, so a unit costs one round trip for its operands
-// however long its list; the fold reads them from there.  A unit with more than ENT_SCAP
-// active contributions loads its operands from global memory instead (4 steps in flight).
+// A lane's operands are one double of each active contributor's run, whose addresses follow from
+// the unit record and its activity bits: it copies up to ENT_DEPTH of them into its column of
+// shared memory with 8-byte cp.async, all in flight at once and none in a register, then adds them
+// in order; only the lane itself reads its column, so no barrier is needed.
 // Operands, order and operations are those of k_fold_flat, so the values are the same bits.
 // ------------------------------------------------------------------------------------------
 constexpr int ENT_DG = 5;      // diagonal units per warp round (6 lanes each: 30 lanes)
 constexpr int ENT_PG = 3;      // pair units per warp round (9 lanes each: 27 lanes)
-constexpr int ENT_DCAP = 64;   // listed active contributions of a diagonal unit (larger: direct)
-constexpr int ENT_PCAP = 96;   // the same for a pair unit
-constexpr int ENT_SCAP = 24;   // active contributions whose runs are staged in shared memory
+constexpr int ENT_DEPTH = 24;  // operands of a lane in flight
 constexpr int ENT_WARPS = 4;
-constexpr int ENT_SOP = ENT_DG * ENT_DCAP > ENT_PG * ENT_PCAP ? ENT_DG * ENT_DCAP : ENT_PG * ENT_PCAP;
-constexpr int ENT_STAGE = ENT_DG * ENT_SCAP * 6;  // doubles per warp: = ENT_PG * ENT_SCAP * 10
-static_assert(ENT_DG * ENT_SCAP * 6 == ENT_PG * ENT_SCAP * 10, "stage shared by both kinds");
-
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sa), "l"(gmem) : "memory");
-}
 
 // One warp round over units first .. first+NG-1 of one kind (k-th diagonal unit at list[k],
-// k-th pair unit at list[cap - 1 - k]); `sop`, `stage` are the warp's shared buffers.
+// k-th pair unit at list[cap - 1 - k]); `col`: the lane's column of the warp's shared buffer.
 template <bool DIAG>
-__device__ __forceinline__ void fold_units(const FoldArgs &A, const int32_t *__restrict__ list,
-                                           int64_t first, int64_t n_units, int64_t cap,
-                                           int32_t *__restrict__ owner, uint32_t *sop_w,
-                                           double *stage_w, int lane, bool has_eps) {
-    constexpr int GW = DIAG ? 6 : 9;                 // lanes (entries) per unit
+__device__ __forceinline__ void fold_units(const FoldArgs &A, UnitState *__restrict__ ustate,
+                                           const int32_t *__restrict__ list, int64_t first,
+                                           int64_t n_units, int64_t cap, double *col, int lane,
+                                           bool has_eps) {
+    constexpr int GW = DIAG ? RUN_DIAG : RUN_PAIR;   // lanes (entries) per unit
     constexpr int NG = DIAG ? ENT_DG : ENT_PG;       // units per warp round
-    constexpr int CAP = DIAG ? ENT_DCAP : ENT_PCAP;  // listed active contributions
-    constexpr int RUN = DIAG ? 6 : 10;               // staged doubles per run (48 B, 80 B)
-    constexpr int CPR = DIAG ? 3 : 5;                // 16-byte copies per run
-    const unsigned FULL = 0xffffffffu;
     const int g = lane / GW, q = lane % GW;          // g == NG: idle lanes
     const int64_t k = first + g;
     const bool valid = g < NG && k < n_units;
-    uint32_t *sop = sop_w + (g < NG ? g : 0) * CAP;
-    double *stage = stage_w + (g < NG ? g : 0) * (ENT_SCAP * RUN);  // run j at stage[RUN j]
     int4 bm = make_int4(0, 0, 0, 0);
     int2 mir = make_int2(0, 0);
+    uint4 st = make_uint4(0, 0, 0, 0);
+    int32_t u = 0;
     if (valid) {
-        const int32_t u = __ldg(list + (DIAG ? k : cap - 1 - k));
+        u = __ldg(list + (DIAG ? k : cap - 1 - k));
         bm = __ldg(A.bmeta + u);
         if (!DIAG) mir = __ldg(A.bmirror + u);
-        if (q == 0) owner[u] = INT32_MAX;  // release the claim (all claims are done)
+        st = *reinterpret_cast<const uint4 *>(ustate + u);
     }
-    // compact the unit's active contributors (as operand bases), its GW lanes striding over its
-    // list, three GW-code chunks loaded together and taken in list order
-    int nact = 0;
-    const int span = valid ? bm.w - bm.z : 0;
-    const int max_span = __reduce_max_sync(FULL, span);
-    const unsigned below_q = (1u << q) - 1u;
-    for (int c0 = 0; c0 < max_span; c0 += 3 * GW) {
-        int32_t kc[3];
-#pragma unroll
-        for (int h = 0; h < 3; ++h) {
-            const int c = c0 + GW * h + q;
-            kc[h] = (valid && c < span) ? __ldg(A.ccode + bm.z + c) : 0;
-        }
-#pragma unroll
-        for (int h = 0; h < 3; ++h) {
-            const unsigned m = __ballot_sync(FULL, kc[h] < 0);
-            const unsigned gm = (m >> (GW * g)) & ((1u << GW) - 1u);
-            const int pos = nact + __popc(gm & below_q);
-            if (kc[h] < 0 && pos < CAP) sop[pos] = word_offset((uint32_t)kc[h]);
-            nact += __popc(gm);
-        }
-    }
-    __syncwarp();
-    const bool big = valid && nact > CAP;
-    if (big && q == 0) fold_direct(A, bm, mir);  // rare: more active contributions than listed
-    const bool mine = valid && !big;
-    // stage the runs of the unit's active contributors, the unit's GW lanes sharing the copies
-    const bool staged = mine && nact <= ENT_SCAP;
-    if (staged) {
-        for (int kk = q; kk < nact * CPR; kk += GW) {
-            const int j = kk / CPR, p = kk - j * CPR;
-            cp_async16(stage + RUN * j + 2 * p, A.Ke + sop[j] + 2 * p);
-        }
-    }
-    asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
-    __syncwarp();
+    ActiveRuns it(valid, st, bm.w, bm.z + q, GW, A.uext);
+    const int n = it.count();
+    const int maxn = __reduce_max_sync(0xffffffffu, n);
     double acc = 0.0;
-    const int ns = staged ? nact : 0;
-    const int maxs = __reduce_max_sync(FULL, ns);
-    if (maxs > 0) {  // warp-uniform; the same operands in the same order as below
-        if (ns > 0) acc = plus_zero(stage[q]);  // the first contribution: +0.0 + v
-        for (int j = 1; j < maxs; ++j)
-            if (j < ns) acc += stage[RUN * j + q];
+    for (int j0 = 0; j0 < maxn; j0 += ENT_DEPTH) {  // warp-uniform
+        const int c = n - j0 < ENT_DEPTH ? n - j0 : ENT_DEPTH;  // this lane's operands (may be < 0)
+        const int cm = maxn - j0 < ENT_DEPTH ? maxn - j0 : ENT_DEPTH;
+        for (int j = 0; j < c; ++j) cp_async<8>(col + 32 * j, A.Ke + it.next());
+        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+        __syncwarp();
+        for (int j = 0; j < cm; ++j)
+            if (j < c) acc = j0 + j == 0 ? plus_zero(col[0]) : acc + col[32 * j];
+        __syncwarp();
     }
-    const int n = mine && !staged ? nact : 0;  // longer lists: operands from global memory
-    const int maxn = __reduce_max_sync(FULL, n);
-#define STA_LD(j) ((j) < n ? __ldg(A.Ke + sop[(j)] + q) : 0.0)
-    if (maxn > 0) {  // warp-uniform guards, as in k_fold_flat
-        if (n > 0) acc = plus_zero(STA_LD(0));  // the first contribution: +0.0 + v
-        double v0 = 0.0, v1 = 0.0, v2 = 0.0, v3 = 0.0;
-        if (maxn > 1) v0 = STA_LD(1);
-        if (maxn > 2) v1 = STA_LD(2);
-        if (maxn > 3) v2 = STA_LD(3);
-        if (maxn > 4) v3 = STA_LD(4);
-        int j = 1;
-        for (; j + 4 <= maxn; j += 4) {  // next 4 operands in flight
-            double x0 = 0.0, x1 = 0.0, x2 = 0.0, x3 = 0.0;
-            if (j + 4 < maxn) x0 = STA_LD(j + 4);
-            if (j + 5 < maxn) x1 = STA_LD(j + 5);
-            if (j + 6 < maxn) x2 = STA_LD(j + 6);
-            if (j + 7 < maxn) x3 = STA_LD(j + 7);
-            if (j < n) acc += v0;
-            if (j + 1 < n) acc += v1;
-            if (j + 2 < n) acc += v2;
-            if (j + 3 < n) acc += v3;
-            v0 = x0;
-            v1 = x1;
-            v2 = x2;
-            v3 = x3;
-        }
-        if (j < maxn && j < n) acc += v0;
-        if (j + 1 < maxn && j + 1 < n) acc += v1;
-        if (j + 2 < maxn && j + 2 < n) acc += v2;
+    if (!valid) return;
+    // release the claim: all claims are done, and the other lanes of the unit do not read it
+    if (q == 0) ustate[u].claims = 0;
+    if (DIAG) {
+        // 6-run entry q = (i, j), i <= j
+        const int i = q < 3 ? 0 : (q < 5 ? 1 : 2), j = q < 3 ? q : (q < 5 ? q - 2 : 2);
+        double a = acc;
+        if (i == j && has_eps) a += A.eps;
+        double *out = A.val + bm.x;
+        const int rs = bm.y >> 1;
+        out[i * rs + j] = a;
+        if (i != j) out[j * rs + i] = a;
+    } else {
+        const int qi = q / 3, qj = q % 3;
+        A.val[bm.x + qi * (bm.y >> 1) + qj] = acc;
+        A.val[mir.x + qj * mir.y + qi] = acc;
     }
-#undef STA_LD
-    if (mine) {
-        if (DIAG) {
-            // 6-run entry q = (i, j), i <= j
-            const int i = q < 3 ? 0 : (q < 5 ? 1 : 2), j = q < 3 ? q : (q < 5 ? q - 2 : 2);
-            double a = acc;
-            if (i == j && has_eps) a += A.eps;
-            double *out = A.val + bm.x;
-            const int rs = bm.y >> 1;
-            out[i * rs + j] = a;
-            if (i != j) out[j * rs + i] = a;
-        } else {
-            const int qi = q / 3, qj = q % 3;
-            A.val[bm.x + qi * (bm.y >> 1) + qj] = acc;
-            A.val[mir.x + qj * mir.y + qi] = acc;
-        }
-    }
-    __syncwarp();
 }
 
 // count[0]: diagonal units | pair units << 32 (the claim kernel's); count[2] gets the frame's
@@ -167,12 +92,12 @@ __device__ __forceinline__ void fold_units(const FoldArgs &A, const int32_t *__r
 // given, is the count pair of the next frame (graph mode alternates two), zeroed here so that
 // the captured frame needs no memset node of its own.
 __global__ void __launch_bounds__(ENT_WARPS * 32)
-k_fold_entries(FoldArgs A, const int32_t *__restrict__ list, unsigned long long *count, int64_t cap,
-               int32_t *__restrict__ owner, unsigned long long *host_count,
+k_fold_entries(FoldArgs A, UnitState *__restrict__ ustate, const int32_t *__restrict__ list,
+               unsigned long long *count, int64_t cap, unsigned long long *host_count,
                unsigned long long *next_count) {
-    __shared__ uint32_t sop_all[ENT_WARPS][ENT_SOP];
-    __shared__ __align__(16) double stage_all[ENT_WARPS][ENT_STAGE];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __shared__ double stage[ENT_WARPS][ENT_DEPTH * 32];
+    const int lane = threadIdx.x & 31;
+    double *col = stage[threadIdx.x >> 5] + lane;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     const unsigned long long packed = *count;  // final: the claim kernel has ended
@@ -190,33 +115,31 @@ k_fold_entries(FoldArgs A, const int32_t *__restrict__ list, unsigned long long 
     const bool has_eps = A.eps != 0.0;
     for (int64_t item = warp; item < gd + gp; item += nwarps) {  // warp-uniform
         if (item < gd)
-            fold_units<true>(A, list, item * ENT_DG, nd, cap, owner, sop_all[wid], stage_all[wid],
-                             lane, has_eps);
+            fold_units<true>(A, ustate, list, item * ENT_DG, nd, cap, col, lane, has_eps);
         else
-            fold_units<false>(A, list, (item - gd) * ENT_PG, np, cap, owner, sop_all[wid],
-                              stage_all[wid], lane, has_eps);
+            fold_units<false>(A, ustate, list, (item - gd) * ENT_PG, np, cap, col, lane, has_eps);
     }
 }
 
 // Streaming, phase 1: apply the frame's mask changes and collect the touched fold units.  One
-// thread per (edited tet k, unit slot s): it writes the contributor's new activity bit, and
-// claims the slot's unit with a compare-and-swap on its owner word (INT32_MAX = free); the
-// thread that wins appends the unit to the fold list, a diagonal unit (slots 0-3) at the front
-// and a pair unit at the back of the `cap` entries, both counted by one CTA-aggregated atomic
-// on counters[1] = diagonal units | pair units << 32 (a large frame's warps all appending to
-// that one word serialise at the L2; per CTA there are 8 times fewer).  The fold releases the claims and counts
-// the touched entries.  The list order depends on scheduling, the values do not (each unit
-// folds independently).  edited[k] = tet id | (new state << 31); the edited count is *m_dev if
-// m_dev, else m; counters[1] starts at zero; a frame lists at most 10 units per edited tet and
-// at most every unit once, so the two ends never meet when cap >= min(10 m, units).
+// thread per (edited tet k, unit slot s): it moves the contributor's activity bit and claims the
+// slot's unit (claim_unit); the thread that wins appends the unit to the fold list, a diagonal
+// unit (slots 0-3) at the front and a pair unit at the back of the `cap` entries, both counted by
+// one CTA-aggregated atomic on counters[1] = diagonal units | pair units << 32 (a large frame's
+// warps all appending to that one word serialise at the L2; per CTA there are 8 times fewer).
+// The fold releases the claims and counts the touched entries.  The list order depends on
+// scheduling, the values do not (each unit folds independently).  edited[k] = tet id | (new
+// state << 31); the edited count is *m_dev if m_dev, else m; counters[1] starts at zero; a frame
+// lists at most 10 units per edited tet and at most every unit once, so the two ends never meet
+// when cap >= min(10 m, units).
 constexpr int CLAIM_THREADS = 256;
 
 __global__ void __launch_bounds__(CLAIM_THREADS)
 k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
-                               const int64_t *__restrict__ m_dev, int64_t T,
+                               const int64_t *__restrict__ m_dev,
                                const int32_t *__restrict__ tunit,
-                               const int32_t *__restrict__ cslot, int32_t *__restrict__ ccode,
-                               uint8_t *__restrict__ mask, int32_t *__restrict__ owner,
+                               const int32_t *__restrict__ tpos, UnitState *__restrict__ ustate,
+                               uint32_t *__restrict__ uext, uint8_t *__restrict__ mask,
                                int32_t *__restrict__ list, int64_t cap,
                                unsigned long long *counters) {
     // per warp of the CTA: its packed winner counts, then its offset; the CTA's base
@@ -235,12 +158,9 @@ k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
             const uint32_t on = w >> 31;
             const int s = (int)(i % 10);
             if (s == 0) mask[t] = (uint8_t)on;
-            const int32_t slot = cslot[10 * (int64_t)t + s];
             u = tunit[10 * (int64_t)t + s];
-            // the word is (t, s)'s run offset | activity: written without reading it back
-            ccode[slot] = (int32_t)((uint32_t)ke_slot_at(T, t, s) | (on << 31));
             diag = s < 4;
-            won = atomicCAS(&owner[u], INT32_MAX, 0) == INT32_MAX;
+            won = claim_unit(ustate, uext, u, tpos[10 * (int64_t)t + s], on != 0u);
         }
         const unsigned dball = __ballot_sync(0xffffffffu, won && diag);
         const unsigned pball = __ballot_sync(0xffffffffu, won && !diag);
@@ -266,14 +186,37 @@ k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
     }
 }
 
-// Activity bits of all contributor codes from the mask (full rebuild with a new mask).
-__global__ void k_mask_bits(int32_t *__restrict__ ccode, int64_t n, int64_t T,
-                            const uint8_t *__restrict__ mask) {
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-         k += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t code = (uint32_t)ccode[k];
-        const uint32_t on = mask[word_tet(code, T)] ? CODE_ACTIVE : 0u;
-        ccode[k] = (int32_t)((code & ~CODE_ACTIVE) | on);
+// Activity bits of every unit from the mask (full rebuild with a new mask).  A lane per unit, four
+// contributors in flight (neighbouring units have lists of equal length, and their lists are
+// neighbours in memory); whole state words are written back.
+__global__ void __launch_bounds__(256)
+k_mask_bits(int64_t nunits, const int32_t *__restrict__ uc0, const int32_t *__restrict__ ctet,
+            const uint8_t *__restrict__ mask, uint4 *__restrict__ ustate,
+            uint32_t *__restrict__ uext) {
+    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < nunits;
+         u += (int64_t)gridDim.x * blockDim.x) {
+        const int32_t c0 = __ldg(uc0 + u), cnt = __ldg(uc0 + u + 1) - c0;
+        uint4 st = ustate[u];
+        uint32_t word = 0;
+        st.x = st.z = 0u;
+        for (int32_t j = 0; j < cnt; j += 4) {
+            int32_t t[4];
+            uint32_t on[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) t[k] = j + k < cnt ? __ldg(ctet + c0 + j + k) : -1;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) on[k] = t[k] >= 0 && __ldg(mask + t[k]) ? 1u : 0u;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) word |= on[k] << ((j + k) & 31);
+            if (((j + 4) & 31) == 0 || j + 4 >= cnt) {  // a word of 32 is complete
+                const int w = j >> 5;
+                if (w == 0) st.x = word;
+                else if (w == 1) st.z = word;
+                else uext[st.w + w - 2] = word;
+                word = 0;
+            }
+        }
+        ustate[u] = st;
     }
 }
 
@@ -300,7 +243,7 @@ int launch_fold_list(Ctx *c, const int32_t *list, int64_t cap, unsigned long lon
     // resident CTAs
     const int grid = persistent_grid(c, (const void *)k_fold_entries, threads,
                                      (max_items + ENT_PG - 1) / ENT_PG * 32);
-    k_fold_entries<<<grid, threads, 0, s>>>(fold_args(c), list, count, cap, c->owner, host_count,
+    k_fold_entries<<<grid, threads, 0, s>>>(fold_args(c), c->ustate, list, count, cap, host_count,
                                             next_count);
     STA_CUDA_TRY(cudaGetLastError());
     return STA_OK;
@@ -308,11 +251,11 @@ int launch_fold_list(Ctx *c, const int32_t *list, int64_t cap, unsigned long lon
 
 int launch_mask_bits(Ctx *c, cudaStream_t s) {
     if (c->T == 0 || c->op == STA_OP_PROXY) return STA_OK;  // the proxy reads the mask itself
-    const int64_t n = 10 * c->T;
-    int64_t grid = (n + 255) / 256;
+    int64_t grid = (c->nunits + 255) / 256;
     const int64_t cap = (int64_t)c->num_sms * 8;
     if (grid > cap) grid = cap;
-    k_mask_bits<<<(unsigned)grid, 256, 0, s>>>(c->ccode, n, c->T, c->mask);
+    k_mask_bits<<<(unsigned)grid, 256, 0, s>>>(c->nunits, c->uc0, c->ctet, c->mask,
+                                             reinterpret_cast<uint4 *>(c->ustate), c->uext);
     STA_CUDA_TRY(cudaGetLastError());
     return STA_OK;
 }
@@ -342,9 +285,8 @@ int launch_stream_frame(Ctx *c, const int32_t *edited, const int64_t *m_dev,
     int64_t g = (10 * cap + threads - 1) / threads;
     const int64_t gmax = (int64_t)c->num_sms * 16;
     g = g < 1 ? 1 : (g > gmax ? gmax : g);
-    k_stream_claim<<<(unsigned)g, threads, 0, s>>>(edited, 0, m_dev, c->T, c->tunit, c->cslot,
-                                                   c->ccode, c->mask, c->owner, c->touched,
-                                                   c->nunits, cnt);
+    k_stream_claim<<<(unsigned)g, threads, 0, s>>>(edited, 0, m_dev, c->tunit, c->tpos, c->ustate,
+                                                   c->uext, c->mask, c->touched, c->nunits, cnt);
     STA_CUDA_TRY(cudaGetLastError());
     STA_TRY(launch_fold_list(c, c->touched, c->nunits, cnt + 1, 10 * (cap > 0 ? cap : 1), s,
                              c->d_count_mapped, next_cnt ? next_cnt + 1 : nullptr));
@@ -375,9 +317,9 @@ int launch_stream_scratch(Ctx *c, int64_t m, const int32_t *d_edited, int32_t *t
         const int threads = CLAIM_THREADS;
         const int64_t g = (10 * m + threads - 1) / threads;
         // the touched list holds 10 m units (at most 10 per edited tet)
-        k_stream_claim<<<(unsigned)g, threads, 0, s>>>(d_edited, m, nullptr, c->T, c->tunit, c->cslot,
-                                                       c->ccode, c->mask, c->owner, touched,
-                                                       10 * m, counters);
+        k_stream_claim<<<(unsigned)g, threads, 0, s>>>(d_edited, m, nullptr, c->tunit, c->tpos,
+                                                       c->ustate, c->uext, c->mask, touched, 10 * m,
+                                                       counters);
         STA_CUDA_TRY(cudaGetLastError());
         STA_TRY(launch_fold_list(c, touched, 10 * m, counters + 1, 10 * m, s, nullptr, nullptr));
     }
