@@ -559,13 +559,19 @@ def sta_batch_instance(h: int, i: int, owner=None):
 
 def sta_batch_apply_edits(h: int, edits_per_instance, stream=None) -> None:
     """edits_per_instance: list of (m_i, 3) int32 arrays with instance-local tet ids."""
-    parts = [_host(e, np.int32).reshape(-1, 3) for e in edits_per_instance]
+    parts = list(edits_per_instance)
+    try:  # (m_i, 3) int32 arrays are joined as they are
+        allp = np.concatenate(parts)
+    except ValueError:  # none, or of other shapes
+        allp = None
+    if allp is None or allp.dtype != np.int32 or allp.ndim != 2 or allp.shape[1] != 3:
+        parts = [_host(e, np.int32).reshape(-1, 3) for e in parts]
+        allp = np.concatenate(parts, 0) if parts else np.zeros((0, 3), np.int32)
     k = _sizes(h)["k"]
     if len(parts) != k:
         raise ValueError(f"one edit list per instance: {k} expected, got {len(parts)}")
-    counts = (C.c_int64 * len(parts))(*[p.shape[0] for p in parts])
-    allp = np.ascontiguousarray(np.concatenate(parts, 0)) if parts else np.zeros((0, 3), np.int32)
-    _check(load_library().sta_batch_apply_edits(h, counts, allp.ctypes.data if allp.shape[0] else None,
+    counts = (C.c_int64 * k)(*map(len, parts))
+    _check(load_library().sta_batch_apply_edits(h, counts, _ptr(allp) if allp.shape[0] else None,
                                                  _stream_handle(stream)))
 
 

@@ -160,22 +160,7 @@ int sta_batch_apply_edits(sta_ctx *x, const int64_t *counts, const sta_edit *edi
         total += counts[i];
     }
     if (total > 0 && !edits) return fail(STA_EINVAL, "edits is NULL");
-    std::vector<sta_edit> g((size_t)total);
-    int64_t e = 0;
-    for (int i = 0; i < c->n_inst; ++i) {
-        const int64_t Ti = c->tet_off[i + 1] - c->tet_off[i], off = c->tet_off[i];
-        for (int64_t j = 0; j < counts[i]; ++j, ++e) {
-            sta_edit E = edits[e];
-            const bool two = E.op == STA_SWAP;
-            if (E.tet < 0 || E.tet >= Ti || (two && (E.tet2 < 0 || E.tet2 >= Ti)))
-                return fail(STA_EINVAL, "instance " + std::to_string(i) + ", edit " +
-                                            std::to_string(j) + ": tet out of the instance's range");
-            E.tet += (int32_t)off;
-            if (two) E.tet2 += (int32_t)off;
-            g[e] = E;
-        }
-    }
-    return sta_apply_edits(x, g.data(), total, stream);
+    return apply_frame(x, edits, total, counts, stream);
 }
 
 }  // extern "C"

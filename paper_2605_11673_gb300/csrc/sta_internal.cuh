@@ -331,6 +331,8 @@ int create_impl(const double *nodes, int64_t n_nodes, const int32_t *tets, int64
                 const double *young, const double *poisson, const sta_options *opt, void *stream,
                 sta_ctx **out);
 void graph_release(Ctx *c);  // sta_graph.cu
+int apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const int64_t *counts,
+                void *stream);  // sta_api.cu
 
 }  // namespace sta
 
