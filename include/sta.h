@@ -240,9 +240,9 @@ int sta_spmv(sta_ctx *ctx, const double *val, const double *x, double *y, void *
 
 /*
  * sta_apply_edits_noalloc -- the same streaming update as sta_apply_edits, for callers that
- * must not allocate (no counterpart in the paper).  sta_apply_edits may grow a pinned host
- * buffer and a device buffer on its first call or when a frame edits more tetrahedra than
- * before; a frame loop that must never stall on cudaMalloc, or a process whose GPU memory is
+ * must not allocate (no counterpart in the paper).  sta_apply_edits may allocate or grow
+ * pinned host buffers and device counters on its first calls or when a frame edits more
+ * tetrahedra than before; a frame loop that must never stall on cudaMalloc, or a process whose GPU memory is
  * held by a framework's caching allocator, cannot allow that.  This variant calls no
  * allocator: its per-call scratch (edited-tet list, touched-unit list, counters) is one
  * fixed device array of 44 x STA_NOALLOC_MAX_EDITED + 32 bytes (about 1.4 MB) that every GPU
@@ -297,8 +297,9 @@ int sta_batch_apply_edits(sta_ctx *ctx, const int64_t *counts, const sta_edit *e
  * list read from the staging block below, grids sized for max_edited), the refold, and the
  * fold of a full rebuild.  Afterwards sta_apply_edits (frames of at most max_edited edited tetrahedra; a
  * swap counts two), sta_refold and sta_full_rebuild replay them with one cudaGraphLaunch each;
- * results are unchanged.  A frame is staged in one of two host-mapped pinned blocks (used in
- * turn) that the captured kernels read directly, so it costs no copy call; the block is
+ * results are unchanged.  Frames of up to some hundred edits are launched without the graph where
+ * that is faster.  A frame is staged in one of two host-mapped pinned blocks (used in
+ * turn) that the kernels read directly, so it costs no copy call; the block is
  * reused once the frame two calls back has finished.  Allocates those blocks and two sets of
  * device counters (each frame's last kernel zeroes the set of the frame after it) and
  * synchronises `stream`.  sta_graph_disable releases them and returns to plain

@@ -70,8 +70,9 @@ static void free_ctx(sta_ctx *x) {
     if (!x) return;
     for (void *p : x->c.allocations) cudaFree(p);
     x->c.allocations.clear();
-    if (x->c.h_frame) cudaFreeHost(x->c.h_frame);
-    if (x->c.d_frame) cudaFree(x->c.d_frame);
+    if (x->c.h_frame[0]) cudaFreeHost(x->c.h_frame[0]);
+    for (cudaEvent_t e : x->c.f_done)
+        if (e) cudaEventDestroy(e);
     if (x->h_mask) cudaFreeHost(x->h_mask);
     if (x->h_count) cudaFreeHost(x->h_count);
     if (x->c.h_count_mapped) cudaFreeHost(x->c.h_count_mapped);
@@ -364,6 +365,39 @@ int sta_apply_edits(sta_ctx *x, const sta_edit *edits, int64_t n_edits, void *st
 
 }  // extern "C"
 
+// Host-mapped frame blocks for `cap` edited tetrahedra each (the old ones are free once the frames
+// that read them are done), and on first use their events and counters.
+static int grow_frames(Ctx *c, int64_t cap, cudaStream_t s) {
+    for (int b = 0; b < 2; ++b) {
+        if (!c->f_done[b])
+            STA_CUDA_TRY(cudaEventCreateWithFlags(&c->f_done[b], cudaEventDisableTiming));
+        if (c->f_pending[b]) {
+            STA_CUDA_TRY(cudaEventSynchronize(c->f_done[b]));
+            c->f_pending[b] = false;
+        }
+    }
+    if (!c->f_cnt) {
+        STA_TRY(dev_alloc(c, &c->f_cnt, 8));
+        STA_CUDA_TRY(cudaMemsetAsync(c->f_cnt, 0, 8 * sizeof(unsigned long long), s));
+    }
+    c->edit_cap = 0;
+    if (c->h_frame[0]) cudaFreeHost(c->h_frame[0]);
+    c->h_frame[0] = c->h_frame[1] = nullptr;
+    const size_t stride = (frame_bytes(cap) + 127) & ~(size_t)127;
+    char *h = nullptr;
+    void *d = nullptr;
+    if (cudaHostAlloc((void **)&h, 2 * stride, cudaHostAllocMapped) != cudaSuccess)
+        return fail(STA_ENOMEM, "pinned edit buffer");
+    c->h_frame[0] = reinterpret_cast<FrameHeader *>(h);
+    c->h_frame[1] = reinterpret_cast<FrameHeader *>(h + stride);
+    if (cudaHostGetDevicePointer(&d, h, 0) != cudaSuccess)
+        return fail(STA_ENOMEM, "pinned edit buffer (host-mapped)");
+    c->m_frame[0] = static_cast<FrameHeader *>(d);
+    c->m_frame[1] = reinterpret_cast<FrameHeader *>(static_cast<char *>(d) + stride);
+    c->edit_cap = cap;
+    return STA_OK;
+}
+
 // What is wrong with an edit of tetrahedra [0, T) shifted by off, in the order of the checks.
 static const char *edit_error(const Ctx *c, const sta_edit &E, int64_t T, int64_t off, uint8_t gen,
                               bool batch) {
@@ -392,19 +426,24 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
     if (n_edits > (INT32_MAX / 32)) return fail(STA_ERANGE, "too many edits in one call");
     cudaStream_t s = (cudaStream_t)stream;
     // edited tetrahedra (a swap edits two): 2 n_edits bounds them; they are counted first only where
-    // that bound is past the capacity of the block at hand.  Staging counts them exactly either way.
+    // that bound is past the capacity of the block at hand, or the frame is a small one.  Staging
+    // counts them exactly either way.
     int64_t m = 2 * n_edits;
-    if (m > (c->graph_on ? c->gcap : c->edit_cap)) {
+    if (m > (c->graph_on ? c->gcap : c->edit_cap) || n_edits <= SMALL_FRAME) {
         m = n_edits;
         for (int64_t e = 0; e < n_edits; ++e) m += edits[e].op == STA_SWAP;
     }
 
     // the frame block to stage into: one of the graph mode's two host-mapped blocks (fixed
-    // capacity), or the context's pinned block (grown on demand)
-    const bool use_graph = c->graph_on && m <= c->gcap;
+    // capacity), or the context's pinned block (grown on demand); a small frame needs neither
+    const bool two_kernels = c->op == STA_OP_ELASTICITY && !c->dyn;
+    const bool small = m > 0 && m <= SMALL_FRAME && two_kernels && c->policy == STA_POLICY_REFOLD;
+    const bool use_graph = c->graph_on && m <= c->gcap && !small;
     FrameHeader *h = nullptr, *d = nullptr;
+    int32_t by_value[SMALL_FRAME];
     int gb = 0;
-    if (use_graph) {  // the staging block last used two frames ago: its kernels are done
+    if (small) {  // staged here: the edits go with the launch
+    } else if (use_graph) {  // the staging block last used two frames ago: its kernels are done
         gb = c->g_next;
         if (c->g_pending[gb]) {
             STA_CUDA_TRY(cudaEventSynchronize(c->g_done[gb]));
@@ -413,33 +452,18 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
         h = c->h_gframe[gb];
         d = c->m_gframe[gb];
     } else {
-        STA_TRY(wait_staging(x));
-        if (m > c->edit_cap || !c->h_frame) {
+        gb = c->f_next;
+        if (m > c->edit_cap || c->edit_cap == 0) {
             // (room for as many swaps: a frame of this size is not counted beforehand again)
             const int64_t cap = m < 1024 ? 1024 : std::max(m + m / 2, 2 * n_edits);
-            if (c->h_frame) cudaFreeHost(c->h_frame);
-            c->h_frame = nullptr;
-            if (c->d_frame) {
-                if (c->last_counters == frame_counters(c->d_frame)) {
-                    STA_CUDA_TRY(cudaMemcpyAsync(c->counters + 1, c->last_counters + 1,
-                                                 3 * sizeof(unsigned long long),
-                                                 cudaMemcpyDeviceToDevice, s));
-                    c->last_counters = c->counters;
-                }
-                cudaFree(c->d_frame);  // implicit device synchronisation
-                c->device_bytes -= (int64_t)frame_bytes(c->edit_cap);
-            }
-            c->d_frame = nullptr;
-            c->edit_cap = 0;
-            if (cudaMallocHost((void **)&c->h_frame, frame_bytes(cap)) != cudaSuccess)
-                return fail(STA_ENOMEM, "pinned edit buffer");
-            if (cudaMalloc((void **)&c->d_frame, frame_bytes(cap)) != cudaSuccess)
-                return fail(STA_ENOMEM, "device edit buffer");
-            c->device_bytes += (int64_t)frame_bytes(cap);
-            c->edit_cap = cap;
+            STA_TRY(grow_frames(c, cap, s));
         }
-        h = c->h_frame;
-        d = c->d_frame;
+        if (c->f_pending[gb]) {  // the block's last frame, two frames ago, has read it
+            STA_CUDA_TRY(cudaEventSynchronize(c->f_done[gb]));
+            c->f_pending[gb] = false;
+        }
+        h = c->h_frame[gb];
+        d = c->m_frame[gb];
     }
 
     // one pass: validate each edit against the host mirror of the mask, stage it and apply it
@@ -450,7 +474,7 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
     }
     const uint8_t gen = c->stamp_gen;
     uint8_t *ts = c->tstate.data();
-    int32_t *stage = frame_edited(h);
+    int32_t *stage = small ? by_value : frame_edited(h);
     int64_t k = 0, e = 0, dact = 0;  // dact: change of the active count
     bool bad = false;
     // (ids compare as unsigned, and an edit's state tests are one condition: the order of the
@@ -510,30 +534,44 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
     }
     c->n_active += dact;
     m = k;
-
-    // header (count, zeroed counters) before the list: in graph mode the captured kernels read
-    // the host-mapped block itself; otherwise block and list go to the device in one copy
-    h->m = m;
-    h->cnt[0] = h->cnt[1] = h->cnt[2] = 0ull;
     c->last_edited = m;
+    if (small) {
+        c->last_counters = c->counters;
+        c->count_on_host = true;
+        return launch_small_frame(c, stage, (int)m, s);
+    }
+
+    // the kernels read the host-mapped block itself: no copy call
+    h->m = m;
     // the fold kernel stores the frame's touched count into the host-mapped word (a frame
     // without edits launches no kernel outside graph mode)
     c->count_on_host = frame_counts_to_host(c) && (use_graph || m > 0);
-    if (use_graph) {  // the captured sequence reads the host-mapped block itself: no copy call
-        c->last_counters = c->d_gcnt + 4 * gb;
-        std::atomic_thread_fence(std::memory_order_seq_cst);  // the block before the launch
-        STA_CUDA_TRY(cudaGraphLaunch(c->g_streams[gb], s));
+    std::atomic_thread_fence(std::memory_order_seq_cst);  // the block before the launch
+    if (use_graph) {
+        unsigned long long *cnt = c->d_gcnt + 4 * gb;
+        c->last_counters = cnt;
+        if (m > 0 && m <= DIRECT_FRAME && two_kernels)
+            STA_TRY(launch_stream_frame(c, frame_edited(d), m, nullptr, cnt, m, s,
+                                        c->d_gcnt + 4 * (gb ^ 1)));
+        else
+            STA_CUDA_TRY(cudaGraphLaunch(c->g_streams[gb], s));
         STA_CUDA_TRY(cudaEventRecord(c->g_done[gb], s));
         c->g_pending[gb] = true;
         c->g_next = gb ^ 1;
         return STA_OK;
     }
-    c->last_counters = frame_counters(d);
-    STA_CUDA_TRY(cudaMemcpyAsync(d, h, frame_bytes(m), cudaMemcpyHostToDevice, s));
-    STA_CUDA_TRY(cudaEventRecord(x->h2d_done, s));
-    x->h2d_pending = true;
-    if (m == 0) return STA_OK;  // the copy has zeroed the frame's counters
-    return launch_stream_frame(c, d, m, s);
+    if (m == 0) {
+        c->last_counters = c->counters;
+        STA_CUDA_TRY(cudaMemsetAsync(c->counters + 1, 0, 3 * sizeof(unsigned long long), s));
+        return STA_OK;
+    }
+    unsigned long long *cnt = c->f_cnt + 4 * gb;
+    c->last_counters = cnt;
+    STA_TRY(launch_stream_frame(c, frame_edited(d), m, nullptr, cnt, m, s, c->f_cnt + 4 * (gb ^ 1)));
+    STA_CUDA_TRY(cudaEventRecord(c->f_done[gb], s));
+    c->f_pending[gb] = true;
+    c->f_next = gb ^ 1;
+    return STA_OK;
 }
 
 extern "C" {

@@ -127,12 +127,16 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
     const int64_t n = 10 * (m_dev ? *m_dev : m);
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n; i0 += stride) {  // CTA-uniform
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x;
+    // (the thread's first edit, while the frame before this one may still run)
+    const uint32_t w1 = first + threadIdx.x < n ? (uint32_t)edited[(first + threadIdx.x) / 10] : 0u;
+    dependency_wait();
+    for (int64_t i0 = first; i0 < n; i0 += stride) {  // CTA-uniform
         const int64_t i = i0 + threadIdx.x;
         bool won = false, diag = false;
         int32_t u = 0;
         if (i < n) {
-            const uint32_t w = (uint32_t)edited[i / 10];
+            const uint32_t w = i0 == first ? w1 : (uint32_t)edited[i / 10];
             const int32_t t = (int32_t)(w & 0x7fffffffu);
             const uint32_t on = w >> 31;
             const int s = (int)(i % 10);
@@ -154,6 +158,7 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
             counters, __popc(ball), 18 * __popc(ball) - 9 * __popc(dball));
         if (won) list[base + __popc(ball & ((1u << lane) - 1u))] = u;
     }
+    launch_dependents();
 }
 
 // Fixed-point frame, phase 2: convert the touched units' entries and release the claims.
@@ -163,6 +168,7 @@ __global__ void k_fx_convert(FoldArgs A, const int32_t *__restrict__ list,
                              const unsigned long long *__restrict__ count,
                              const int16_t *__restrict__ e, const long long *__restrict__ S,
                              UnitState *__restrict__ ustate, unsigned long long *next_count) {
+    dependency_wait();
     if (next_count && blockIdx.x == 0 && threadIdx.x == 0) {
         next_count[0] = 0;
         next_count[2] = 0;
@@ -219,14 +225,12 @@ int launch_fx_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_d
                     int32_t *touched, unsigned long long *counters, cudaStream_t s,
                     unsigned long long *next_cnt) {
     const int threads = FX_CLAIM_THREADS;
-    k_fx_claim<<<grid_cap(c, 10 * cap, threads), threads, 0, s>>>(
-        edited, m, m_dev, c->tunit, c->tpos, c->krun, c->ustate, c->uext, c->mask, touched,
-        counters, c->bmeta, c->fx_q, c->fx_s);
-    k_fx_convert<<<grid_cap(c, (10 * (cap > 0 ? cap : 1) + 2) / 3 * 32, 128), 128, 0, s>>>(
-        fold_args(c), touched, counters + 1, c->fx_e, c->fx_s, c->ustate,
-        next_cnt ? next_cnt + 1 : nullptr);
-    STA_CUDA_TRY(cudaGetLastError());
-    return STA_OK;
+    STA_TRY(launch_overlapped(k_fx_claim, grid_cap(c, 10 * cap, threads), threads, s, edited, m, m_dev,
+                              c->tunit, c->tpos, c->krun, c->ustate, c->uext, c->mask, touched, counters,
+                              c->bmeta, c->fx_q, c->fx_s));
+    return launch_overlapped(k_fx_convert, grid_cap(c, (10 * (cap > 0 ? cap : 1) + 2) / 3 * 32, 128), 128, s,
+                             fold_args(c), touched, counters + 1, c->fx_e, c->fx_s, c->ustate,
+                             next_cnt ? next_cnt + 1 : nullptr);
 }
 
 }  // namespace sta

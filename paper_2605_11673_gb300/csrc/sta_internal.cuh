@@ -86,19 +86,14 @@ __host__ __device__ inline int slot_of(int la, int lb) {  // unordered local pai
 // whole rounds of 32 lanes, the last one nearly -- and the bytes of their runs.
 constexpr int CHUNK_PAIR = 28, CHUNK_DIAG = 16, CHUNK_BYTES = 12 * 1024;
 
-// Frame block: what one streaming frame moves to the device in a single transfer -- the
-// edited count, the frame's counters (zeroed by the host) and the edited list (tet id | new
-// state << 31) right after the header.
+// Frame block: what one streaming frame brings -- the edited count and, right after the header, the
+// edited list (tet id | new state << 31).  A frame's counters: [1] touched units (the FP64 re-fold
+// counts them as diagonal | pair << 32), [3] touched CSR entries.
 struct FrameHeader {
     int64_t m;                     // edited tetrahedra
-    unsigned long long cnt[3];     // touched units, unused, touched CSR entries (the FP64
-                                   // re-fold counts its units as diagonal | pair << 32)
+    int64_t pad[3];
 };
 static_assert(sizeof(FrameHeader) == 32, "frame header layout");
-// counter view with the indices of Ctx::counters: [1] touched units, [3] touched entries
-inline unsigned long long *frame_counters(FrameHeader *f) {
-    return reinterpret_cast<unsigned long long *>(f);
-}
 inline int32_t *frame_edited(FrameHeader *f) { return reinterpret_cast<int32_t *>(f + 1); }
 inline size_t frame_bytes(int64_t m) { return sizeof(FrameHeader) + sizeof(int32_t) * (size_t)m; }
 
@@ -183,8 +178,15 @@ struct Ctx {
     // [0] bad elements, [1] touched units, [2] first bad element, [3] touched CSR entries
     unsigned long long *counters = nullptr;
 
-    // streaming staging: one frame block on the device and its pinned host copy
-    FrameHeader *d_frame = nullptr, *h_frame = nullptr;
+    // streaming staging outside graph mode: two host-mapped pinned blocks used in turn, which the
+    // kernels read where they are, each with an event of its last frame's end; and two sets of
+    // device counters (each frame's last kernel zeroes the other set)
+    // (one allocation, the first block's)
+    FrameHeader *h_frame[2] = {nullptr, nullptr}, *m_frame[2] = {nullptr, nullptr};
+    cudaEvent_t f_done[2] = {nullptr, nullptr};
+    bool f_pending[2] = {false, false};
+    int f_next = 0;
+    unsigned long long *f_cnt = nullptr;  // 2 x 4
     int64_t edit_cap = 0;         // edited tetrahedra a frame block holds
     int64_t last_edited = 0;
     unsigned long long *last_counters = nullptr;  // device counters of the last frame
@@ -265,6 +267,33 @@ inline void ts_set_active(Ctx *c, int64_t t, bool on) {
     c->tstate[t] = (uint8_t)((c->tstate[t] & TS_STAMP) | (on ? TS_ACTIVE : 0));
 }
 
+// Launch of a kernel that may start while the stream's kernel before it still runs: it orders itself
+// with dependency_wait(), before which it reads only what no kernel writes.
+template <typename... P, typename... Q>
+int launch_overlapped(void (*kern)(P...), unsigned grid, unsigned threads, cudaStream_t s, Q... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    STA_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, P(args)...));
+    return STA_OK;
+}
+#ifdef __CUDACC__
+// the CTA has done what the kernel's successor has to wait for but for its end
+__device__ __forceinline__ void launch_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// every kernel before this one in its stream is complete, its writes visible
+__device__ __forceinline__ void dependency_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+#endif
+
 template <typename T> int dev_alloc(Ctx *c, T **p, int64_t count) {
     size_t bytes = sizeof(T) * (size_t)(count > 0 ? count : 1);
     cudaError_t e = cudaMalloc((void **)p, bytes);
@@ -296,15 +325,26 @@ int launch_adjoint(Ctx *c, const double *gval, double *dE, double *dnu, double *
 int launch_spmv(Ctx *c, const double *val, const double *x, double *y, cudaStream_t s);
 int launch_rebuild(Ctx *c, cudaStream_t s);                      // sta_rebuild.cu
 int rebuild_form_of(const Ctx *c);  // the form the next rebuild takes (AUTO resolved)
-int launch_stream_frame(Ctx *c, FrameHeader *frame, int64_t cap, cudaStream_t s);  // sta_stream.cu
+// Frames of at most this many edited tetrahedra take one launch, k_frame_small (elasticity, re-fold
+// policy, without the dynamics' mass update).  Two kernels take 8.3-8.9 us a frame back to back from
+// 16 edits to 122, one cluster 5.8 us for 16, 7.5 for 32, 8.9 for 48, 9.4 for 60 and 14 for 90; a
+// frame that is waited for is at 48 edits 1 us longer, at 32 even.
+constexpr int SMALL_FRAME = 40;
+// In graph mode, frames of at most this many edited tetrahedra are launched kernel by kernel all the
+// same: of such launches a frame's first kernel starts while the last one of the frame before runs,
+// which graph launches don't (600 scattered edits: 12.6 -> 10.4 us a frame, 643 of a crack front:
+// 13.3 -> 12.8).  Larger ones gain or lose with their host time, which a second launch adds 2 us to
+// (2,488 scattered: 19.5 -> 14.7, 2,179 of a crack front: 13.3 -> 14.8): they stay with the graph.
+constexpr int DIRECT_FRAME = 1024;
+int launch_small_frame(Ctx *c, const int32_t *edited, int m, cudaStream_t s);
 // whether a streaming frame of this context stores its touched count into h_count_mapped
 bool frame_counts_to_host(const Ctx *c);
-// the same with the edited list, its count and the counters at separate addresses (the graph
-// mode's host-mapped frames keep their counters in device memory); next_cnt: the counters the
-// frame's last kernel zeroes for the next frame, or nullptr
-int launch_stream_frame(Ctx *c, const int32_t *edited, const int64_t *m_dev,
+// one streaming frame: the edited list, its count (*m_dev, or m) and the counters; cap: edited
+// tetrahedra the grids are sized for; next_cnt: the counters the frame's last kernel zeroes for the
+// next frame, or nullptr
+int launch_stream_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_dev,
                         unsigned long long *cnt, int64_t cap, cudaStream_t s,
-                        unsigned long long *next_cnt);
+                        unsigned long long *next_cnt);  // sta_stream.cu
 int launch_fx_prepare(Ctx *c, cudaStream_t s);                   // sta_fixed.cu
 int launch_fx_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_dev, int64_t cap,
                     int32_t *touched, unsigned long long *counters, cudaStream_t s,

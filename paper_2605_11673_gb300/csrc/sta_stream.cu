@@ -3,6 +3,8 @@
 // exactly those with the rebuild's operands, order and operations.  Also the mask-to-activity
 // pass of a full rebuild with a new mask.  Fold definition and shared device code:
 // sta_fold.cuh.
+#include <cstring>
+
 #include "sta_bulk.cuh"
 #include "sta_claim.cuh"
 #include "sta_fold.cuh"
@@ -31,12 +33,11 @@ constexpr int ENT_PG = 3;      // pair units per warp round (9 lanes each: 27 la
 constexpr int ENT_DEPTH = 24;  // operands of a lane in flight
 constexpr int ENT_WARPS = 4;
 
-// One warp round over units first .. first+NG-1 of one kind (k-th diagonal unit at list[k],
-// k-th pair unit at list[cap - 1 - k]); `col`: the lane's column of the warp's shared buffer.
-template <bool DIAG>
-__device__ __forceinline__ void fold_units(const FoldArgs &A, UnitState *__restrict__ ustate,
-                                           const int32_t *__restrict__ list, int64_t first,
-                                           int64_t n_units, int64_t cap, double *col, int lane,
+// One warp round over units first .. first+NG-1 of one kind of the n_units that unit(k) names;
+// `col`: the lane's column of the warp's shared buffer.
+template <bool DIAG, typename F>
+__device__ __forceinline__ void fold_units(const FoldArgs &A, UnitState *__restrict__ ustate, F unit,
+                                           int64_t first, int64_t n_units, double *col, int lane,
                                            bool has_eps) {
     constexpr int GW = DIAG ? RUN_DIAG : RUN_PAIR;   // lanes (entries) per unit
     constexpr int NG = DIAG ? ENT_DG : ENT_PG;       // units per warp round
@@ -48,10 +49,10 @@ __device__ __forceinline__ void fold_units(const FoldArgs &A, UnitState *__restr
     uint4 st = make_uint4(0, 0, 0, 0);
     int32_t u = 0;
     if (valid) {
-        u = __ldg(list + (DIAG ? k : cap - 1 - k));
+        u = unit(k);
         bm = __ldg(A.bmeta + u);
         if (!DIAG) mir = __ldg(A.bmirror + u);
-        st = *reinterpret_cast<const uint4 *>(ustate + u);
+        st = __ldcg(reinterpret_cast<const uint4 *>(ustate + u));  // (claimed in this very kernel, or before)
     }
     ActiveRuns it(valid, st, bm.w, bm.z + q, GW, A.uext);
     const int n = it.count();
@@ -100,6 +101,7 @@ k_fold_entries(FoldArgs A, UnitState *__restrict__ ustate, const int32_t *__rest
     double *col = stage[threadIdx.x >> 5] + lane;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    dependency_wait();
     const unsigned long long packed = *count;  // final: the claim kernel has ended
     const int64_t nd = (int64_t)(packed & 0xffffffffull), np = (int64_t)(packed >> 32);
     const int64_t gd = (nd + ENT_DG - 1) / ENT_DG, gp = (np + ENT_PG - 1) / ENT_PG;
@@ -115,9 +117,11 @@ k_fold_entries(FoldArgs A, UnitState *__restrict__ ustate, const int32_t *__rest
     const bool has_eps = A.eps != 0.0;
     for (int64_t item = warp; item < gd + gp; item += nwarps) {  // warp-uniform
         if (item < gd)
-            fold_units<true>(A, ustate, list, item * ENT_DG, nd, cap, col, lane, has_eps);
+            fold_units<true>(A, ustate, [&](int64_t k) { return __ldg(list + k); }, item * ENT_DG, nd,
+                             col, lane, has_eps);
         else
-            fold_units<false>(A, ustate, list, (item - gd) * ENT_PG, np, cap, col, lane, has_eps);
+            fold_units<false>(A, ustate, [&](int64_t k) { return __ldg(list + (cap - 1 - k)); },
+                              (item - gd) * ENT_PG, np, col, lane, has_eps);
     }
 }
 
@@ -148,19 +152,34 @@ k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
     const int64_t n = 10 * (m_dev ? *m_dev : m);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < n; i0 += stride) {  // CTA-uniform
+    // the thread's first edit and its unit, which no kernel writes, while the frame before this one
+    // may still run (direct launches of 600 edits back to back: 18.5-20 us -> 10.4, with the edits
+    // read from host memory instead of copied)
+    uint32_t w1 = 0;
+    int32_t u1 = 0, p1 = 0;
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x;
+    if (first + threadIdx.x < n) {
+        const int64_t i = first + threadIdx.x;
+        w1 = (uint32_t)edited[i / 10];
+        const int64_t k = 10 * (int64_t)(w1 & 0x7fffffffu) + i % 10;
+        u1 = __ldg(tunit + k);
+        p1 = __ldg(tpos + k);
+    }
+    dependency_wait();
+    for (int64_t i0 = first; i0 < n; i0 += stride) {  // CTA-uniform
         const int64_t i = i0 + threadIdx.x;
         bool won = false, diag = false;
         int32_t u = 0;
         if (i < n) {
-            const uint32_t w = (uint32_t)edited[i / 10];
+            const bool again = i0 != first;
+            const uint32_t w = again ? (uint32_t)edited[i / 10] : w1;
             const int32_t t = (int32_t)(w & 0x7fffffffu);
             const uint32_t on = w >> 31;
             const int s = (int)(i % 10);
             if (s == 0) mask[t] = (uint8_t)on;
-            u = tunit[10 * (int64_t)t + s];
+            u = again ? __ldg(tunit + 10 * (int64_t)t + s) : u1;
             diag = s < 4;
-            won = claim_unit(ustate, uext, u, tpos[10 * (int64_t)t + s], on != 0u);
+            won = claim_unit(ustate, uext, u, again ? __ldg(tpos + 10 * (int64_t)t + s) : p1, on != 0u);
         }
         const unsigned dball = __ballot_sync(0xffffffffu, won && diag);
         const unsigned pball = __ballot_sync(0xffffffffu, won && !diag);
@@ -183,6 +202,90 @@ k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
         const unsigned below = (1u << lane) - 1u;
         if (won && diag) list[(base & 0xffffffffull) + __popc(dball & below)] = u;
         if (won && !diag) list[cap - 1 - (int64_t)((base >> 32) + __popc(pball & below))] = u;
+    }
+    launch_dependents();
+}
+
+// A small frame in one launch: a cluster of SF_CTAS CTAs claims the units of the frame's edits, which
+// come by value with the launch, and after a cluster barrier each CTA folds the units that its own
+// threads won, listed in its shared memory (diagonal units from the front, pair units from the
+// back).  Such a frame is all latency: launch, drain and dependent round trips (edit count, edits,
+// list, list count), which this kernel does not make or overlaps with the frame before.  Frames of 4
+// edits back to back: 10.9 us as two kernels of a graph, 5.4 here; of 32 edits: 11.3 and 7.4.
+constexpr int SF_CTAS = 8;
+constexpr int SF_WARPS = 7;  // (their operand columns: 42 KB)
+constexpr int SF_THREADS = 32 * SF_WARPS;
+constexpr int SF_ROUNDS = (10 * SMALL_FRAME + SF_CTAS * SF_THREADS - 1) / (SF_CTAS * SF_THREADS);
+
+struct SmallFrame {
+    int32_t m;
+    int32_t edited[SMALL_FRAME];
+};
+
+__global__ void __cluster_dims__(SF_CTAS, 1, 1) __launch_bounds__(SF_THREADS)
+k_frame_small(const __grid_constant__ SmallFrame F, FoldArgs A, const int32_t *__restrict__ tunit,
+              const int32_t *__restrict__ tpos, UnitState *__restrict__ ustate,
+              uint32_t *__restrict__ uext, uint8_t *__restrict__ mask, unsigned long long *counters,
+              unsigned long long *host_count) {
+    constexpr int CAP = SF_ROUNDS * SF_THREADS;
+    __shared__ double stage[SF_WARPS][ENT_DEPTH * 32];
+    __shared__ int32_t won[CAP];
+    __shared__ int n_won[2];        // diagonal, pair units of this CTA
+    __shared__ unsigned touched;    // of the cluster, in CTA 0
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x < 2) n_won[threadIdx.x] = 0;
+    if (threadIdx.x == 2) touched = 0u;
+    // items are dealt to the CTAs in turn, so that each gets its share of a short frame; their edits
+    // and units, which no kernel writes, are read while the frame before may still run
+    uint32_t w[SF_ROUNDS];
+    int32_t u[SF_ROUNDS], pos[SF_ROUNDS];
+#pragma unroll
+    for (int r = 0; r < SF_ROUNDS; ++r) {
+        const int i = (int)((r * SF_THREADS + threadIdx.x) * SF_CTAS + blockIdx.x);
+        if (i < 10 * F.m) {
+            w[r] = (uint32_t)F.edited[i / 10];
+            const int64_t k = 10 * (int64_t)(w[r] & 0x7fffffffu) + i % 10;
+            u[r] = __ldg(tunit + k);
+            pos[r] = __ldg(tpos + k);
+        }
+    }
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    dependency_wait();
+#pragma unroll
+    for (int r = 0; r < SF_ROUNDS; ++r) {
+        const int i = (int)((r * SF_THREADS + threadIdx.x) * SF_CTAS + blockIdx.x);
+        if (i < 10 * F.m) {
+            const int s = i % 10;
+            if (s == 0) mask[w[r] & 0x7fffffffu] = (uint8_t)(w[r] >> 31);
+            if (claim_unit(ustate, uext, u[r], pos[r], (w[r] >> 31) != 0u)) {
+                if (s < 4) won[atomicAdd(&n_won[0], 1)] = u[r];
+                else won[CAP - 1 - atomicAdd(&n_won[1], 1)] = u[r];
+            }
+        }
+    }
+    __syncthreads();
+    const int nd = n_won[0], np = n_won[1];
+    if (threadIdx.x == 0) {  // the touched entries of the frame, summed in CTA 0
+        unsigned a;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_addr(&touched)));
+        asm volatile("red.relaxed.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(a),
+                     "r"((unsigned)(9 * nd + 18 * np)) : "memory");
+    }
+    // every claim and activity change of the frame is done and visible
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        counters[3] = touched;
+        *host_count = touched;
+    }
+    const bool has_eps = A.eps != 0.0;
+    double *col = stage[wid] + lane;
+    const int gd = (nd + ENT_DG - 1) / ENT_DG, gp = (np + ENT_PG - 1) / ENT_PG;
+    for (int item = wid; item < gd + gp; item += SF_WARPS) {  // warp-uniform
+        if (item < gd)
+            fold_units<true>(A, ustate, [&](int64_t k) { return won[k]; }, item * ENT_DG, nd, col, lane, has_eps);
+        else
+            fold_units<false>(A, ustate, [&](int64_t k) { return won[CAP - 1 - k]; }, (item - gd) * ENT_PG, np,
+                              col, lane, has_eps);
     }
 }
 
@@ -243,10 +346,8 @@ int launch_fold_list(Ctx *c, const int32_t *list, int64_t cap, unsigned long lon
     // resident CTAs
     const int grid = persistent_grid(c, (const void *)k_fold_entries, threads,
                                      (max_items + ENT_PG - 1) / ENT_PG * 32);
-    k_fold_entries<<<grid, threads, 0, s>>>(fold_args(c), c->ustate, list, count, cap, host_count,
-                                            next_count);
-    STA_CUDA_TRY(cudaGetLastError());
-    return STA_OK;
+    return launch_overlapped(k_fold_entries, (unsigned)grid, threads, s, fold_args(c), c->ustate, list,
+                             count, cap, host_count, next_count);
 }
 
 int launch_mask_bits(Ctx *c, cudaStream_t s) {
@@ -267,39 +368,41 @@ int launch_values(Ctx *c, cudaStream_t s) {
     return launch_dyn_mass_all(c, s);  // the lumped mass, when the dynamics are set up
 }
 
-// One streaming frame: claim kernel, then the fold of the touched units.  `frame` is a device
-// frame block (FrameHeader + edited list) already holding the frame; the count is read from
-// it, grids are sized for `cap` edited tetrahedra (so the sequence can be captured once and
-// replayed for any frame up to `cap`).  `next_cnt`: the counters of the next frame, which the
-// frame's last kernel zeroes (graph mode), or nullptr.
-int launch_stream_frame(Ctx *c, const int32_t *edited, const int64_t *m_dev,
+// One streaming frame: claim kernel, then the fold of the touched units.  The edited count is *m_dev
+// if given (a sequence captured once and replayed for any frame up to `cap`, for which the grids are
+// sized), else m.  `next_cnt`: the counters of the next frame, which the frame's last kernel zeroes,
+// or nullptr.
+int launch_stream_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_dev,
                         unsigned long long *cnt, int64_t cap, cudaStream_t s,
                         unsigned long long *next_cnt) {
     if (c->op == STA_OP_PROXY)
-        return launch_proxy_frame(c, edited, 0, m_dev, cap, c->plist, cnt, s, next_cnt);
+        return launch_proxy_frame(c, edited, m, m_dev, cap, c->plist, cnt, s, next_cnt);
     if (c->policy == STA_POLICY_FIXED) {
-        STA_TRY(launch_fx_frame(c, edited, 0, m_dev, cap, c->touched, cnt, s, next_cnt));
-        return launch_dyn_mass_edited(c, edited, 0, m_dev, cap, s);
+        STA_TRY(launch_fx_frame(c, edited, m, m_dev, cap, c->touched, cnt, s, next_cnt));
+        return launch_dyn_mass_edited(c, edited, m, m_dev, cap, s);
     }
     const int threads = CLAIM_THREADS;
     int64_t g = (10 * cap + threads - 1) / threads;
     const int64_t gmax = (int64_t)c->num_sms * 16;
     g = g < 1 ? 1 : (g > gmax ? gmax : g);
-    k_stream_claim<<<(unsigned)g, threads, 0, s>>>(edited, 0, m_dev, c->tunit, c->tpos, c->ustate,
-                                                   c->uext, c->mask, c->touched, c->nunits, cnt);
-    STA_CUDA_TRY(cudaGetLastError());
+    STA_TRY(launch_overlapped(k_stream_claim, (unsigned)g, threads, s, edited, m, m_dev, c->tunit,
+                              c->tpos, c->ustate, c->uext, c->mask, c->touched, c->nunits, cnt));
     STA_TRY(launch_fold_list(c, c->touched, c->nunits, cnt + 1, 10 * (cap > 0 ? cap : 1), s,
                              c->d_count_mapped, next_cnt ? next_cnt + 1 : nullptr));
-    return launch_dyn_mass_edited(c, edited, 0, m_dev, cap, s);
+    return launch_dyn_mass_edited(c, edited, m, m_dev, cap, s);
+}
+
+// A frame of m <= SMALL_FRAME edited tetrahedra (tet id | new state << 31, host memory) in one launch.
+int launch_small_frame(Ctx *c, const int32_t *edited, int m, cudaStream_t s) {
+    SmallFrame F;
+    F.m = m;
+    std::memcpy(F.edited, edited, sizeof(int32_t) * m);
+    return launch_overlapped(k_frame_small, SF_CTAS, SF_THREADS, s, F, fold_args(c), c->tunit, c->tpos,
+                             c->ustate, c->uext, c->mask, c->counters, c->d_count_mapped);
 }
 
 bool frame_counts_to_host(const Ctx *c) {
     return c->op == STA_OP_ELASTICITY && c->policy == STA_POLICY_REFOLD && c->d_count_mapped;
-}
-
-int launch_stream_frame(Ctx *c, FrameHeader *frame, int64_t cap, cudaStream_t s) {
-    return launch_stream_frame(c, frame_edited(frame), &frame->m, frame_counters(frame), cap, s,
-                               nullptr);
 }
 
 // Streaming update with caller-chosen scratch (the allocation-free entry point): the same two
@@ -317,10 +420,11 @@ int launch_stream_scratch(Ctx *c, int64_t m, const int32_t *d_edited, int32_t *t
         const int threads = CLAIM_THREADS;
         const int64_t g = (10 * m + threads - 1) / threads;
         // the touched list holds 10 m units (at most 10 per edited tet)
-        k_stream_claim<<<(unsigned)g, threads, 0, s>>>(d_edited, m, nullptr, c->tunit, c->tpos,
-                                                       c->ustate, c->uext, c->mask, touched, 10 * m,
-                                                       counters);
-        STA_CUDA_TRY(cudaGetLastError());
+        // (the claim reads d_edited before its dependency_wait: it was copied there before the
+        // memset above, and a kernel that follows a memset starts when that is done)
+        STA_TRY(launch_overlapped(k_stream_claim, (unsigned)g, threads, s, d_edited, m, (const int64_t *)nullptr,
+                                  c->tunit, c->tpos, c->ustate, c->uext, c->mask, touched, 10 * m,
+                                  counters));
         STA_TRY(launch_fold_list(c, touched, 10 * m, counters + 1, 10 * m, s, nullptr, nullptr));
     }
     if (m > 0) STA_TRY(launch_dyn_mass_edited(c, d_edited, m, nullptr, m, s));
