@@ -225,10 +225,10 @@ int launch_fx_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_d
                     int32_t *touched, unsigned long long *counters, cudaStream_t s,
                     unsigned long long *next_cnt) {
     const int threads = FX_CLAIM_THREADS;
-    STA_TRY(launch_overlapped(k_fx_claim, grid_cap(c, 10 * cap, threads), threads, s, edited, m, m_dev,
+    STA_TRY(launch_overlapped(k_fx_claim, grid_cap(c, 10 * cap, threads), threads, 0, s, edited, m, m_dev,
                               c->tunit, c->tpos, c->krun, c->ustate, c->uext, c->mask, touched, counters,
                               c->bmeta, c->fx_q, c->fx_s));
-    return launch_overlapped(k_fx_convert, grid_cap(c, (10 * (cap > 0 ? cap : 1) + 2) / 3 * 32, 128), 128, s,
+    return launch_overlapped(k_fx_convert, grid_cap(c, (10 * (cap > 0 ? cap : 1) + 2) / 3 * 32, 128), 128, 0, s,
                              fold_args(c), touched, counters + 1, c->fx_e, c->fx_s, c->ustate,
                              next_cnt ? next_cnt + 1 : nullptr);
 }

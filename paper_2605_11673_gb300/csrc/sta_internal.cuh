@@ -270,10 +270,12 @@ inline void ts_set_active(Ctx *c, int64_t t, bool on) {
 // Launch of a kernel that may start while the stream's kernel before it still runs: it orders itself
 // with dependency_wait(), before which it reads only what no kernel writes.
 template <typename... P, typename... Q>
-int launch_overlapped(void (*kern)(P...), unsigned grid, unsigned threads, cudaStream_t s, Q... args) {
+int launch_overlapped(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
+                      Q... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -246,6 +246,7 @@ k_fold_flat(FoldArgs A, const int2 *__restrict__ chunks, int32_t nchunks,
         bar_init_fence();
     }
     __syncthreads();
+    dependency_wait();
 
     if (wid == FOLD_CONS) {  // producer
         const int32_t G = (int32_t)gridDim.x, b = (int32_t)blockIdx.x;
@@ -408,6 +409,8 @@ __global__ void k_zero_fill(const int2 *__restrict__ chunks, int32_t nchunks,
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
+    launch_dependents();
+    dependency_wait();
     for (int64_t c = tid >> 5; c < nchunks; c += nthreads >> 5) {  // warp-uniform
         const int2 r = __ldg(chunks + c);
         bool on = eps && r.y >> 8;
@@ -469,6 +472,7 @@ __global__ void __launch_bounds__(32 * FOLD_CONS)
 k_fold_small(FoldArgs A, const int2 *__restrict__ chunks, FxArgs X) {
     const int2 rec = __ldg(chunks + blockIdx.x);
     const int r = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    dependency_wait();
     if (rec.y >> 8) small_round<FX, true>(A, X, rec, r, lane);
     else small_round<FX, false>(A, X, rec, r, lane);
 }
@@ -478,26 +482,22 @@ int launch_fold(Ctx *c, cudaStream_t s) {
     const FxArgs X{c->fx_q, c->fx_e, c->fx_s};
     const FoldArgs A = fold_args(c);
     if (c->nchunks <= (int64_t)(FX || ZF ? SMALL_CHUNKS_LONG : SMALL_CHUNKS) * FOLD_CTAS * c->num_sms) {
-        k_fold_small<FX><<<(unsigned)c->nchunks, 32 * FOLD_CONS, 0, s>>>(A, c->chunks, X);
-        STA_CUDA_TRY(cudaGetLastError());
-        return STA_OK;
+        return launch_overlapped(k_fold_small<FX>, (unsigned)c->nchunks, 32 * FOLD_CONS, 0, s, A,
+                                 (const int2 *)c->chunks, X);
     }
-    if (ZF) {
-        k_zero_fill<<<c->num_sms * 8, 256, 0, s>>>(c->chunks, (int32_t)c->nchunks, c->ustate,
-                                                   c->eps != 0.0, c->cflag, c->val,
-                                                   FX ? c->fx_s : nullptr, c->nnz);
-        STA_CUDA_TRY(cudaGetLastError());
-    }
+    if (ZF)
+        STA_TRY(launch_overlapped(k_zero_fill, c->num_sms * 8, 256, 0, s, (const int2 *)c->chunks,
+                                  (int32_t)c->nchunks, (const UnitState *)c->ustate, c->eps != 0.0, c->cflag,
+                                  c->val, FX ? c->fx_s : nullptr, c->nnz));
     STA_CUDA_TRY(cudaFuncSetAttribute(k_fold_flat<FX, ZF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)sizeof(FoldShared)));
     int per_sm = c->blocks_per_sm;
     if (per_sm <= 0 || per_sm > FOLD_CTAS) per_sm = FOLD_CTAS;
     const int64_t cap = (int64_t)per_sm * c->num_sms;
     const unsigned grid = (unsigned)(c->nchunks < cap ? c->nchunks : cap);
-    k_fold_flat<FX, ZF><<<grid, FOLD_THREADS, sizeof(FoldShared), s>>>(A, c->chunks, (int32_t)c->nchunks,
-                                                                       c->cflag, X, c->d_fault);
-    STA_CUDA_TRY(cudaGetLastError());
-    return STA_OK;
+    return launch_overlapped(k_fold_flat<FX, ZF>, grid, FOLD_THREADS, sizeof(FoldShared), s, A,
+                             (const int2 *)c->chunks, (int32_t)c->nchunks, (const uint8_t *)c->cflag, X,
+                             c->d_fault);
 }
 
 }  // namespace

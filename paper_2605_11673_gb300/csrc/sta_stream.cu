@@ -289,38 +289,66 @@ k_frame_small(const __grid_constant__ SmallFrame F, FoldArgs A, const int32_t *_
     }
 }
 
-// Activity bits of every unit from the mask (full rebuild with a new mask).  A lane per unit, four
-// contributors in flight (neighbouring units have lists of equal length, and their lists are
-// neighbours in memory); whole state words are written back.
-__global__ void __launch_bounds__(256)
+// Activity bits of every unit from the mask (full rebuild with a new mask).  A CTA takes as many
+// consecutive units as it has threads; their contributors stand side by side, so it reads them
+// coalesced, BITS_WINDOW at a time, keeps one bit each in shared memory (a ballot per warp load), and
+// then every thread cuts its unit's words out of the bits.  Bound by the gathers of the mask and
+// their latency; a lane per unit over its own list needed a request per lane for the list as well.
+// Pre-fractured block of 577,000 tetrahedra (5.8 M contributors, 0.9 M units): 33 -> 17 us.
+constexpr int BITS_THREADS = 256, BITS_LOADS = 8;
+constexpr int BITS_WINDOW = BITS_THREADS * BITS_LOADS;
+
+__global__ void __launch_bounds__(BITS_THREADS, 8)
 k_mask_bits(int64_t nunits, const int32_t *__restrict__ uc0, const int32_t *__restrict__ ctet,
             const uint8_t *__restrict__ mask, uint4 *__restrict__ ustate,
             uint32_t *__restrict__ uext) {
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < nunits;
-         u += (int64_t)gridDim.x * blockDim.x) {
-        const int32_t c0 = __ldg(uc0 + u), cnt = __ldg(uc0 + u + 1) - c0;
-        uint4 st = ustate[u];
-        uint32_t word = 0;
-        st.x = st.z = 0u;
-        for (int32_t j = 0; j < cnt; j += 4) {
-            int32_t t[4];
-            uint32_t on[4];
+    __shared__ uint32_t bits[BITS_WINDOW / 32 + 1];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t u0 = (int64_t)blockIdx.x * BITS_THREADS, u = u0 + threadIdx.x;
+    const bool valid = u < nunits;
+    const int32_t lo = __ldg(uc0 + u0);
+    const int32_t hi = __ldg(uc0 + (u0 + BITS_THREADS < nunits ? u0 + BITS_THREADS : nunits));
+    const int32_t b = valid ? __ldg(uc0 + u) : hi, e = valid ? __ldg(uc0 + u + 1) : hi;
+    launch_dependents();  // (the fold's CTAs set up while the last of these run)
+    dependency_wait();
+    uint4 st = valid ? ustate[u] : make_uint4(0, 0, 0, 0);
+    st.x = st.z = 0u;
+    uint32_t word = 0;
+    int32_t j = b;  // the unit's next contributor
+    for (int32_t w0 = lo; w0 < hi; w0 += BITS_WINDOW) {
+        int32_t t[BITS_LOADS];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) t[k] = j + k < cnt ? __ldg(ctet + c0 + j + k) : -1;
+        for (int k = 0; k < BITS_LOADS; ++k) {
+            const int32_t i = w0 + k * BITS_THREADS + (int)threadIdx.x;
+            t[k] = i < hi ? __ldg(ctet + i) : -1;
+        }
+        bool on[BITS_LOADS];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) on[k] = t[k] >= 0 && __ldg(mask + t[k]) ? 1u : 0u;
+        for (int k = 0; k < BITS_LOADS; ++k) on[k] = t[k] >= 0 && __ldg(mask + t[k]);
 #pragma unroll
-            for (int k = 0; k < 4; ++k) word |= on[k] << ((j + k) & 31);
-            if (((j + 4) & 31) == 0 || j + 4 >= cnt) {  // a word of 32 is complete
-                const int w = j >> 5;
+        for (int k = 0; k < BITS_LOADS; ++k) {
+            const uint32_t m = __ballot_sync(0xffffffffu, on[k]);
+            if (lane == 0) bits[k * (BITS_THREADS / 32) + wid] = m;
+        }
+        __syncthreads();
+        const int32_t end = e < w0 + BITS_WINDOW ? e : w0 + BITS_WINDOW;
+        while (j < end) {  // the rest of one of the unit's words, as far as it is in the window
+            const int at = (j - b) & 31, f = j - w0;
+            const int n = 32 - at < end - j ? 32 - at : end - j;
+            const uint32_t v = __funnelshift_r(bits[f >> 5], bits[(f >> 5) + 1], f & 31);
+            word |= (n == 32 ? v : v & ((1u << n) - 1u)) << at;
+            j += n;
+            if (at + n == 32 || j == e) {
+                const int w = (j - 1 - b) >> 5;
                 if (w == 0) st.x = word;
                 else if (w == 1) st.z = word;
                 else uext[st.w + w - 2] = word;
                 word = 0;
             }
         }
-        ustate[u] = st;
+        __syncthreads();
     }
+    if (valid) ustate[u] = st;
 }
 
 }  // namespace
@@ -346,19 +374,15 @@ int launch_fold_list(Ctx *c, const int32_t *list, int64_t cap, unsigned long lon
     // resident CTAs
     const int grid = persistent_grid(c, (const void *)k_fold_entries, threads,
                                      (max_items + ENT_PG - 1) / ENT_PG * 32);
-    return launch_overlapped(k_fold_entries, (unsigned)grid, threads, s, fold_args(c), c->ustate, list,
+    return launch_overlapped(k_fold_entries, (unsigned)grid, threads, 0, s, fold_args(c), c->ustate, list,
                              count, cap, host_count, next_count);
 }
 
 int launch_mask_bits(Ctx *c, cudaStream_t s) {
     if (c->T == 0 || c->op == STA_OP_PROXY) return STA_OK;  // the proxy reads the mask itself
-    int64_t grid = (c->nunits + 255) / 256;
-    const int64_t cap = (int64_t)c->num_sms * 8;
-    if (grid > cap) grid = cap;
-    k_mask_bits<<<(unsigned)grid, 256, 0, s>>>(c->nunits, c->uc0, c->ctet, c->mask,
-                                             reinterpret_cast<uint4 *>(c->ustate), c->uext);
-    STA_CUDA_TRY(cudaGetLastError());
-    return STA_OK;
+    const int64_t grid = (c->nunits + BITS_THREADS - 1) / BITS_THREADS;
+    return launch_overlapped(k_mask_bits, (unsigned)grid, BITS_THREADS, 0, s, c->nunits, c->uc0, c->ctet,
+                             c->mask, reinterpret_cast<uint4 *>(c->ustate), c->uext);
 }
 
 // Every value from the current mask: the operator's full rebuild.
@@ -385,7 +409,7 @@ int launch_stream_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t 
     int64_t g = (10 * cap + threads - 1) / threads;
     const int64_t gmax = (int64_t)c->num_sms * 16;
     g = g < 1 ? 1 : (g > gmax ? gmax : g);
-    STA_TRY(launch_overlapped(k_stream_claim, (unsigned)g, threads, s, edited, m, m_dev, c->tunit,
+    STA_TRY(launch_overlapped(k_stream_claim, (unsigned)g, threads, 0, s, edited, m, m_dev, c->tunit,
                               c->tpos, c->ustate, c->uext, c->mask, c->touched, c->nunits, cnt));
     STA_TRY(launch_fold_list(c, c->touched, c->nunits, cnt + 1, 10 * (cap > 0 ? cap : 1), s,
                              c->d_count_mapped, next_cnt ? next_cnt + 1 : nullptr));
@@ -397,7 +421,7 @@ int launch_small_frame(Ctx *c, const int32_t *edited, int m, cudaStream_t s) {
     SmallFrame F;
     F.m = m;
     std::memcpy(F.edited, edited, sizeof(int32_t) * m);
-    return launch_overlapped(k_frame_small, SF_CTAS, SF_THREADS, s, F, fold_args(c), c->tunit, c->tpos,
+    return launch_overlapped(k_frame_small, SF_CTAS, SF_THREADS, 0, s, F, fold_args(c), c->tunit, c->tpos,
                              c->ustate, c->uext, c->mask, c->counters, c->d_count_mapped);
 }
 
@@ -422,7 +446,7 @@ int launch_stream_scratch(Ctx *c, int64_t m, const int32_t *d_edited, int32_t *t
         // the touched list holds 10 m units (at most 10 per edited tet)
         // (the claim reads d_edited before its dependency_wait: it was copied there before the
         // memset above, and a kernel that follows a memset starts when that is done)
-        STA_TRY(launch_overlapped(k_stream_claim, (unsigned)g, threads, s, d_edited, m, (const int64_t *)nullptr,
+        STA_TRY(launch_overlapped(k_stream_claim, (unsigned)g, threads, 0, s, d_edited, m, (const int64_t *)nullptr,
                                   c->tunit, c->tpos, c->ustate, c->uext, c->mask, touched, 10 * m,
                                   counters));
         STA_TRY(launch_fold_list(c, touched, 10 * m, counters + 1, 10 * m, s, nullptr, nullptr));

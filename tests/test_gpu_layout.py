@@ -85,3 +85,12 @@ def test_sizes_and_activity_patterns(sta, orc, kind, size, eps):
              (rng.uniform(size=T) < 0.01).astype(np.uint8)]
     _check(sta, orc, X, tets, W.lognormal_E(rng, T), np.full(T, 0.3), masks, eps,
            (sta.STA_REBUILD_FUSED, sta.STA_REBUILD_ZERO_FILL))
+
+
+@pytest.mark.parametrize("K", [2047, 2048, 2049, 4100])
+def test_units_longer_than_a_pass_over_the_mask(sta, orc, K):
+    """Activity words of one unit formed from several windows of its contributors."""
+    wl = W.edge_fan(K=K)
+    rng = np.random.default_rng(K)
+    masks = [(rng.uniform(size=K) < 0.5).astype(np.uint8), np.ones(K, np.uint8)]
+    _check(sta, orc, wl.X, wl.tets, wl.E, wl.nu, masks, 0.0, (sta.STA_REBUILD_FUSED,))
