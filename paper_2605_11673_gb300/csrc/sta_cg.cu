@@ -24,18 +24,21 @@
 // it fits (a 27,783-DOF block, the proxy operator of 113,000 nodes); only z, which the products
 // gather, goes through global memory.
 //
-// Grid-wide sums.  A CTA adds its threads' partial sums in a fixed order and stores the sum with
-// the sum's number as one 16-byte word; one warp of every CTA then reads all CTAs' words until
+// Grid-wide sums.  A CTA adds its threads' partial sums in a fixed order and stores the sum with the
+// iteration's number as one 16-byte word; one warp of every CTA then reads all CTAs' words until
 // each carries that number and adds them in CTA order.  So every CTA has the same bits without a
-// second exchange, and the sum is the barrier as well.  Two sets of words alternate: a CTA stores
-// sum k + 2 only after it has read every CTA's sum k + 1, so nobody still waits for sum k.  The
-// waits are bounded (CG_SPINS); a CTA whose wait runs out marks the solve as failed and leaves,
-// and so do, one after another, all others.
+// second exchange, and the sum is the barrier as well.  An iteration has three exchanges: p.q,
+// the new z (a word without a sum: the stores are visible), and r.z with r.r, which only the end
+// of the next product needs: warps of their own add and exchange them while the others already
+// multiply.  Each has its own words; a CTA can store the next word of an exchange only after an
+// exchange that every CTA enters when it has read the last one.  The waits are bounded (CG_SPINS);
+// a CTA whose wait runs out marks the solve as failed and leaves, and so do, one after another,
+// all others.
 //
-// Measured (GB300, time of an iteration with two launches -> now): 27,783-DOF block 29 -> 11.4 us,
-// 341,000-DOF pre-fractured block 62 -> 48 us (FP64 floor of its product 24 us), scalar operator of
-// 113,800 rows 34 -> 13 us.  Of the small block's 11.4 us the product takes 3 us, the two grid-wide
-// sums 3 and 3.8 us (the second one publishes z), the updates 0.6 us.
+// Measured (GB300, time of an iteration with two launches -> now): 27,783-DOF block 29 -> 10.3 us,
+// 341,000-DOF pre-fractured block 62 -> 41 us (FP64 floor of its product 24 us), scalar operator of
+// 113,800 rows 34 -> 12 us.  With both sums on the path of the iteration (11.4, 48 and 13 us), the
+// small block's product took 3 us, the sums 3 and 3.8 us, the updates 0.6 us.
 #include <algorithm>
 #include <cmath>
 #include <vector>
@@ -45,11 +48,16 @@
 namespace sta {
 namespace {
 
-constexpr int CG_WARPS = 16;             // warps of a CTA at most (one CTA per SM)
-constexpr int CG_MAX_GRID = 160;         // CTAs at most: 5 words a lane in a grid-wide sum
+// Working warps of a CTA at most (one CTA per SM).  A full SM has 24 slices: two for each of 12 warps,
+// three for each of 8, one or two for 15.  Steps of the 341,000-DOF block with 8, 12 and 15: 1.25, 1.15
+// and 1.19 ms; the scalar operator's frame 4.2, 4.1 and 4.3 ms.
+constexpr int CG_WARPS = 12;
+constexpr int CG_SUMS = 2;               // warps for the sums (a third one would take the working
+                                         // warps registers: 16,384 for the warps of a quadrant)
+constexpr int CG_MAX_GRID = 160;         // CTAs at most: 5 words a lane in an exchange
 constexpr int CG_CHECK = 8;              // iterations between two looks at stagnation
 constexpr unsigned CG_SPINS = 1u << 22;  // polls of a wait (seconds)
-constexpr size_t CG_SMEM = 208 * 1024;   // dynamic shared memory at most (CgShared: 18 KB)
+constexpr size_t CG_SMEM = 216 * 1024;   // dynamic shared memory at most (CgShared: 9 KB)
 
 // One CTA's word of a grid-wide sum, alone in its 128-byte line: packed 16 bytes apart, the words
 // took 5,500 cycles a sum instead of 3,600 (152 CTAs polling the same few lines).
@@ -80,10 +88,11 @@ struct CgArgs {
     const int32_t *col;    // per step and lane: column node
     const double *val;     // per step: B * B values of 32 lanes each
     const double *b, *dinv;
-    double *x, *z;
+    double *x, *z;         // z: a node's B values at z_stride<B>
     double *vec;           // 5 vectors in slice order when shared memory does not hold them
     int64_t vec_len;       // of one of them
-    CgSlot *slots;         // 2 sets x 3 sums x CG_MAX_GRID
+    bool plan_shared;
+    CgSlot *slots;         // CG_WORDS exchanges x CG_MAX_GRID
     unsigned long long epoch;
     CgResult *out;         // host-mapped
     double tol2;
@@ -95,89 +104,106 @@ struct CgArgs {
     double h;
 };
 
+// The exchanges: r.z, r.r and (once) b.b, p.q, z.
+enum { W_RZ, W_RR, W_BB, W_PQ, W_Z, CG_WORDS };
+
+// Nodes of three values are gathered as one aligned word of four: the three loads of a 24-byte
+// record cost the L1 cache nearly three times as much.
+template <int B> constexpr int z_stride = B == 3 ? 4 : 1;
+
 // Shared scratch of the sums.
 struct CgShared {
     double part[3][CG_WARPS * 32];
-    double sum[3], ratio;
-    int failed[3];
+    double sum[3], beta;  // of the sum warps
+    double pq, alpha;
+    int late[3], failed, quit;
 };
 
-// Sums v[0..NV) over the grid: NV partial sums of every thread in, the NV sums (same bits in every
-// thread of the grid) out; warp k sums value k.  False when a wait ran out.  ratio: num / v[0], or
-// v[0] / num with `inverse` -- an FP64 division is a dozen dependent FP64 instructions, formed by
-// one warp instead of all 24.  FENCE: what the CTA stored before the call is visible to every CTA
-// after it; without it the sum only orders loads before it ahead of stores after it (the loaded
-// values went into the sum).
-template <int NV, bool FENCE>
-__device__ __forceinline__ bool grid_sum(double (&v)[NV], double &ratio, double num, bool inverse,
-                                         const CgArgs &a, unsigned long long epoch, CgShared &sh) {
-    constexpr unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, n = blockDim.x;
-    // through shared memory: a shuffle tree in every warp would cost 5 FP64 instructions per warp
-    // and value
+// Barriers between a CTA's warps: the working warps among themselves, partial sums to the sum
+// warps, sums to the working warps.
+enum { BAR_WORK = 1, BAR_PARTS, BAR_SUMS };
+__device__ __forceinline__ void named_sync(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void named_arrive(int id, int threads) {
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+__device__ __forceinline__ double warp_sum(double t) {
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
+}
+
+// The sum of n (a multiple of 32) partial sums, in every lane.  Through shared memory: a shuffle
+// tree in every warp would cost 5 FP64 instructions per warp and value.
+__device__ __forceinline__ double sum_parts(const double *p, int n, int lane) {
+    double t0 = p[lane], t1 = 0.0, t2 = 0.0, t3 = 0.0;
+    int i = 32 + lane;
+    for (; i + 96 < n; i += 128) {
+        t0 += p[i];
+        t1 += p[i + 32];
+        t2 += p[i + 64];
+        t3 += p[i + 96];
+    }
+    for (; i < n; i += 32) t0 += p[i];
+    return warp_sum((t0 + t1) + (t2 + t3));
+}
+
+// Waits until every CTA's word of one exchange carries `epoch`.  Returns the lane's part of their
+// sum; `late` (same in all lanes): the wait ran out.
+__device__ __forceinline__ double wait_words(const CgSlot *set, unsigned long long epoch, int lane, bool &late) {
+    constexpr int PER = CG_MAX_GRID / 32;
+    double got[PER];
+    unsigned need = 0;  // words still to come
 #pragma unroll
-    for (int k = 0; k < NV; ++k) sh.part[k][threadIdx.x] = v[k];
-    __syncthreads();
-    if (wid < NV) {
-        const double *p = sh.part[wid];
-        double t0 = p[lane], t1 = 0.0, t2 = 0.0, t3 = 0.0;
-        int i = 32 + lane;
-        for (; i + 96 < n; i += 128) {
-            t0 += p[i];
-            t1 += p[i + 32];
-            t2 += p[i + 64];
-            t3 += p[i + 96];
-        }
-        for (; i < n; i += 32) t0 += p[i];
-        double t = (t0 + t1) + (t2 + t3);
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
-        CgSlot *set = a.slots + ((epoch & 1) * 3 + wid) * CG_MAX_GRID;
-        if (lane == 0) {
-            if constexpr (FENCE) __threadfence();  // the CTA's z
-            st_slot(set + blockIdx.x, t, epoch);
-        }
-        constexpr int PER = CG_MAX_GRID / 32;
-        double got[PER];
-        unsigned need = 0;  // words still to come
+    for (int i = 0; i < PER; ++i) {
+        got[i] = 0.0;
+        if (lane + 32 * i < (int)gridDim.x) need |= 1u << i;
+    }
+    for (unsigned spin = 0; need && spin < CG_SPINS; ++spin) {
+        double w[PER];
+        unsigned long long e[PER];
 #pragma unroll
         for (int i = 0; i < PER; ++i) {
-            got[i] = 0.0;
-            if (lane + 32 * i < (int)gridDim.x) need |= 1u << i;
+            e[i] = 0;
+            if (need >> i & 1) ld_slot(set + lane + 32 * i, w[i], e[i]);
         }
-        for (unsigned spin = 0; need && spin < CG_SPINS; ++spin) {
-            double w[PER];
-            unsigned long long e[PER];
 #pragma unroll
-            for (int i = 0; i < PER; ++i) {
-                e[i] = 0;
-                if (need >> i & 1) ld_slot(set + lane + 32 * i, w[i], e[i]);
+        for (int i = 0; i < PER; ++i)
+            if ((need >> i & 1) && e[i] == epoch) {
+                got[i] = w[i];
+                need &= ~(1u << i);
             }
-#pragma unroll
-            for (int i = 0; i < PER; ++i)
-                if ((need >> i & 1) && e[i] == epoch) {
-                    got[i] = w[i];
-                    need &= ~(1u << i);
-                }
-        }
-        if constexpr (FENCE) __threadfence();
-        const bool late = __any_sync(FULL, need != 0);
-        t = ((got[0] + got[1]) + (got[2] + got[3])) + got[4];
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(FULL, t, o);
-        if (lane == 0) {
-            sh.sum[wid] = t;
-            sh.failed[wid] = late;
-            if (wid == 0) sh.ratio = inverse ? t / num : num / t;
-        }
     }
-    __syncthreads();
-    bool ok = true;
-    ratio = sh.ratio;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-        v[k] = sh.sum[k];
-        ok = ok && !sh.failed[k];
+    late = __any_sync(0xffffffffu, need != 0);
+    return ((got[0] + got[1]) + (got[2] + got[3])) + got[4];
+}
+
+// The sum warps: r.z, r.r and at first b.b of every iteration, and beta.
+__device__ void sum_warps(const CgArgs &a, CgShared &sh, int me, int work, int all) {
+    const int lane = threadIdx.x & 31;
+    double rz = 0.0;
+    for (unsigned long long epoch = a.epoch + 1;; ++epoch) {
+        named_sync(BAR_PARTS, all);
+        if (sh.quit) return;
+        const int nv = epoch == a.epoch + 1 ? 3 : 2;
+        for (int k = me; k < nv; k += CG_SUMS) {
+            const double t = sum_parts(sh.part[k], work, lane);
+            if (lane == 0) st_slot(a.slots + k * CG_MAX_GRID + blockIdx.x, t, epoch);
+        }
+        for (int k = me; k < nv; k += CG_SUMS) {
+            bool late;
+            const double t = warp_sum(wait_words(a.slots + k * CG_MAX_GRID, epoch, lane, late));
+            if (lane == 0) {
+                sh.sum[k] = t;
+                sh.late[k] = late;
+                if (k == W_RZ) sh.beta = rz == 0.0 ? 0.0 : t / rz;
+            }
+            if (k == W_RZ) rz = t;
+        }
+        __syncwarp();
+        named_arrive(BAR_SUMS, all);
     }
-    return ok;
 }
 
 // Value loads of the part of the matrix that is not kept in shared memory: read once an iteration,
@@ -188,9 +214,36 @@ __device__ __forceinline__ double ld_stream(const double *p) {
     return v;
 }
 
+// Brings memory to the L2 cache (16-byte aligned address and size).
+__device__ __forceinline__ void prefetch_l2(const void *p, unsigned bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+// Steps from HBM to L2 ahead of the loads (with the first slices brought there while the sums wait: a
+// step of the 341,000-DOF block 1.155 -> 1.114 ms; 4 to 10: the same within 1%).
+constexpr int CG_AHEAD = 6;
+
+// The B values of a node in y, a vector of YS values a node; 0 where not `on` (same in all lanes; a
+// branch around the one wide load was faster than the load predicated).
+template <int B, int YS>
+__device__ __forceinline__ void gather(const double *y, int32_t node, bool on, double (&w)[B]) {
+    const double *p = y + YS * (int64_t)node;
+    if constexpr (YS == 4) {
+#pragma unroll
+        for (int j = 0; j < B; ++j) w[j] = 0.0;
+        double pad;
+        if (on)
+            asm volatile("ld.global.v4.f64 {%0, %1, %2, %3}, [%4];"
+                         : "=d"(w[0]), "=d"(w[1]), "=d"(w[2]), "=d"(pad)
+                         : "l"(p));
+    } else {
+#pragma unroll
+        for (int j = 0; j < B; ++j) w[j] = on ? p[j] : 0.0;
+    }
+}
+
 // Rows of A y of the lane's node in one slice: S = 1: acc[c] is component c of the lane's node.
 // S = 4: acc[0] is component (lane & 3) of the quad's node.
-template <int B, int S, bool RES>
+template <int B, int S, bool RES, int YS>
 __device__ __forceinline__ void slice_rows(const double *val, const int32_t *col, int steps, int lane,
                                            const double *y, double (&acc)[S == 1 ? B : 1]) {
     double s[B];
@@ -217,8 +270,7 @@ __device__ __forceinline__ void slice_rows(const double *val, const int32_t *col
                 const double *q = vp + 32 * ((t + u) * (B * B) + e);
                 mm[u][e] = !on ? 0.0 : RES ? *q : ld_stream(q);
             }
-#pragma unroll
-            for (int j = 0; j < B; ++j) ww[u][j] = on ? y[B * (int64_t)c[u] + j] : 0.0;
+            gather<B, YS>(y, c[u], on, ww[u]);
         }
     };
     cols(0);
@@ -226,6 +278,9 @@ __device__ __forceinline__ void slice_rows(const double *val, const int32_t *col
     cols(U);
     for (int t = 0; t < steps; t += U) {
         double mn[U][B * B], wn[U][B];
+        if (!RES && lane == 0 && t + CG_AHEAD < steps)
+            prefetch_l2(val + (int64_t)(32 * B * B) * (t + CG_AHEAD),
+                        256 * B * B * (steps - t - CG_AHEAD < U ? steps - t - CG_AHEAD : U));
         load(t + U, mn, wn);
         cols(t + 2 * U);
 #pragma unroll
@@ -262,40 +317,61 @@ __device__ __forceinline__ void slice_rows(const double *val, const int32_t *col
     }
 }
 
+// 8-byte words of a plan of ns slices in shared memory (even: the matrix behind it is copied 16 bytes
+// at a time).
+__host__ __device__ constexpr int plan_words(int ns) { return (33 * ns + 1 + 3) / 4 * 2; }
+
 template <int B, int S, bool RES>
-__global__ void __launch_bounds__(CG_WARPS * 32, 1) k_cg_solve(CgArgs a) {
+__global__ void __launch_bounds__((CG_WARPS + CG_SUMS) * 32, 1) k_cg_solve(CgArgs a, int warps) {
     constexpr int NR = S == 1 ? B : 1;  // rows of a lane
     extern __shared__ __align__(16) unsigned char dyn[];
     __shared__ CgShared sh;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int work = 32 * warps, all = blockDim.x;  // threads that work; with the sum warps
     const int s0 = a.cta[blockIdx.x], ns = a.cta[blockIdx.x + 1] - s0;
     const int step0 = a.sbase[s0];
     // vectors of the CTA's rows, in slice order
-    double *vec = a.vec ? a.vec + (int64_t)s0 * NR * 32 : reinterpret_cast<double *>(dyn);
-    const int64_t len = a.vec ? a.vec_len : (int64_t)ns * NR * 32;
+    const bool in_shared = RES || !a.vec;
+    const int64_t own = (int64_t)ns * NR * 32, len = in_shared ? own : a.vec_len;
+    double *vec = in_shared ? reinterpret_cast<double *>(dyn) : a.vec + (int64_t)s0 * NR * 32;
     double *X = vec, *R = X + len, *Pv = R + len, *Q = Pv + len, *D = Q + len;
     const double *val = a.val + (int64_t)step0 * (32 * B * B);
     const int32_t *col = a.col + (int64_t)step0 * 32;
+    // first steps and nodes of the CTA's slices, behind the vectors: every fence empties the L1 cache
+    double *behind = reinterpret_cast<double *>(dyn) + 5 * own;
+    const int32_t *snode = a.snode + 32 * s0, *sbase = a.sbase + s0;
+    if (a.plan_shared) {
+        int32_t *plan = reinterpret_cast<int32_t *>(behind);
+        for (int i = threadIdx.x; i < 32 * ns; i += blockDim.x) plan[i] = snode[i];
+        for (int i = threadIdx.x; i <= ns; i += blockDim.x) plan[32 * ns + i] = sbase[i];
+        snode = plan;
+        sbase = plan + 32 * ns;
+        behind += plan_words(ns);
+    }
     if constexpr (RES) {  // the CTA's part of the matrix
         const int steps = a.sbase[s0 + ns] - step0;
-        double *sv = reinterpret_cast<double *>(dyn) + 5 * len;
+        double *sv = behind;
         int32_t *sc = reinterpret_cast<int32_t *>(sv + (int64_t)steps * (32 * B * B));
         for (int i = threadIdx.x; i < steps * (16 * B * B); i += blockDim.x)
             reinterpret_cast<double2 *>(sv)[i] = __ldg(reinterpret_cast<const double2 *>(val) + i);
         for (int i = threadIdx.x; i < steps * 32; i += blockDim.x) sc[i] = __ldg(col + i);
         val = sv;
         col = sc;
-        __syncthreads();
     }
-    unsigned long long epoch = a.epoch;
+    if (threadIdx.x == 0) sh.quit = 0;
+    __syncthreads();
+    if (wid >= warps) {
+        sum_warps(a, sh, wid - warps, work, all);
+        return;
+    }
     // r = b - A x, z = D^-1 r, p = q = 0 (with beta = 0 the first step forms p = z, q = A z)
-    double v3[3] = {0.0, 0.0, 0.0};
+    double v0 = 0.0, v1 = 0.0, v2 = 0.0;
     for (int sl = wid; sl < ns; sl += warps) {
-        const int t0 = a.sbase[s0 + sl] - step0, t1 = a.sbase[s0 + sl + 1] - step0;
-        const int32_t node = a.snode[32 * (s0 + sl) + lane];
+        const int t0 = sbase[sl] - step0, t1 = sbase[sl + 1] - step0;
+        const int32_t node = snode[32 * sl + lane];
         double acc[NR];
-        slice_rows<B, S, RES>(val + (int64_t)t0 * (32 * B * B), col + (int64_t)t0 * 32, t1 - t0, lane,
-                              a.x, acc);
+        slice_rows<B, S, RES, B>(val + (int64_t)t0 * (32 * B * B), col + (int64_t)t0 * 32, t1 - t0, lane,
+                                 a.x, acc);
 #pragma unroll
         for (int c = 0; c < NR; ++c) {
             const int k = (sl * NR + c) * 32 + lane;
@@ -308,10 +384,10 @@ __global__ void __launch_bounds__(CG_WARPS * 32, 1) k_cg_solve(CgArgs a) {
                 di = a.dinv[i];
                 ri = bi - acc[c];
                 const double zi = di * ri;
-                a.z[i] = zi;
-                v3[0] = __fma_rn(ri, zi, v3[0]);
-                v3[1] = __fma_rn(ri, ri, v3[1]);
-                v3[2] = __fma_rn(bi, bi, v3[2]);
+                a.z[z_stride<B> * (int64_t)node + comp] = zi;
+                v0 = __fma_rn(ri, zi, v0);
+                v1 = __fma_rn(ri, ri, v1);
+                v2 = __fma_rn(bi, bi, v2);
             }
             X[k] = xi;
             R[k] = ri;
@@ -320,41 +396,109 @@ __global__ void __launch_bounds__(CG_WARPS * 32, 1) k_cg_solve(CgArgs a) {
             Q[k] = 0.0;
         }
     }
-    double alpha, beta;
-    bool ok = grid_sum<3, true>(v3, beta, 1.0, false, a, ++epoch, sh);
-    double rz = v3[0], rr = v3[1], best = -1.0;
-    beta = 0.0;
-    const double bb = v3[2];
+    sh.part[W_RZ][threadIdx.x] = v0;
+    sh.part[W_RR][threadIdx.x] = v1;
+    sh.part[W_BB][threadIdx.x] = v2;
+    named_arrive(BAR_PARTS, all);
+    // Whether a product starts before it is known that the iteration takes place: the last one, for
+    // nothing, then costs a product (30 us at 750 nodes an SM, where the sums wait 1 us for it).
+    constexpr bool EARLY = S == 4 || B == 1;
+    double rz = 0.0, rr = 0.0, bb = 0.0, beta = 0.0, best = -1.0;
     int iters = 0, best_it = 0;
-    bool done = rr <= a.tol2 * bb;
-    while (ok && !done && iters < a.max_iter) {
-        double pq[1] = {0.0};
-        for (int sl = wid; sl < ns; sl += warps) {
-            const int t0 = a.sbase[s0 + sl] - step0, t1 = a.sbase[s0 + sl + 1] - step0;
-            const int32_t node = a.snode[32 * (s0 + sl) + lane];
+    bool ok = true, first = true;
+    for (unsigned long long epoch = a.epoch + 1;; ++epoch) {
+        // every CTA's z is visible
+        named_sync(BAR_WORK, work);
+        if (wid == 0) {
+            if (lane == 0) {
+                __threadfence();  // the CTA's z
+                st_slot(a.slots + W_Z * CG_MAX_GRID + blockIdx.x, 0.0, epoch);
+            }
+            bool late;
+            wait_words(a.slots + W_Z * CG_MAX_GRID, epoch, lane, late);
+            __threadfence();
+            if (lane == 0) sh.failed = late;
+        }
+        named_sync(BAR_WORK, work);
+        ok = !sh.failed;
+        bool stop = false, taken = false;
+        auto take = [&]() {  // the sums of the residual: the end, or beta
+            named_sync(BAR_SUMS, all);
+            taken = true;
+            rz = sh.sum[W_RZ];
+            rr = sh.sum[W_RR];
+            beta = sh.beta;
+            ok = ok && !sh.late[W_RZ] && !sh.late[W_RR];
+            if (first) {
+                bb = sh.sum[W_BB];
+                ok = ok && !sh.late[W_BB];
+            } else {
+                ++iters;
+            }
+            const bool done = rr <= a.tol2 * bb;
+            stop = !ok || done || iters >= a.max_iter;
+            if (!first && a.stagnate && iters % CG_CHECK == 0 && !done) {
+                if (best < 0.0 || rr < 0.25 * best) {
+                    best = rr;
+                    best_it = iters;
+                } else if (iters - best_it > 1000) {
+                    stop = true;
+                }
+            }
+            first = false;
+        };
+        if (!EARLY || !ok) take();
+        double pq = 0.0;
+        for (int sl = wid; sl < ns && !stop; sl += warps) {
+            const int t0 = sbase[sl] - step0, t1 = sbase[sl + 1] - step0;
+            const int32_t node = snode[32 * sl + lane];
             double acc[NR], zi[NR];
 #pragma unroll
             for (int c = 0; c < NR; ++c) {
                 const int comp = S == 1 ? c : lane & 3;
-                zi[c] = node >= 0 && comp < B ? a.z[B * (int64_t)node + comp] : 0.0;
+                zi[c] = node >= 0 && comp < B ? a.z[z_stride<B> * (int64_t)node + comp] : 0.0;
             }
-            slice_rows<B, S, RES>(val + (int64_t)t0 * (32 * B * B), col + (int64_t)t0 * 32, t1 - t0,
-                                  lane, a.z, acc);
+            slice_rows<B, S, RES, z_stride<B>>(val + (int64_t)t0 * (32 * B * B), col + (int64_t)t0 * 32,
+                                               t1 - t0, lane, a.z, acc);
+            if (!taken) take();
+            if (stop) break;
 #pragma unroll
             for (int c = 0; c < NR; ++c) {
                 const int k = (sl * NR + c) * 32 + lane;
                 const double pi = __fma_rn(beta, Pv[k], zi[c]), qi = __fma_rn(beta, Q[k], acc[c]);
                 Pv[k] = pi;
                 Q[k] = qi;
-                pq[0] = __fma_rn(pi, qi, pq[0]);
+                pq = __fma_rn(pi, qi, pq);
             }
         }
-        if (!(ok = grid_sum<1, false>(pq, alpha, rz, false, a, ++epoch, sh))) break;
+        if (!taken) take();
+        if (stop) break;
+        if (!RES && lane == 0 && wid < ns) {  // the warp's next slice, while HBM is idle
+            const int t0 = sbase[wid] - step0, t1 = sbase[wid + 1] - step0;
+            if (t1 > t0) prefetch_l2(val + (int64_t)t0 * (32 * B * B), (t1 - t0) * (256 * B * B));
+        }
+        sh.part[0][threadIdx.x] = pq;
+        named_sync(BAR_WORK, work);
+        if (wid == 0) {
+            CgSlot *set = a.slots + W_PQ * CG_MAX_GRID;
+            double t = sum_parts(sh.part[0], work, lane);
+            if (lane == 0) st_slot(set + blockIdx.x, t, epoch);
+            bool late;
+            t = warp_sum(wait_words(set, epoch, lane, late));
+            if (lane == 0) {
+                sh.pq = t;
+                sh.alpha = rz / t;  // by one warp: a division is a dozen dependent FP64 instructions
+                sh.failed = late;
+            }
+        }
+        named_sync(BAR_WORK, work);
+        if (!(ok = !sh.failed)) break;
         // breakdown: p = 0 (already converged) or A not positive definite
-        if (!(pq[0] > 0.0)) break;
-        double v2[2] = {0.0, 0.0};
+        if (!(sh.pq > 0.0)) break;
+        const double alpha = sh.alpha;
+        v0 = v1 = 0.0;
         for (int sl = wid; sl < ns; sl += warps) {
-            const int32_t node = a.snode[32 * (s0 + sl) + lane];
+            const int32_t node = snode[32 * sl + lane];
 #pragma unroll
             for (int c = 0; c < NR; ++c) {
                 const int k = (sl * NR + c) * 32 + lane;
@@ -362,30 +506,22 @@ __global__ void __launch_bounds__(CG_WARPS * 32, 1) k_cg_solve(CgArgs a) {
                 X[k] = __fma_rn(alpha, Pv[k], X[k]);
                 const double ri = __fma_rn(-alpha, Q[k], R[k]), zi = D[k] * ri;
                 R[k] = ri;
-                if (node >= 0 && comp < B) a.z[B * (int64_t)node + comp] = zi;
-                v2[0] = __fma_rn(ri, zi, v2[0]);
-                v2[1] = __fma_rn(ri, ri, v2[1]);
+                if (node >= 0 && comp < B) a.z[z_stride<B> * (int64_t)node + comp] = zi;
+                v0 = __fma_rn(ri, zi, v0);
+                v1 = __fma_rn(ri, ri, v1);
             }
         }
-        if (!(ok = grid_sum<2, true>(v2, beta, rz, true, a, ++epoch, sh))) break;
-        if (rz == 0.0) beta = 0.0;
-        rz = v2[0];
-        rr = v2[1];
-        ++iters;
-        done = rr <= a.tol2 * bb;
-        if (a.stagnate && iters % CG_CHECK == 0 && !done) {
-            if (best < 0.0 || rr < 0.25 * best) {
-                best = rr;
-                best_it = iters;
-            } else if (iters - best_it > 1000) {
-                break;
-            }
-        }
+        sh.part[W_RZ][threadIdx.x] = v0;
+        sh.part[W_RR][threadIdx.x] = v1;
+        named_arrive(BAR_PARTS, all);
     }
+    // (on every way out of the loop the sum warps wait for partial sums)
+    if (threadIdx.x == 0) sh.quit = 1;
+    named_arrive(BAR_PARTS, all);
     // the solution to the caller, or the state advanced: free rows u = x, v = (x - u) / h; a
     // clamped row is held at 0, a row without mass keeps u
     for (int sl = wid; sl < ns; sl += warps) {
-        const int32_t node = a.snode[32 * (s0 + sl) + lane];
+        const int32_t node = snode[32 * sl + lane];
 #pragma unroll
         for (int c = 0; c < NR; ++c) {
             const int comp = S == 1 ? c : lane & 3;
@@ -488,10 +624,10 @@ int launch_fill(Ctx *c, const double *val, const double *mass, double h2, cudaSt
 }
 
 template <int B, int S, bool RES> int launch_solve(Ctx *c, CgArgs &a, cudaStream_t s) {
-    void *args[] = {&a};
+    void *args[] = {&a, &c->cg_warps};
     const void *kern = (const void *)k_cg_solve<B, S, RES>;
     STA_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CG_SMEM));
-    STA_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(c->cg_grid), dim3(32 * c->cg_warps), args,
+    STA_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(c->cg_grid), dim3(32 * (c->cg_warps + CG_SUMS)), args,
                                              c->cg_smem, s));
     return STA_OK;
 }
@@ -583,7 +719,19 @@ int cg_alloc(Ctx *c) {
     const int64_t slices = (int64_t)sbase.size() - 1, steps = sbase.back();
     const size_t vec_bytes = 5 * sizeof(double) * 32 * rows * (size_t)max_slices;
     const size_t mat_bytes = (size_t)max_steps * 32 * (B * B * sizeof(double) + sizeof(int32_t));
-    const bool vec_shared = vec_bytes <= CG_SMEM;
+    const size_t plan_bytes = sizeof(double) * plan_words(max_slices);
+    const bool vec_shared = vec_bytes <= CG_SMEM, resident = vec_bytes + mat_bytes <= CG_SMEM;
+    size_t smem = resident ? vec_bytes + mat_bytes : (vec_shared ? vec_bytes : 0);
+    // The plan goes to shared memory unless the cache would pay for it with the next one of the sizes
+    // that shared memory is set aside in (scalar operator of 113,800 rows: 182 KB without the plan,
+    // 196 set aside; with it 228, and a frame's solve takes 4.3 ms instead of 4.15).
+    auto set_aside = [](size_t used) {
+        for (size_t kb : {32, 64, 100, 132, 164, 196})
+            if (used + sizeof(CgShared) + 1024 <= kb * 1024) return kb;
+        return (size_t)228;
+    };
+    c->cg_plan_shared = vec_shared && smem + plan_bytes <= CG_SMEM && set_aside(smem + plan_bytes) == set_aside(smem);
+    if (c->cg_plan_shared) smem += plan_bytes;
     STA_TRY(dev_alloc(c, &c->cg_free, n3));
     STA_TRY(dev_alloc(c, &c->cg_snode, 32 * slices));
     STA_TRY(dev_alloc(c, &c->cg_sbase, slices + 1));
@@ -593,9 +741,9 @@ int cg_alloc(Ctx *c) {
     c->cg_vec = nullptr;
     if (!vec_shared) STA_TRY(dev_alloc(c, &c->cg_vec, 5 * 32 * rows * slices));
     CgSlot *slots = nullptr;
-    STA_TRY(dev_alloc(c, &slots, 6 * CG_MAX_GRID));
+    STA_TRY(dev_alloc(c, &slots, CG_WORDS * CG_MAX_GRID));
     c->cg_slots = slots;
-    STA_CUDA_TRY(cudaMemset(slots, 0, sizeof(CgSlot) * 6 * CG_MAX_GRID));
+    STA_CUDA_TRY(cudaMemset(slots, 0, sizeof(CgSlot) * CG_WORDS * CG_MAX_GRID));
     if (!c->h_cg) {
         STA_CUDA_TRY(cudaHostAlloc((void **)&c->h_cg, sizeof(CgResult), cudaHostAllocMapped));
         STA_CUDA_TRY(cudaHostGetDevicePointer((void **)&c->d_cg, c->h_cg, 0));
@@ -615,9 +763,10 @@ int cg_alloc(Ctx *c) {
     c->cg_slices = slices;
     c->cg_steps = steps;
     c->cg_warps = warps;
-    c->cg_resident = vec_shared && vec_bytes + mat_bytes <= CG_SMEM;
-    c->cg_smem = c->cg_resident ? vec_bytes + mat_bytes : (vec_shared ? vec_bytes : 0);
-    STA_TRY(dev_alloc(c, &c->cg, 4 * n3));  // x, b, D^-1, z; last: marks the plan as complete
+    c->cg_resident = resident;
+    c->cg_smem = smem;
+    // x, b, D^-1, z (whole 32-byte words); last: marks the plan as complete
+    STA_TRY(dev_alloc(c, &c->cg, (3 * n3 + 3) / 4 * 4 + (B == 3 ? 4 : 1) * n));
     return STA_OK;
 }
 
@@ -639,12 +788,13 @@ int launch_cg_solve(Ctx *c, const double *val, const double *mass, double h2, do
     a.x = c->cg;
     a.b = c->cg + n3;
     a.dinv = c->cg + 2 * n3;
-    a.z = c->cg + 3 * n3;
+    a.z = c->cg + (3 * n3 + 3) / 4 * 4;
     a.vec = c->cg_vec;
     a.vec_len = (int64_t)c->cg_slices * 32 * (c->cg_S == 1 && !scalar ? 3 : 1);
+    a.plan_shared = c->cg_plan_shared;
     a.slots = static_cast<CgSlot *>(c->cg_slots);
     a.epoch = c->cg_epoch;
-    c->cg_epoch += 2 * (unsigned long long)max_iter + 4;  // past every sum of this solve
+    c->cg_epoch += (unsigned long long)max_iter + 2;  // past every exchange of this solve
     a.out = c->d_cg;
     a.tol2 = tol * tol;
     a.max_iter = max_iter;

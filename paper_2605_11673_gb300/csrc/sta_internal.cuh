@@ -225,7 +225,8 @@ struct Ctx {
     unsigned long long cg_epoch = 0;  // number of the last grid-wide sum given out
     int cg_grid = 0, cg_S = 1, cg_warps = 1;
     int64_t cg_slices = 0, cg_steps = 0;
-    bool cg_resident = false;   // the matrix is kept in shared memory
+    bool cg_resident = false;   // shared memory keeps the matrix,
+    bool cg_plan_shared = false;  // the nodes and steps of the slices
     size_t cg_smem = 0;
     CgResult *h_cg = nullptr, *d_cg = nullptr;  // host-mapped: a solve's result
 
