@@ -52,8 +52,7 @@ namespace {
 // three for each of 8, one or two for 15.  Steps of the 341,000-DOF block with 8, 12 and 15: 1.25, 1.15
 // and 1.19 ms; the scalar operator's frame 4.2, 4.1 and 4.3 ms.
 constexpr int CG_WARPS = 12;
-constexpr int CG_SUMS = 2;               // warps for the sums (a third one would take the working
-                                         // warps registers: 16,384 for the warps of a quadrant)
+constexpr int CG_SUMS = 2;               // warps for the sums: r.z and r.r side by side
 constexpr int CG_MAX_GRID = 160;         // CTAs at most: 5 words a lane in an exchange
 constexpr int CG_CHECK = 8;              // iterations between two looks at stagnation
 constexpr unsigned CG_SPINS = 1u << 22;  // polls of a wait (seconds)

@@ -128,29 +128,45 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t first = (int64_t)blockIdx.x * blockDim.x;
-    // (the thread's first edit, while the frame before this one may still run)
-    const uint32_t w1 = first + threadIdx.x < n ? (uint32_t)edited[(first + threadIdx.x) / 10] : 0u;
+    // the thread's first edit, its unit and its run, which no kernel of a frame writes, while the frame
+    // before this one may still run
+    uint32_t w1 = 0;
+    int32_t u1 = 0, o1 = 0, p1 = 0;
+    if (first + threadIdx.x < n) {
+        const int64_t i = first + threadIdx.x;
+        w1 = (uint32_t)edited[i / 10];
+        const int64_t k = 10 * (int64_t)(w1 & 0x7fffffffu) + i % 10;
+        u1 = __ldg(tunit + k);
+        o1 = __ldg(krun + k);
+        p1 = __ldg(tpos + k);
+    }
     dependency_wait();
     for (int64_t i0 = first; i0 < n; i0 += stride) {  // CTA-uniform
         const int64_t i = i0 + threadIdx.x;
         bool won = false, diag = false;
         int32_t u = 0;
         if (i < n) {
-            const uint32_t w = i0 == first ? w1 : (uint32_t)edited[i / 10];
+            const bool again = i0 != first;
+            const uint32_t w = again ? (uint32_t)edited[i / 10] : w1;
             const int32_t t = (int32_t)(w & 0x7fffffffu);
             const uint32_t on = w >> 31;
             const int s = (int)(i % 10);
             if (s == 0) mask[t] = (uint8_t)on;
-            u = tunit[10 * (int64_t)t + s];
-            const int64_t off = krun[10 * (int64_t)t + s];
+            u = again ? __ldg(tunit + 10 * (int64_t)t + s) : u1;
+            const int64_t off = again ? __ldg(krun + 10 * (int64_t)t + s) : o1;
             diag = s < 4;
             const int4 bm = __ldg(bmeta + u);
-            for (int q = 0; q < (diag ? 6 : 9); ++q) {
-                const long long v = __ldg(Kq + off + q);
-                atomicAdd(reinterpret_cast<unsigned long long *>(&S[unit_key(bm, diag, q)]),
-                          (unsigned long long)(on ? v : -v));
-            }
-            won = claim_unit(ustate, uext, u, tpos[10 * (int64_t)t + s], on != 0u);
+            // (all in flight with the unit's record and the claim; one after another, each before its
+            // atomic, a graph-mode frame of 2,179 swaps took 14.9 us back to back, now 13.8)
+            long long v[9];
+#pragma unroll
+            for (int q = 0; q < 9; ++q) v[q] = q < 6 || !diag ? __ldg(Kq + off + q) : 0;
+            won = claim_unit(ustate, uext, u, again ? __ldg(tpos + 10 * (int64_t)t + s) : p1, on != 0u);
+#pragma unroll
+            for (int q = 0; q < 9; ++q)
+                if (q < 6 || !diag)
+                    atomicAdd(reinterpret_cast<unsigned long long *>(&S[unit_key(bm, diag, q)]),
+                              (unsigned long long)(on ? v[q] : -v[q]));
         }
         const unsigned ball = __ballot_sync(0xffffffffu, won);
         const unsigned dball = __ballot_sync(0xffffffffu, won && diag);
