@@ -7,7 +7,7 @@
 // update kernel whose last CTA finished the sums), an iteration of a 27,783-DOF block took 29 us
 // of which under 3 us is work: the rest was launches, last-CTA tails and, every eighth iteration, a
 // host round trip.  On large systems the product was bound by the FP64 pipe (a warp FP64
-// instruction holds it for 16 cycles whatever its lanes do): the four-lane row sums and their
+// instruction holds its SM quadrant's for 64 cycles whatever its lanes do): the four-lane row sums and their
 // half-empty ends cost 1.4 times the FMAs.
 //
 // Layout.  The matrix is copied once per solve into slices (k_cg_fill): a slice is 32 lanes, a
