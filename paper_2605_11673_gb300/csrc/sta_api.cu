@@ -478,7 +478,9 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
     int64_t k = 0, e = 0, dact = 0;  // dact: change of the active count
     bool bad = false;
     // (ids compare as unsigned, and an edit's state tests are one condition: the order of the
-    // checks matters only for the message, which edit_error finds again)
+    // checks matters only for the message, which edit_error finds again.  The kinds of edit keep
+    // branches of their own: edits of a kind come in runs, and one branchless form for both cost a
+    // frame of 40,000 deactivations 75 us instead of 65.)
     const int64_t segments = counts ? c->n_inst : 1;
     int64_t seg = 0, seg0 = 0;
     for (; seg < segments && !bad; seg += !bad) {
@@ -512,12 +514,16 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
                 stage[k] = (int32_t)(a + o32);
                 stage[k + 1] = (int32_t)((b + o32) | 0x80000000u);
                 k += 2;
-            } else {  // DEACTIVATE wants the active bit, ACTIVATE does not
-                const uint8_t want = E.op == STA_ACTIVATE ? 0 : TS_ACTIVE;
-                if (((s1 & TS_STAMP) == gen) | ((s1 & TS_ACTIVE) != want)) { bad = true; break; }
-                st[a] = (uint8_t)(gen | (want ^ TS_ACTIVE));
-                stage[k++] = (int32_t)((a + o32) | ((uint32_t)E.op << 31));
-                dact += 2 * E.op - 1;
+            } else if (E.op == STA_DEACTIVATE) {
+                if (((s1 & TS_STAMP) == gen) | ((s1 & TS_ACTIVE) == 0)) { bad = true; break; }
+                st[a] = gen;
+                stage[k++] = (int32_t)(a + o32);
+                --dact;
+            } else {
+                if (((s1 & TS_STAMP) == gen) | ((s1 & TS_ACTIVE) != 0)) { bad = true; break; }
+                st[a] = (uint8_t)(TS_ACTIVE | gen);
+                stage[k++] = (int32_t)((a + o32) | 0x80000000u);
+                ++dact;
             }
         }
     }
