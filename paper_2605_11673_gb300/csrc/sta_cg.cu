@@ -35,9 +35,9 @@
 // a CTA whose wait runs out marks the solve as failed and leaves, and so do, one after another,
 // all others.
 //
-// Measured (GB300, time of an iteration with two launches -> now): 27,783-DOF block 29 -> 10.3 us,
-// 341,000-DOF pre-fractured block 62 -> 41 us (FP64 floor of its product 24 us), scalar operator of
-// 113,800 rows 34 -> 12 us.  With both sums on the path of the iteration (11.4, 48 and 13 us), the
+// Measured (GB300, time of an iteration with two launches -> now): 27,783-DOF block 29 -> 10.2 us,
+// 341,000-DOF pre-fractured block 62 -> 40 us (FP64 floor of its product 24 us), scalar operator of
+// 113,800 rows 34 -> 11.6 us.  With both sums on the path of the iteration (11.4, 48 and 13 us), the
 // small block's product took 3 us, the sums 3 and 3.8 us, the updates 0.6 us.
 #include <algorithm>
 #include <cmath>
@@ -701,9 +701,16 @@ int cg_alloc(Ctx *c) {
             quad[k % 4] += weight(order[i * per]);
         }
         const int32_t first = sbase.back();
-        size_t deep = 0;
-        for (auto &q : of) deep = std::max(deep, q.size());
-        for (size_t i = 0; i < warps * deep; ++i) {
+        // the warps of a quadrant in descending number of slices, and no places past the last slice: an
+        // empty one costs a warp its turn and shared memory (36 places for 32 slices: solves of the
+        // scalar operator of 113,800 rows 4.15 ms, now 3.99; steps of 341,000 DOFs 1.10, now 1.08)
+        for (int w = 0; w < warps; ++w)
+            for (int v = w + 4; v < warps; v += 4)
+                if (of[v].size() > of[w].size()) std::swap(of[v], of[w]);
+        size_t places = 0;
+        for (int w = 0; w < warps; ++w)
+            if (!of[w].empty()) places = std::max(places, w + 1 + warps * (of[w].size() - 1));
+        for (size_t i = 0; i < places; ++i) {
             const auto &q = of[i % warps];
             const bool has = i / warps < q.size();  // else an empty slice
             const size_t at = has ? (size_t)q[i / warps] * per : 0;
