@@ -159,6 +159,7 @@ int sta::create_impl(const double *nodes, int64_t n_nodes, const int32_t *tets, 
     if (cudaGetDevice(&c->device) != cudaSuccess ||
         cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess)
         return bail(fail(STA_ECUDA, "no CUDA device"));
+    c->small_frames = small_frames_fit();
     if (cudaEventCreateWithFlags(&x->h2d_done, cudaEventDisableTiming) != cudaSuccess)
         return bail(fail(STA_ECUDA, "cudaEventCreate failed"));
 
@@ -437,7 +438,8 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
     // the frame block to stage into: one of the graph mode's two host-mapped blocks (fixed
     // capacity), or the context's pinned block (grown on demand); a small frame needs neither
     const bool two_kernels = c->op == STA_OP_ELASTICITY && !c->dyn;
-    const bool small = m > 0 && m <= SMALL_FRAME && two_kernels && c->policy == STA_POLICY_REFOLD;
+    const bool small = m > 0 && m <= SMALL_FRAME && two_kernels && c->policy == STA_POLICY_REFOLD &&
+                       c->small_frames;
     const bool use_graph = c->graph_on && m <= c->gcap && !small;
     FrameHeader *h = nullptr, *d = nullptr;
     int32_t by_value[SMALL_FRAME];

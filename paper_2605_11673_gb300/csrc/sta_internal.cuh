@@ -121,6 +121,7 @@ struct Ctx {
     int rebuild_form = STA_REBUILD_AUTO;  // sta_set_rebuild_form
     int64_t n_active = 0;                 // active tetrahedra (host mirror count)
     int num_sms = 0;
+    bool small_frames = false;    // the device runs k_frame_small
     int device = 0;
 
     // inputs
@@ -330,8 +331,8 @@ int launch_rebuild(Ctx *c, cudaStream_t s);                      // sta_rebuild.
 int rebuild_form_of(const Ctx *c);  // the form the next rebuild takes (AUTO resolved)
 // Frames of at most this many edited tetrahedra take one launch, k_frame_small (elasticity, re-fold
 // policy, without the dynamics' mass update).  Two kernels take 8.3-8.9 us a frame back to back from
-// 16 edits to 122, one cluster 5.8 us for 16, 7.5 for 32, 8.9 for 48, 9.4 for 60 and 14 for 90; a
-// frame that is waited for is at 48 edits 1 us longer, at 32 even.
+// 16 edits to 122, one cluster 5.6 us for 16, 5.8 for 32, 7.2 for 48, 7.4 for 60 and 9.2 for 90; but
+// a frame that is waited for is even at 32 edits and 1.5 us longer at 48 (21.5 us).
 constexpr int SMALL_FRAME = 40;
 // In graph mode, frames of at most this many edited tetrahedra are launched kernel by kernel all the
 // same: of such launches a frame's first kernel starts while the last one of the frame before runs,
@@ -340,6 +341,7 @@ constexpr int SMALL_FRAME = 40;
 // (2,488 scattered: 19.5 -> 14.7, 2,179 of a crack front: 13.3 -> 14.8): they stay with the graph.
 constexpr int DIRECT_FRAME = 1024;
 int launch_small_frame(Ctx *c, const int32_t *edited, int m, cudaStream_t s);
+bool small_frames_fit();
 // whether a streaming frame of this context stores its touched count into h_count_mapped
 bool frame_counts_to_host(const Ctx *c);
 // one streaming frame: the edited list, its count (*m_dev, or m) and the counters; cap: edited

@@ -206,13 +206,14 @@ k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
     launch_dependents();
 }
 
-// A small frame in one launch: a cluster of SF_CTAS CTAs claims the units of the frame's edits, which
+// A small frame in one launch: a cluster of SF_CTAS CTAs, one an SM, claims the units of the frame's edits, which
 // come by value with the launch, and after a cluster barrier each CTA folds the units that its own
 // threads won, listed in its shared memory (diagonal units from the front, pair units from the
 // back).  Such a frame is all latency: launch, drain and dependent round trips (edit count, edits,
 // list, list count), which this kernel does not make or overlaps with the frame before.  Frames of 4
-// edits back to back: 10.9 us as two kernels of a graph, 5.4 here; of 32 edits: 11.3 and 7.4.
-constexpr int SF_CTAS = 8;
+// edits back to back: 10.9 us as two kernels of a graph, 5.4 here; of 32 edits: 11.3 and 5.8 (7.4 with
+// 8 CTAs, whose warps fold two rounds one after the other; 7.1 with 16 of 4 warps).
+constexpr int SF_CTAS = 16;
 constexpr int SF_WARPS = 7;  // (their operand columns: 42 KB)
 constexpr int SF_THREADS = 32 * SF_WARPS;
 constexpr int SF_ROUNDS = (10 * SMALL_FRAME + SF_CTAS * SF_THREADS - 1) / (SF_CTAS * SF_THREADS);
@@ -414,6 +415,24 @@ int launch_stream_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t 
     STA_TRY(launch_fold_list(c, c->touched, c->nunits, cnt + 1, 10 * (cap > 0 ? cap : 1), s,
                              c->d_count_mapped, next_cnt ? next_cnt + 1 : nullptr));
     return launch_dyn_mass_edited(c, edited, m, m_dev, cap, s);
+}
+
+// Whether the device can run k_frame_small's cluster (more than 8 CTAs is not a size every one has).
+bool small_frames_fit() {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(SF_CTAS);
+    cfg.blockDim = dim3(SF_THREADS);
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = SF_CTAS;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int clusters = 0;
+    const bool fits = cudaFuncSetAttribute(k_frame_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+                      cudaOccupancyMaxActiveClusters(&clusters, k_frame_small, &cfg) == cudaSuccess && clusters > 0;
+    if (!fits) cudaGetLastError();
+    return fits;
 }
 
 // A frame of m <= SMALL_FRAME edited tetrahedra (tet id | new state << 31, host memory) in one launch.
