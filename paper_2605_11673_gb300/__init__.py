@@ -159,10 +159,12 @@ def _host(a, dtype):
 def _ptr(a) -> int:
     """Address of a non-empty C-contiguous host array's data: through the buffer protocol,
     which costs half of `a.ctypes.data` on the per-frame path; read-only arrays take the
-    latter."""
+    latter.  Any other memory order raises: its address would be read as rows."""
     try:
         return C.addressof(C.c_char.from_buffer(a))
     except TypeError:
+        if not a.flags.c_contiguous:
+            raise ValueError("a C-contiguous array is needed") from None
         return a.ctypes.data
 
 
@@ -567,6 +569,7 @@ def sta_batch_apply_edits(h: int, edits_per_instance, stream=None) -> None:
     if allp is None or allp.dtype != np.int32 or allp.ndim != 2 or allp.shape[1] != 3:
         parts = [_host(e, np.int32).reshape(-1, 3) for e in parts]
         allp = np.concatenate(parts, 0) if parts else np.zeros((0, 3), np.int32)
+    allp = np.ascontiguousarray(allp)  # (parts that are all column-major join to a column-major array)
     k = _sizes(h)["k"]
     if len(parts) != k:
         raise ValueError(f"one edit list per instance: {k} expected, got {len(parts)}")
