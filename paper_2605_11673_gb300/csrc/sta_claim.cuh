@@ -13,7 +13,7 @@ namespace {
 // Contributor j of unit u becomes active (`on`) or inactive: moves its bit (which holds the other
 // state: edits are validated) and counts a claim of the unit, for j < 32 in one atomic; true for
 // the thread that claims the unit first in its frame.
-__device__ __forceinline__ bool claim_unit(UnitState *__restrict__ ustate, uint32_t *__restrict__ uext,
+__device__ __forceinline__ bool claim_unit(UnitState *ustate, uint32_t *uext,
                                            int32_t u, int32_t j, bool on) {
     unsigned long long step = 1ull << 32;  // one claim
     if (j < 32) {

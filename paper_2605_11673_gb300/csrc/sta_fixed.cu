@@ -180,10 +180,9 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
 // Fixed-point frame, phase 2: convert the touched units' entries and release the claims.
 // 9 lanes per listed unit (6 used by a diagonal unit), 3 units per warp.  `next_count`, when
 // given, is the next frame's count pair (graph mode alternates two), zeroed here.
-__global__ void k_fx_convert(FoldArgs A, const int32_t *__restrict__ list,
-                             const unsigned long long *__restrict__ count,
-                             const int16_t *__restrict__ e, const long long *__restrict__ S,
-                             UnitState *__restrict__ ustate, unsigned long long *next_count) {
+__global__ void k_fx_convert(FoldArgs A, const int32_t *list, const unsigned long long *count,
+                             const int16_t *__restrict__ e, const long long *S, UnitState *ustate,
+                             unsigned long long *next_count) {
     dependency_wait();
     if (next_count && blockIdx.x == 0 && threadIdx.x == 0) {
         next_count[0] = 0;
@@ -193,16 +192,16 @@ __global__ void k_fx_convert(FoldArgs A, const int32_t *__restrict__ list,
     const int g = lane / 9, q = lane % 9;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t nitems = (int64_t)*count;
+    const int64_t nitems = (int64_t)__ldcg(count);
     for (int64_t base = warp * 3; base < nitems; base += nwarps * 3) {
         const int64_t item = base + g;
         if (g >= 3 || item >= nitems) continue;
-        const int32_t u = __ldg(list + item);
+        const int32_t u = __ldcg(list + item);
         const int4 bm = __ldg(A.bmeta + u);
         const bool diag = bm.y & 1;
         if (diag && q >= 6) continue;
         const int2 mir = diag ? make_int2(0, 0) : __ldg(A.bmirror + u);
-        fx_write(A, e, bm, mir, diag, q, S[unit_key(bm, diag, q)]);
+        fx_write(A, e, bm, mir, diag, q, __ldcg(S + unit_key(bm, diag, q)));
         if (q == 0) ustate[u].claims = 0;
     }
 }

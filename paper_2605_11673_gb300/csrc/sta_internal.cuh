@@ -270,7 +270,9 @@ inline void ts_set_active(Ctx *c, int64_t t, bool on) {
 }
 
 // Launch of a kernel that may start while the stream's kernel before it still runs: it orders itself
-// with dependency_wait(), before which it reads only what no kernel writes.
+// with dependency_wait(), before which it reads only what no kernel writes.  What the kernel before
+// writes it reads after that with plain loads or from L2 (__ldcg), never over the read-only path
+// (__ldg, const __restrict__), which asks that memory stays as it is from the kernel's start.
 template <typename... P, typename... Q>
 int launch_overlapped(void (*kern)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
                       Q... args) {

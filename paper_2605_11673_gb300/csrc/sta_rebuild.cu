@@ -86,13 +86,13 @@ struct FlagStream {
     int32_t base;    // stripe position of bit 0 of `mask`
     unsigned mask;   // set flags of positions base .. base+31 not yet handed out
     uint8_t ahead;   // this lane's flag of position base + 32 + lane
-    __device__ __forceinline__ void load_ahead(const uint8_t *__restrict__ flags, int32_t b, int32_t G,
+    __device__ __forceinline__ void load_ahead(const uint8_t *flags, int32_t b, int32_t G,
                                                int32_t n, int lane) {
         const int64_t t = b + (int64_t)(base + 32 + lane) * G;
-        ahead = t < n ? __ldg(flags + t) : 0;
+        ahead = t < n ? __ldcg(flags + t) : 0;
     }
     // the next flagged chunk, or n past the end of the stripe
-    __device__ __forceinline__ int32_t next(const uint8_t *__restrict__ flags, int32_t b, int32_t G,
+    __device__ __forceinline__ int32_t next(const uint8_t *flags, int32_t b, int32_t G,
                                             int32_t n, int lane) {
         while (mask == 0) {  // warp-uniform
             base += 32;
@@ -216,7 +216,7 @@ __device__ __forceinline__ void fold_round(const FoldArgs &A, const FxArgs &X, c
     if (lane == 0) bar_arrive(empty);
     if (direct) {
         const int4 bm = __ldg(A.bmeta + first + ul);
-        const uint4 st = __ldg(reinterpret_cast<const uint4 *>(A.ustate) + first + ul);
+        const uint4 st = __ldcg(reinterpret_cast<const uint4 *>(A.ustate) + first + ul);
         acc = fold_global<FX, V>(src, ActiveRuns(true, st, bm.w, bm.z + q, W, A.uext));
     }
     if (valid) write_entry<FX, DIAG, V>(A, X, P, m.out, m.rs, m.out2, m.rs2, key, acc, ex);
@@ -230,7 +230,7 @@ __device__ __forceinline__ void fold_round(const FoldArgs &A, const FxArgs &X, c
 template <bool FX, bool ZF>
 __global__ void __launch_bounds__(FOLD_THREADS, FOLD_CTAS)
 k_fold_flat(FoldArgs A, const int2 *__restrict__ chunks, int32_t nchunks,
-            const uint8_t *__restrict__ cflag, FxArgs X, unsigned int *__restrict__ fault) {
+            const uint8_t *cflag, FxArgs X, unsigned int *__restrict__ fault) {
     using V = typename std::conditional<FX, long long, double>::type;
     const V *src;
     if constexpr (FX) src = X.Kq; else src = A.Ke;
@@ -404,7 +404,7 @@ k_fold_flat(FoldArgs A, const int2 *__restrict__ chunks, int32_t nchunks,
 // 512 contiguous bytes), and sets every value (and, for the fixed-point fold, every integer sum) to
 // zero with 16-byte stores.
 __global__ void k_zero_fill(const int2 *__restrict__ chunks, int32_t nchunks,
-                            const UnitState *__restrict__ ustate, bool eps, uint8_t *__restrict__ cflag, double *__restrict__ val,
+                            const UnitState *ustate, bool eps, uint8_t *__restrict__ cflag, double *__restrict__ val,
                             long long *__restrict__ S, int64_t nnz) {
     const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
@@ -415,7 +415,7 @@ __global__ void k_zero_fill(const int2 *__restrict__ chunks, int32_t nchunks,
         const int2 r = __ldg(chunks + c);
         bool on = eps && r.y >> 8;
         if (lane < (r.y & 255)) {
-            const uint4 st = __ldg(reinterpret_cast<const uint4 *>(ustate) + r.x + lane);
+            const uint4 st = __ldcg(reinterpret_cast<const uint4 *>(ustate) + r.x + lane);
             on = on || (st.x | st.z) != 0u || st.w != UNIT_NARROW;
         }
         on = __any_sync(0xffffffffu, on);
@@ -459,7 +459,7 @@ __device__ __forceinline__ void small_round(const FoldArgs &A, const FxArgs &X, 
     const int32_t u = rec.x + P.ul;
     const int4 bm = __ldg(A.bmeta + u);
     const int2 mir = __ldg(A.bmirror + u);
-    const uint4 st = __ldg(reinterpret_cast<const uint4 *>(A.ustate) + u);
+    const uint4 st = __ldcg(reinterpret_cast<const uint4 *>(A.ustate) + u);
     const int32_t key = bm.x + P.ei * (bm.y >> 1) + P.ej;
     int ex = 0;
     if constexpr (FX) ex = (int)__ldg(X.e + key);

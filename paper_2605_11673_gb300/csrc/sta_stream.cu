@@ -36,7 +36,7 @@ constexpr int ENT_WARPS = 4;
 // One warp round over units first .. first+NG-1 of one kind of the n_units that unit(k) names;
 // `col`: the lane's column of the warp's shared buffer.
 template <bool DIAG, typename F>
-__device__ __forceinline__ void fold_units(const FoldArgs &A, UnitState *__restrict__ ustate, F unit,
+__device__ __forceinline__ void fold_units(const FoldArgs &A, UnitState *ustate, F unit,
                                            int64_t first, int64_t n_units, double *col, int lane,
                                            bool has_eps) {
     constexpr int GW = DIAG ? RUN_DIAG : RUN_PAIR;   // lanes (entries) per unit
@@ -93,7 +93,7 @@ __device__ __forceinline__ void fold_units(const FoldArgs &A, UnitState *__restr
 // given, is the count pair of the next frame (graph mode alternates two), zeroed here so that
 // the captured frame needs no memset node of its own.
 __global__ void __launch_bounds__(ENT_WARPS * 32)
-k_fold_entries(FoldArgs A, UnitState *__restrict__ ustate, const int32_t *__restrict__ list,
+k_fold_entries(FoldArgs A, UnitState *ustate, const int32_t *list,
                unsigned long long *count, int64_t cap, unsigned long long *host_count,
                unsigned long long *next_count) {
     __shared__ double stage[ENT_WARPS][ENT_DEPTH * 32];
@@ -117,10 +117,10 @@ k_fold_entries(FoldArgs A, UnitState *__restrict__ ustate, const int32_t *__rest
     const bool has_eps = A.eps != 0.0;
     for (int64_t item = warp; item < gd + gp; item += nwarps) {  // warp-uniform
         if (item < gd)
-            fold_units<true>(A, ustate, [&](int64_t k) { return __ldg(list + k); }, item * ENT_DG, nd,
+            fold_units<true>(A, ustate, [&](int64_t k) { return __ldcg(list + k); }, item * ENT_DG, nd,
                              col, lane, has_eps);
         else
-            fold_units<false>(A, ustate, [&](int64_t k) { return __ldg(list + (cap - 1 - k)); },
+            fold_units<false>(A, ustate, [&](int64_t k) { return __ldcg(list + (cap - 1 - k)); },
                               (item - gd) * ENT_PG, np, col, lane, has_eps);
     }
 }
@@ -225,9 +225,9 @@ struct SmallFrame {
 
 __global__ void __cluster_dims__(SF_CTAS, 1, 1) __launch_bounds__(SF_THREADS)
 k_frame_small(const __grid_constant__ SmallFrame F, FoldArgs A, const int32_t *__restrict__ tunit,
-              const int32_t *__restrict__ tpos, UnitState *__restrict__ ustate,
-              uint32_t *__restrict__ uext, uint8_t *__restrict__ mask, unsigned long long *counters,
-              unsigned long long *host_count) {
+              const int32_t *__restrict__ tpos, UnitState *ustate, uint32_t *uext,
+              uint8_t *__restrict__ mask, unsigned long long *counters,
+              unsigned long long *host_count) {  // (the folds read ustate's and uext's words through A)
     constexpr int CAP = SF_ROUNDS * SF_THREADS;
     __shared__ double stage[SF_WARPS][ENT_DEPTH * 32];
     __shared__ int32_t won[CAP];
