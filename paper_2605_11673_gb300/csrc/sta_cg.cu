@@ -119,12 +119,15 @@ struct CgShared {
 };
 
 // Barriers between a CTA's warps: the working warps among themselves, partial sums to the sum
-// warps, sums to the working warps.
+// warps, sums to the working warps.  (bar.sync and bar.arrive are aligned instructions, which a warp
+// has to execute as a whole: it is brought together first, as it may come from a branch of one lane.)
 enum { BAR_WORK = 1, BAR_PARTS, BAR_SUMS };
 __device__ __forceinline__ void named_sync(int id, int threads) {
+    __syncwarp();
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 __device__ __forceinline__ void named_arrive(int id, int threads) {
+    __syncwarp();
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
@@ -200,7 +203,6 @@ __device__ void sum_warps(const CgArgs &a, CgShared &sh, int me, int work, int a
             }
             if (k == W_RZ) rz = t;
         }
-        __syncwarp();
         named_arrive(BAR_SUMS, all);
     }
 }

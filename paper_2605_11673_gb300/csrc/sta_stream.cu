@@ -218,6 +218,13 @@ constexpr int SF_WARPS = 7;  // (their operand columns: 42 KB)
 constexpr int SF_THREADS = 32 * SF_WARPS;
 constexpr int SF_ROUNDS = (10 * SMALL_FRAME + SF_CTAS * SF_THREADS - 1) / (SF_CTAS * SF_THREADS);
 
+// Every thread of the cluster, whose earlier writes are visible afterwards.  The aligned forms want whole
+// warps: each is brought together first, as it may come from a branch of one lane.
+__device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 struct SmallFrame {
     int32_t m;
     int32_t edited[SMALL_FRAME];
@@ -250,7 +257,7 @@ k_frame_small(const __grid_constant__ SmallFrame F, FoldArgs A, const int32_t *_
             pos[r] = __ldg(tpos + k);
         }
     }
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_sync();
     dependency_wait();
 #pragma unroll
     for (int r = 0; r < SF_ROUNDS; ++r) {
@@ -273,7 +280,7 @@ k_frame_small(const __grid_constant__ SmallFrame F, FoldArgs A, const int32_t *_
                      "r"((unsigned)(9 * nd + 18 * np)) : "memory");
     }
     // every claim and activity change of the frame is done and visible
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_sync();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         counters[3] = touched;
         *host_count = touched;
