@@ -20,7 +20,11 @@
 //    parts are formed once per pair by a pass over the gradient (k_grad_units), which also turns
 //    the 144 scattered 8-byte loads of a tetrahedron into 42 16-byte ones;
 //  * g_0 = -(g_1 + g_2 + g_3) is put into the quadratic forms: 6 blocks instead of 10, 3 gradients
-//    instead of 4, and dx_0 = -(dx_1 + dx_2 + dx_3);
+//    instead of 4, and dx_0 = -(dx_1 + dx_2 + dx_3).  Node 0 here is the node with the largest
+//    gradient (k_elements notes which: the edges' differences start at it as well): the others'
+//    gradients are no larger than what they add up to, so nothing cancels.  With a node of small
+//    gradient in its place, the far tip of a tetrahedron 100 times as high as wide, and the upstream
+//    gradient on that node, the results lost four digits;
 //  * the value of a form is half its gradient's product with g; 3 divisions instead of 8.
 // No evaluation order is fixed here; every product-sum is an FMA chain.
 #include "sta_internal.cuh"
@@ -110,6 +114,17 @@ struct Sym {  // 00 01 02 11 12 22
     double c[6];
 };
 
+template <typename T> __device__ __forceinline__ void swap_if(bool on, T &a, T &b) {
+    const T t = on ? b : a;
+    b = on ? a : b;
+    a = t;
+}
+__device__ __forceinline__ void swap_if(bool on, V3 &a, V3 &b) {
+    swap_if(on, a.x, b.x);
+    swap_if(on, a.y, b.y);
+    swap_if(on, a.z, b.z);
+}
+
 __device__ __forceinline__ double tr(const Sym &s) { return (s.c[0] + s.c[3]) + s.c[5]; }
 // y += S g
 __device__ __forceinline__ void sym_add(const Sym &s, const V3 &g, V3 &y) {
@@ -141,24 +156,42 @@ __global__ void __launch_bounds__(128, 3)
 k_adjoint(const double4_32a *__restrict__ X, const int4 *__restrict__ tets,
           const double2 *__restrict__ mat, const int32_t *__restrict__ list,
           const unsigned long long *__restrict__ count, const int32_t *__restrict__ tunit,
-          const double *__restrict__ gu, double *__restrict__ dE, double *__restrict__ dnu,
+          const uint8_t *__restrict__ steep, const double *__restrict__ gu, double *__restrict__ dE, double *__restrict__ dnu,
           double *__restrict__ dXe) {
     const int64_t n = (int64_t)*count;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int64_t t = list[i];
-        const int4 q = tets[t];
+        int4 q = tets[t];
         const double2 em = mat[t];
-        const double *row[10];  // slots 0..3 diagonal, 4..9 pairs (01) (02) (03) (12) (13) (23)
+        int32_t unit[10];  // slots 0..3 diagonal, 4..9 pairs (01) (02) (03) (12) (13) (23)
         {
             const int2 *tu = reinterpret_cast<const int2 *>(tunit + 10 * t);
 #pragma unroll
             for (int h = 0; h < 5; ++h) {
                 const int2 v = __ldg(tu + h);
-                row[2 * h] = gu + GU * (int64_t)v.x;
-                row[2 * h + 1] = gu + GU * (int64_t)v.y;
+                unit[2 * h] = v.x;
+                unit[2 * h + 1] = v.y;
             }
         }
+        // node k in the place of k ^ z, z the node to eliminate: an even permutation
+        const int z = __ldg(steep + t);
+        const bool z1 = z & 1, z2 = z & 2;
+        swap_if(z1, q.x, q.y);
+        swap_if(z1, q.z, q.w);
+        swap_if(z1, unit[0], unit[1]);
+        swap_if(z1, unit[2], unit[3]);
+        swap_if(z1, unit[5], unit[8]);
+        swap_if(z1, unit[6], unit[7]);
+        swap_if(z2, q.x, q.z);
+        swap_if(z2, q.y, q.w);
+        swap_if(z2, unit[0], unit[2]);
+        swap_if(z2, unit[1], unit[3]);
+        swap_if(z2, unit[4], unit[9]);
+        swap_if(z2, unit[6], unit[7]);
+        const double *row[10];
+#pragma unroll
+        for (int h = 0; h < 10; ++h) row[h] = gu + GU * (int64_t)unit[h];
         const double4_32a x0 = X[q.x];
         const V3 d1 = diff(X[q.y], x0), d2 = diff(X[q.z], x0), d3 = diff(X[q.w], x0);
         const V3 c1 = cross(d2, d3), c2 = cross(d3, d1), c3 = cross(d1, d2);
@@ -238,6 +271,10 @@ k_adjoint(const double4_32a *__restrict__ X, const int4 *__restrict__ tets,
         }
         o[0] = {-((o[1].x + o[2].x) + o[3].x), -((o[1].y + o[2].y) + o[3].y),
                 -((o[1].z + o[2].z) + o[3].z)};
+        swap_if(z1, o[0], o[1]);
+        swap_if(z1, o[2], o[3]);
+        swap_if(z2, o[0], o[2]);
+        swap_if(z2, o[1], o[3]);
         double2 *out = reinterpret_cast<double2 *>(dXe + 12 * t);
         out[0] = make_double2(o[0].x, o[0].y);
         out[1] = make_double2(o[0].z, o[1].x);
@@ -308,7 +345,7 @@ int launch_adjoint(Ctx *c, const double *gval, double *dE, double *dnu, double *
         k_grad_units<<<(unsigned)capped(c->nunits, 256, c->num_sms * 8), 256, 0, s>>>(
             c->nunits, c->bmeta, c->bmirror, gval, c->gunit);
         k_adjoint<<<(unsigned)capped(c->T, 128, c->num_sms * 3), 128, 0, s>>>(
-            c->X, c->tets, c->mat, c->act_list, c->act_count, c->tunit, c->gunit, dE, dnu, c->dXe);
+            c->X, c->tets, c->mat, c->act_list, c->act_count, c->tunit, c->steep, c->gunit, dE, dnu, c->dXe);
     }
     if (c->n > 0)
         k_node_grad<<<(unsigned)capped(3 * c->n, 256, c->num_sms * 8), 256, 0, s>>>(

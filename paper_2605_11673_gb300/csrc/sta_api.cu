@@ -183,7 +183,7 @@ int sta::create_impl(const double *nodes, int64_t n_nodes, const int32_t *tets, 
     if ((rc = build_pattern(c, s))) return bail(rc);
 
     if ((rc = dev_alloc(c, &c->Ke, c->ke_len)) || (rc = dev_alloc(c, &c->mask, n_tets)) ||
-        (rc = dev_alloc(c, &c->val, c->nnz)))
+        (rc = dev_alloc(c, &c->val, c->nnz)) || (rc = dev_alloc(c, &c->steep, n_tets)))
         return bail(rc);
     unsigned long long init[4] = {0ull, 0ull, ~0ull, 0ull};
     if (cudaMemcpyAsync(c->counters, init, sizeof init, cudaMemcpyHostToDevice, s) ||

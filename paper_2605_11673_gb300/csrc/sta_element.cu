@@ -69,6 +69,22 @@ __device__ __forceinline__ bool element(double4_32a x0, double4_32a x1, double4_
     return true;
 }
 
+// The local node with the largest gradient component, compared by high words (no FP64 operation):
+// its gradient is the largest to within a factor of sqrt(3).  For the adjoint.
+__device__ __forceinline__ int steepest(const Element &e) {
+    int node = 0, most = -1;
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+        const int m = max(max(__double2hiint(e.g[a].x) & 0x7fffffff, __double2hiint(e.g[a].y) & 0x7fffffff),
+                          __double2hiint(e.g[a].z) & 0x7fffffff);
+        if (m > most) {
+            most = m;
+            node = a;
+        }
+    }
+    return node;
+}
+
 // Entries of the block (a, b): a == b the 6 entries i <= j, else all 9, row-major, transposed when
 // `tr` (a run is stored with the lower node id's rows).
 template <int a, int b>
@@ -207,7 +223,8 @@ __global__ void __launch_bounds__(EL_TPB, 4)
 k_elements(const double4_32a *__restrict__ X, const int4 *__restrict__ tets,
            const double2 *__restrict__ mat, const int32_t *__restrict__ list,
            const unsigned long long *__restrict__ count, int64_t T,
-           const int32_t *__restrict__ krun, double *__restrict__ Ke, unsigned long long *bad) {
+           const int32_t *__restrict__ krun, double *__restrict__ Ke, uint8_t *__restrict__ steep,
+           unsigned long long *bad) {
     __shared__ double bufs[EL_TPB / 32][32 * RUN_PAIR];
     const int lane = threadIdx.x & 31;
     double *buf = bufs[threadIdx.x >> 5];
@@ -234,6 +251,7 @@ k_elements(const double4_32a *__restrict__ X, const int4 *__restrict__ tets,
                 atomicAdd(&bad[0], 1ull);
                 atomicMin(&bad[2], (unsigned long long)t);
             }
+            steep[t] = (uint8_t)steepest(e);
             t01 = q.x > q.y; t02 = q.x > q.z; t03 = q.x > q.w;
             t12 = q.y > q.z; t13 = q.y > q.w; t23 = q.z > q.w;
         } else {
@@ -336,7 +354,7 @@ int launch_elements(Ctx *c, bool active_only, cudaStream_t s) {
     k_elements<<<(unsigned)blocks, EL_TPB, 0, s>>>(c->X, c->tets, c->mat,
                                                    active_only ? c->act_list : nullptr,
                                                    active_only ? c->act_count : nullptr, c->T,
-                                                   c->krun, c->Ke, c->counters);
+                                                   c->krun, c->Ke, c->steep, c->counters);
     STA_CUDA_TRY(cudaGetLastError());
     return STA_OK;
 }

@@ -159,6 +159,7 @@ struct Ctx {
     int32_t *tunit = nullptr;      // T x 10: unit of tet t's slot (4 diagonal, 6 pairs)
     int32_t *nt_ptr = nullptr;     // n + 1: node -> incident tetrahedra
     int32_t *nt_list = nullptr;    // 4 T: incident tetrahedra, ascending id
+    uint8_t *steep = nullptr;      // T: local node whose barycentric gradient is about the largest (adjoint)
     double *dXe = nullptr;         // T x 12: per-element position gradients (adjoint, lazily)
     double *gunit = nullptr;       // nunits x 10: parts of each unit's gradient (adjoint, lazily)
     int32_t *nt_run = nullptr;     // 4 T: offset in dXe of each nt_list entry (adjoint, lazily)
