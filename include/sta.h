@@ -15,6 +15,12 @@
  *    any device work, and a rejected call changes no state.
  *  - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  Device
  *    work is enqueued on it; calls return before it finishes unless stated otherwise.
+ *  - The waits inside a rebuild's kernels are bounded.  Should one run out, the values are
+ *    incomplete, and every later call that reads or maintains them (sta_apply_edits and its
+ *    variants, sta_last_touched, sta_spmv, sta_solve, sta_dyn_step, sta_dyn_apply) returns
+ *    STA_ECUDA; those that wait for the stream also look after it, and then what they have
+ *    computed is to be discarded.  A rebuild (sta_full_rebuild, sta_refold, sta_set_policy) puts
+ *    it right; one that finds a failure no call has reported yet reports it instead, once.
  *  - Host arrays passed in are copied; the caller keeps ownership.  Device pointers handed
  *    out by sta_csr / sta_scatter_map are owned by the context and valid until sta_destroy.
  *  - Matrix layout: scalar CSR with 3n rows, DOF 3v + i (node v, component i).  Row 3a+i

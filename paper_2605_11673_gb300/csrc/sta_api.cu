@@ -51,10 +51,25 @@ static int64_t set_host_mask(Ctx *c, const uint8_t *__restrict__ mask, uint8_t *
     return na;
 }
 
-// A bounded wait of an earlier rebuild ran out: its values are incomplete.
-static int check_fault(const Ctx *c) {
-    if (c->h_fault && *reinterpret_cast<volatile unsigned int *>(c->h_fault))
-        return fail(STA_ECUDA, "an earlier rebuild did not complete");
+// Whether a bounded wait of an earlier rebuild ran out, which leaves its values incomplete.
+static bool rebuild_failed(const Ctx *c) {
+    return c->h_fault && *reinterpret_cast<volatile unsigned int *>(c->h_fault);
+}
+
+// For every call that reads or maintains the values.
+int sta::check_values(Ctx *c) {
+    if (!rebuild_failed(c)) return STA_OK;
+    c->fault_told = true;
+    return fail(STA_ECUDA, "an earlier rebuild did not complete: its values are incomplete until the next rebuild");
+}
+
+// For a rebuild: it reports an earlier one's failure that no call has reported yet, else puts it right.
+static int begin_rebuild(Ctx *c, cudaStream_t s) {
+    if (!rebuild_failed(c)) return STA_OK;
+    if (!c->fault_told) return check_values(c);
+    STA_CUDA_TRY(cudaStreamSynchronize(s));  // (the failed one may still be running)
+    *reinterpret_cast<volatile unsigned int *>(c->h_fault) = 0u;
+    c->fault_told = false;
     return STA_OK;
 }
 
@@ -290,7 +305,7 @@ int sta_full_rebuild(sta_ctx *x, const uint8_t *mask, int mask_on_device, void *
     Ctx *c = &x->c;
     if (c->T > 0 && !mask) return fail(STA_EINVAL, "mask is NULL");
     cudaStream_t s = (cudaStream_t)stream;
-    STA_TRY(check_fault(c));
+    STA_TRY(begin_rebuild(c, s));
     if (c->T > 0) {
         STA_TRY(wait_staging(x));
         if (mask_on_device) {  // read back for the host mirror; the device copy is the 0/1 one
@@ -350,7 +365,7 @@ int sta_get_rebuild_form(const sta_ctx *x, int32_t *form) {
 
 int sta_refold(sta_ctx *x, void *stream) {
     if (!x) return fail(STA_EINVAL, "ctx is NULL");
-    STA_TRY(check_fault(&x->c));
+    STA_TRY(begin_rebuild(&x->c, (cudaStream_t)stream));
     if (x->c.graph_on) {
         STA_CUDA_TRY(cudaGraphLaunch(x->c.g_refold, (cudaStream_t)stream));
         return STA_OK;
@@ -425,6 +440,7 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
                      void *stream) {
     Ctx *c = &x->c;
     if (n_edits > (INT32_MAX / 32)) return fail(STA_ERANGE, "too many edits in one call");
+    STA_TRY(check_values(c));
     cudaStream_t s = (cudaStream_t)stream;
     // edited tetrahedra (a swap edits two): 2 n_edits bounds them; they are counted first only where
     // that bound is past the capacity of the block at hand, or the frame is a small one.  Staging
@@ -586,9 +602,11 @@ extern "C" {
 
 int sta_last_touched(sta_ctx *x, int64_t *touched_nnz, void *stream) {
     if (!x || !touched_nnz) return fail(STA_EINVAL, "NULL argument");
+    STA_TRY(check_values(&x->c));
     cudaStream_t s = (cudaStream_t)stream;
     if (x->c.count_on_host) {  // the frame's fold kernel stored it in host-mapped memory
         STA_CUDA_TRY(cudaStreamSynchronize(s));
+        STA_TRY(check_values(&x->c));
         *touched_nnz = (int64_t)*reinterpret_cast<volatile unsigned long long *>(x->c.h_count_mapped);
         return STA_OK;
     }
@@ -596,6 +614,7 @@ int sta_last_touched(sta_ctx *x, int64_t *touched_nnz, void *stream) {
     STA_CUDA_TRY(cudaMemcpyAsync(x->h_count, x->c.last_counters + 3, sizeof *x->h_count,
                                  cudaMemcpyDeviceToHost, s));
     STA_CUDA_TRY(cudaStreamSynchronize(s));
+    STA_TRY(check_values(&x->c));
     *touched_nnz = (int64_t)*x->h_count;
     return STA_OK;
 }
@@ -649,6 +668,7 @@ int sta_set_policy(sta_ctx *x, int32_t policy, void *stream) {
     Ctx *c = &x->c;
     if (c->graph_on) return fail(STA_ESTATE, "disable graph mode before changing the policy");
     cudaStream_t s = (cudaStream_t)stream;
+    STA_TRY(begin_rebuild(c, s));
     if (c->op == STA_OP_PROXY) {  // integer state either way: nothing to prepare
         c->policy = policy;
         return launch_values(c, s);
@@ -712,6 +732,7 @@ int sta_adjoint(sta_ctx *x, const double *grad_val, double *dE, double *dnu, dou
 int sta_spmv(sta_ctx *x, const double *val, const double *xv, double *y, void *stream) {
     if (!x) return fail(STA_EINVAL, "ctx is NULL");
     if (x->c.nrows > 0 && (!xv || !y)) return fail(STA_EINVAL, "NULL argument");
+    STA_TRY(check_values(&x->c));
     return launch_spmv(&x->c, val ? val : x->c.val, xv, y, (cudaStream_t)stream);
 }
 

@@ -358,6 +358,7 @@ extern "C" int sta_dyn_step(sta_ctx *x, double tol, int32_t max_iter, int32_t *i
     Ctx *c = &x->c;
     if (!c->dyn) return fail(STA_ESTATE, "call sta_dyn_setup first");
     if (!(tol >= 0.0) || max_iter < 0) return fail(STA_EINVAL, "tol and max_iter must be >= 0");
+    STA_TRY(check_values(c));
     cudaStream_t s = (cudaStream_t)stream;
     const int64_t n3 = 3 * c->n;
     CgResult res{};
@@ -369,6 +370,7 @@ extern "C" int sta_dyn_step(sta_ctx *x, double tol, int32_t max_iter, int32_t *i
         STA_TRY(launch_cg_solve(c, c->val, c->mass, c->dyn_h * c->dyn_h, tol, max_iter, false, nullptr,
                                 true, s, &res));
     }
+    STA_TRY(check_values(c));  // (a rebuild that was still running before)
     if (iters) *iters = res.iters;
     if (rel_res) *rel_res = res.bb > 0.0 ? std::sqrt(res.rr / res.bb) : 0.0;
     return STA_OK;
@@ -381,6 +383,7 @@ extern "C" int sta_dyn_apply(sta_ctx *x, const double *xv, double *y, void *stre
     const int64_t n3 = 3 * c->n;
     if (n3 == 0) return STA_OK;
     if (!xv || !y) return fail(STA_EINVAL, "NULL argument");
+    STA_TRY(check_values(c));
     cudaStream_t s = (cudaStream_t)stream;
     double *xf = c->cg + 3 * n3;  // the solve's z buffer (free between steps)
     const unsigned gv = dyn_grid(c, n3);
@@ -399,6 +402,7 @@ extern "C" int sta_solve(sta_ctx *x, const double *val, const double *b, const u
     if (!(tol >= 0.0) || max_iter < 0) return fail(STA_EINVAL, "tol and max_iter must be >= 0");
     const int64_t n3 = c->nrows;  // DOFs: 3 per node, or 1 for the proxy operator
     if (n3 > 0 && (!b || !free || !xv)) return fail(STA_EINVAL, "NULL argument");
+    STA_TRY(check_values(c));
     cudaStream_t s = (cudaStream_t)stream;
     STA_TRY(cg_alloc(c));
     const double *A = val ? val : c->val;
@@ -415,6 +419,7 @@ extern "C" int sta_solve(sta_ctx *x, const double *val, const double *b, const u
         STA_CUDA_TRY(cudaGetLastError());
         STA_TRY(launch_cg_solve(c, A, nullptr, 1.0, tol, max_iter, true, xv, false, s, &res));
     }
+    STA_TRY(check_values(c));  // (a rebuild that was still running before)
     if (iters) *iters = res.iters;
     if (rel_res) *rel_res = res.bb > 0.0 ? std::sqrt(res.rr / res.bb) : 0.0;
     return STA_OK;

@@ -147,6 +147,7 @@ struct Ctx {
     uint8_t *cflag = nullptr;      // nchunks: the zero-fill rebuild's "fold this chunk"
     unsigned int *d_fault = nullptr;  // host-mapped word: a fold's bounded wait ran out
     unsigned int *h_fault = nullptr;
+    bool fault_told = false;          // a call has reported it
     int4 *bmeta = nullptr;         // nunits: {value offset of (a,b), rs_a << 1 | diagonal, offset of
                                    //   the unit's first run, contributors}
     int2 *bmirror = nullptr;       // nunits: {value offset of (b,a), rs_b}
@@ -378,6 +379,7 @@ int launch_stream_scratch(Ctx *c, int64_t m, const int32_t *d_edited, int32_t *t
 int create_impl(const double *nodes, int64_t n_nodes, const int32_t *tets, int64_t n_tets,
                 const double *young, const double *poisson, const sta_options *opt, void *stream,
                 sta_ctx **out);
+int check_values(Ctx *c);    // sta_api.cu: STA_ECUDA while the values are a failed rebuild's
 void graph_release(Ctx *c);  // sta_graph.cu
 int apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const int64_t *counts,
                 void *stream);  // sta_api.cu

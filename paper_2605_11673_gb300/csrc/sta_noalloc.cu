@@ -41,6 +41,7 @@ extern "C" int sta_apply_edits_noalloc(sta_ctx *x, const sta_edit *edits, int64_
     if (!x) return fail(STA_EINVAL, "ctx is NULL");
     Ctx *c = &x->c;
     if (n_edits < 0 || (n_edits > 0 && !edits)) return fail(STA_EINVAL, "bad edit list");
+    STA_TRY(check_values(c));
     int dev = -1;
     STA_CUDA_TRY(cudaGetDevice(&dev));
     if (dev != c->device)
