@@ -192,16 +192,16 @@ __global__ void k_fx_convert(FoldArgs A, const int32_t *list, const unsigned lon
     const int g = lane / 9, q = lane % 9;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t nitems = (int64_t)__ldcg(count);
+    const int64_t nitems = (int64_t)*count;
     for (int64_t base = warp * 3; base < nitems; base += nwarps * 3) {
         const int64_t item = base + g;
         if (g >= 3 || item >= nitems) continue;
-        const int32_t u = __ldcg(list + item);
+        const int32_t u = list[item];
         const int4 bm = __ldg(A.bmeta + u);
         const bool diag = bm.y & 1;
         if (diag && q >= 6) continue;
         const int2 mir = diag ? make_int2(0, 0) : __ldg(A.bmirror + u);
-        fx_write(A, e, bm, mir, diag, q, __ldcg(S + unit_key(bm, diag, q)));
+        fx_write(A, e, bm, mir, diag, q, S[unit_key(bm, diag, q)]);
         if (q == 0) ustate[u].claims = 0;
     }
 }

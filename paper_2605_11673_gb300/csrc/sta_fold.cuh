@@ -47,8 +47,8 @@ __device__ __forceinline__ double plus_zero(double v) {
 
 // The active contributors of one unit in list order, as offsets of their runs.  Every lane of a
 // unit walks the same bits: no list is built, and the offset of the next operand is known without
-// a load (but for the words of contributors 64 and up; those come from L2: claims of the same kernel,
-// or of one that still ran when this one started, change them).
+// a load (but for the words of contributors 64 and up, plain loads: claims of the same kernel, or of
+// one that still ran when this one started, change them).
 struct ActiveRuns {
     uint32_t w, w1;       // bits left in the current word; word 1
     int32_t run, stride;  // offset of the current word's first run; doubles per run
@@ -62,14 +62,14 @@ struct ActiveRuns {
     // active contributors in all words (call before next)
     __device__ __forceinline__ int count() const {
         int n = __popc(w) + __popc(w1);
-        for (int i = 0; i < words; ++i) n += __popc(__ldcg(ext + i));
+        for (int i = 0; i < words; ++i) n += __popc(ext[i]);
         return n;
     }
     // offset of the next active contributor's run; called at most count() times
     __device__ __forceinline__ int32_t next() {
         while (w == 0 && k <= words) {
             run += 32 * stride;
-            w = k == 0 ? w1 : __ldcg(ext + (k - 1));
+            w = k == 0 ? w1 : ext[k - 1];
             ++k;
         }
         const int j = __ffs(w) - 1;

@@ -459,7 +459,7 @@ __device__ __forceinline__ void small_round(const FoldArgs &A, const FxArgs &X, 
     const int32_t u = rec.x + P.ul;
     const int4 bm = __ldg(A.bmeta + u);
     const int2 mir = __ldg(A.bmirror + u);
-    const uint4 st = __ldcg(reinterpret_cast<const uint4 *>(A.ustate) + u);
+    const uint4 st = reinterpret_cast<const uint4 *>(A.ustate)[u];
     const int32_t key = bm.x + P.ei * (bm.y >> 1) + P.ej;
     int ex = 0;
     if constexpr (FX) ex = (int)__ldg(X.e + key);

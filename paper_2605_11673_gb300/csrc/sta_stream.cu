@@ -117,10 +117,10 @@ k_fold_entries(FoldArgs A, UnitState *ustate, const int32_t *list,
     const bool has_eps = A.eps != 0.0;
     for (int64_t item = warp; item < gd + gp; item += nwarps) {  // warp-uniform
         if (item < gd)
-            fold_units<true>(A, ustate, [&](int64_t k) { return __ldcg(list + k); }, item * ENT_DG, nd,
+            fold_units<true>(A, ustate, [&](int64_t k) { return list[k]; }, item * ENT_DG, nd,
                              col, lane, has_eps);
         else
-            fold_units<false>(A, ustate, [&](int64_t k) { return __ldcg(list + (cap - 1 - k)); },
+            fold_units<false>(A, ustate, [&](int64_t k) { return list[cap - 1 - k]; },
                               (item - gd) * ENT_PG, np, col, lane, has_eps);
     }
 }
