@@ -414,6 +414,13 @@ static int grow_frames(Ctx *c, int64_t cap, cudaStream_t s) {
     return STA_OK;
 }
 
+// Whether the stream records a CUDA graph of the caller's.
+static bool capturing(cudaStream_t s) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+    return st != cudaStreamCaptureStatusNone;
+}
+
 // What is wrong with an edit of tetrahedra [0, T) shifted by off, in the order of the checks.
 static const char *edit_error(const Ctx *c, const sta_edit &E, int64_t T, int64_t off, uint8_t gen,
                               bool batch) {
@@ -574,7 +581,7 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
     if (use_graph) {
         unsigned long long *cnt = c->d_gcnt + 4 * gb;
         c->last_counters = cnt;
-        if (m > 0 && m <= DIRECT_FRAME && two_kernels)
+        if (m > 0 && m <= DIRECT_FRAME && two_kernels && !capturing(s))
             STA_TRY(launch_stream_frame(c, frame_edited(d), m, nullptr, cnt, m, s,
                                         c->d_gcnt + 4 * (gb ^ 1)));
         else
@@ -591,6 +598,8 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
     }
     unsigned long long *cnt = c->f_cnt + 4 * gb;
     c->last_counters = cnt;
+    // (a captured frame may be replayed without the other block's frame, which zeroes these, in between)
+    if (capturing(s)) STA_CUDA_TRY(cudaMemsetAsync(cnt, 0, 4 * sizeof(unsigned long long), s));
     STA_TRY(launch_stream_frame(c, frame_edited(d), m, nullptr, cnt, m, s, c->f_cnt + 4 * (gb ^ 1)));
     STA_CUDA_TRY(cudaEventRecord(c->f_done[gb], s));
     c->f_pending[gb] = true;

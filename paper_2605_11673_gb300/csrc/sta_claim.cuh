@@ -10,22 +10,15 @@
 namespace sta {
 namespace {
 
-// Contributor j of unit u becomes active (`on`) or inactive: moves its bit (which holds the other
-// state: edits are validated) and counts a claim of the unit, for j < 32 in one atomic; true for
-// the thread that claims the unit first in its frame.
-__device__ __forceinline__ bool claim_unit(UnitState *ustate, uint32_t *uext,
-                                           int32_t u, int32_t j, bool on) {
-    unsigned long long step = 1ull << 32;  // one claim
-    if (j < 32) {
-        const unsigned long long bit = 1ull << j;
-        step = on ? step + bit : step - bit;
-    } else {
-        uint32_t *w = j < 64 ? &ustate[u].w1 : uext + ustate[u].xoff + (j / 32 - 2);
-        const uint32_t bit = 1u << (j & 31);
-        if (on) atomicOr(w, bit);
-        else atomicAnd(w, ~bit);
-    }
-    return (atomicAdd(reinterpret_cast<unsigned long long *>(ustate + u), step) >> 32) == 0ull;
+// Contributor j of unit u becomes active (`on`) or inactive: sets or clears its bit and claims the unit;
+// true for the thread that claims the unit first in its frame.  The bit needs no answer, so the claim's
+// is all a thread waits for.
+__device__ __forceinline__ bool claim_unit(UnitState *ustate, uint32_t *uext, int32_t u, int32_t j, bool on) {
+    uint32_t *w = j < 32 ? &ustate[u].w0 : (j < 64 ? &ustate[u].w1 : uext + ustate[u].xoff + (j / 32 - 2));
+    const uint32_t bit = 1u << (j & 31);
+    if (on) atomicOr(w, bit);
+    else atomicAnd(w, ~bit);
+    return atomicExch(&ustate[u].claimed, 1u) == 0u;
 }
 
 // Called by every thread of a CTA of THREADS threads, the same number of times.  Lane 0 of

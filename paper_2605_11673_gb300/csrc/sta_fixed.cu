@@ -202,7 +202,7 @@ __global__ void k_fx_convert(FoldArgs A, const int32_t *list, const unsigned lon
         if (diag && q >= 6) continue;
         const int2 mir = diag ? make_int2(0, 0) : __ldg(A.bmirror + u);
         fx_write(A, e, bm, mir, diag, q, S[unit_key(bm, diag, q)]);
-        if (q == 0) ustate[u].claims = 0;
+        if (q == 0) ustate[u].claimed = 0;
     }
 }
 

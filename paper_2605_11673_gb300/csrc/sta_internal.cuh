@@ -61,12 +61,11 @@ __host__ __device__ inline int32_t contrib_code(int32_t t, int la, int lb) {
 __host__ __device__ inline int32_t code_tet(int32_t code) { return (code >> 4) & 0x07ffffff; }
 
 // Activity of a unit's contributors, kept equal to the mask by every call that changes it, and the
-// claims of the streaming frame in progress.  Contributor j's bit: w0 bit j (j < 32), w1 bit j - 32
-// (j < 64), else bit j % 32 of uext[xoff + j / 32 - 2].  w0 and claims are one 64-bit word to the
-// claim kernels: one atomic sets or clears the bit (by adding or subtracting it) and counts the
-// claim, and the thread that finds no claim yet has won the unit.  claims is 0 between frames.
+// claim of the streaming frame in progress.  Contributor j's bit: w0 bit j (j < 32), w1 bit j - 32
+// (j < 64), else bit j % 32 of uext[xoff + j / 32 - 2].  claimed is 0 between frames.  Every change is
+// one that may be made again (a bit set or cleared, a claim marked), so a captured frame may be replayed.
 struct __align__(16) UnitState {
-    uint32_t w0, claims, w1, xoff;  // xoff: UNIT_NARROW for at most 64 contributors
+    uint32_t w0, claimed, w1, xoff;  // xoff: UNIT_NARROW for at most 64 contributors
 };
 constexpr uint32_t UNIT_NARROW = 0xffffffffu;
 

@@ -70,7 +70,7 @@ __device__ __forceinline__ void fold_units(const FoldArgs &A, UnitState *ustate,
     }
     if (!valid) return;
     // release the claim: all claims are done, and the other lanes of the unit do not read it
-    if (q == 0) ustate[u].claims = 0;
+    if (q == 0) ustate[u].claimed = 0;
     if (DIAG) {
         // 6-run entry q = (i, j), i <= j
         const int i = q < 3 ? 0 : (q < 5 ? 1 : 2), j = q < 3 ? q : (q < 5 ? q - 2 : 2);
