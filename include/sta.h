@@ -394,6 +394,7 @@ int sta_proxy_state(const sta_ctx *ctx, const int32_t **mult, const int32_t **de
  * the mass update.  May be called again to change rho, h, f or clamped (resets u and v).
  * sta_dyn_step: one step; synchronises `stream`; *iters = CG iterations, *rel_res =
  * ||r|| / ||b|| at exit (0 when b = 0); either may be NULL.  Reaching max_iter is not an error.
+ * STA_ECUDA when a grid-wide wait of the solve ran out: u and v are those of before.
  * sta_dyn_apply: y = (M_t + h^2 K_t) x on the free DOFs, 0 elsewhere (x read on the free DOFs
  * only); x and y are device arrays of 3n doubles, y must not overlap x; asynchronous on
  * `stream`.  The operator the step's CG applies, for a caller's own solver.
@@ -418,7 +419,8 @@ int sta_dyn_set_state(sta_ctx *ctx, const double *u, const double *v, int on_dev
  * (n_rows of sta_csr: 3n for elasticity, n for the proxy operator, whose solve is the paper's
  * per-frame solve of Algorithm 1).  Same kernels as the implicit-Euler step (fixed-order
  * reductions: deterministic).  Synchronises `stream`.  *iters and *rel_res (||r|| / ||b_f||
- * from the recurrence) may be NULL.  Both operators.
+ * from the recurrence) may be NULL.  Both operators.  STA_ECUDA when a grid-wide wait of the solve
+ * ran out: x is as it was.
  *
  * sta_outer_grad -- the adjoint rule of such a solve: grad_val[k] = -lam[row(k)] u[col(k)]
  * for entries k between free DOFs, 0 elsewhere (lam, u: device nrows doubles; free: device

@@ -31,9 +31,11 @@
 // the new z (a word without a sum: the stores are visible), and r.z with r.r, which only the end
 // of the next product needs: warps of their own add and exchange them while the others already
 // multiply.  Each has its own words; a CTA can store the next word of an exchange only after an
-// exchange that every CTA enters when it has read the last one.  The waits are bounded (CG_SPINS);
+// exchange that every CTA enters when it has read the last one.  The waits are bounded;
 // a CTA whose wait runs out marks the solve as failed and leaves, and so do, one after another,
-// all others.
+// all others.  The solution goes to the context's x, and from there to the caller's vector or the
+// state by a kernel of its own that first looks whether any CTA has failed (k_cg_finish): a CTA that
+// was the only one late at the last exchange would otherwise leave its rows alone behind.
 //
 // Measured (GB300, time of an iteration with two launches -> now): 27,783-DOF block 29 -> 10.2 us,
 // 341,000-DOF pre-fractured block 62 -> 40 us (FP64 floor of its product 24 us), scalar operator of
@@ -55,7 +57,6 @@ constexpr int CG_WARPS = 12;
 constexpr int CG_SUMS = 2;               // warps for the sums: r.z and r.r side by side
 constexpr int CG_MAX_GRID = 160;         // CTAs at most: 5 words a lane in an exchange
 constexpr int CG_CHECK = 8;              // iterations between two looks at stagnation
-constexpr unsigned CG_SPINS = 1u << 22;  // polls of a wait (seconds)
 constexpr size_t CG_SMEM = 216 * 1024;   // dynamic shared memory at most (CgShared: 9 KB)
 
 // One CTA's word of a grid-wide sum, alone in its 128-byte line: packed 16 bytes apart, the words
@@ -91,20 +92,18 @@ struct CgArgs {
     double *vec;           // 5 vectors in slice order when shared memory does not hold them
     int64_t vec_len;       // of one of them
     bool plan_shared;
-    CgSlot *slots;         // CG_WORDS exchanges x CG_MAX_GRID
+    CgSlot *slots;         // CG_WORDS exchanges x CG_MAX_GRID, and the failure's
     unsigned long long epoch;
+    unsigned spins;        // polls of a wait at most
     CgResult *out;         // host-mapped
     double tol2;
     int32_t max_iter;
     bool stagnate;
-    double *xout;          // the caller's solution (sta_solve), or
-    double *u, *v;         // the state to advance (implicit Euler)
-    const uint8_t *fr, *clamped;
-    double h;
 };
 
 // The exchanges: r.z, r.r and (once) b.b, p.q, z.
 enum { W_RZ, W_RR, W_BB, W_PQ, W_Z, CG_WORDS };
+constexpr int CG_FAILED = CG_WORDS * CG_MAX_GRID;  // its epoch: the first one of the last solve that failed
 
 // Nodes of three values are gathered as one aligned word of four: the three loads of a 24-byte
 // record cost the L1 cache nearly three times as much.
@@ -153,7 +152,8 @@ __device__ __forceinline__ double sum_parts(const double *p, int n, int lane) {
 
 // Waits until every CTA's word of one exchange carries `epoch`.  Returns the lane's part of their
 // sum; `late` (same in all lanes): the wait ran out.
-__device__ __forceinline__ double wait_words(const CgSlot *set, unsigned long long epoch, int lane, bool &late) {
+__device__ __forceinline__ double wait_words(const CgSlot *set, unsigned long long epoch, unsigned spins, int lane,
+                                             bool &late) {
     constexpr int PER = CG_MAX_GRID / 32;
     double got[PER];
     unsigned need = 0;  // words still to come
@@ -162,7 +162,7 @@ __device__ __forceinline__ double wait_words(const CgSlot *set, unsigned long lo
         got[i] = 0.0;
         if (lane + 32 * i < (int)gridDim.x) need |= 1u << i;
     }
-    for (unsigned spin = 0; need && spin < CG_SPINS; ++spin) {
+    for (unsigned spin = 0; need && spin < spins; ++spin) {
         double w[PER];
         unsigned long long e[PER];
 #pragma unroll
@@ -195,7 +195,7 @@ __device__ void sum_warps(const CgArgs &a, CgShared &sh, int me, int work, int a
         }
         for (int k = me; k < nv; k += CG_SUMS) {
             bool late;
-            const double t = warp_sum(wait_words(a.slots + k * CG_MAX_GRID, epoch, lane, late));
+            const double t = warp_sum(wait_words(a.slots + k * CG_MAX_GRID, epoch, a.spins, lane, late));
             if (lane == 0) {
                 sh.sum[k] = t;
                 sh.late[k] = late;
@@ -416,7 +416,7 @@ __global__ void __launch_bounds__((CG_WARPS + CG_SUMS) * 32, 1) k_cg_solve(CgArg
                 st_slot(a.slots + W_Z * CG_MAX_GRID + blockIdx.x, 0.0, epoch);
             }
             bool late;
-            wait_words(a.slots + W_Z * CG_MAX_GRID, epoch, lane, late);
+            wait_words(a.slots + W_Z * CG_MAX_GRID, epoch, a.spins, lane, late);
             __threadfence();
             if (lane == 0) sh.failed = late;
         }
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__((CG_WARPS + CG_SUMS) * 32, 1) k_cg_solve(CgArg
             double t = sum_parts(sh.part[0], work, lane);
             if (lane == 0) st_slot(set + blockIdx.x, t, epoch);
             bool late;
-            t = warp_sum(wait_words(set, epoch, lane, late));
+            t = warp_sum(wait_words(set, epoch, a.spins, lane, late));
             if (lane == 0) {
                 sh.pq = t;
                 sh.alpha = rz / t;  // by one warp: a division is a dozen dependent FP64 instructions
@@ -519,25 +519,13 @@ __global__ void __launch_bounds__((CG_WARPS + CG_SUMS) * 32, 1) k_cg_solve(CgArg
     // (on every way out of the loop the sum warps wait for partial sums)
     if (threadIdx.x == 0) sh.quit = 1;
     named_arrive(BAR_PARTS, all);
-    // the solution to the caller, or the state advanced: free rows u = x, v = (x - u) / h; a
-    // clamped row is held at 0, a row without mass keeps u
-    for (int sl = wid; sl < ns; sl += warps) {
+    // (ok: the sums of the first residual are complete, so no CTA reads x any more)
+    for (int sl = wid; sl < ns && ok; sl += warps) {
         const int32_t node = snode[32 * sl + lane];
 #pragma unroll
         for (int c = 0; c < NR; ++c) {
             const int comp = S == 1 ? c : lane & 3;
-            if (!ok || node < 0 || comp >= B) continue;
-            const double xi = X[(sl * NR + c) * 32 + lane];
-            const int64_t i = B * (int64_t)node + comp;
-            if (a.xout) a.xout[i] = xi;
-            if (!a.u) continue;
-            if (a.fr[i]) {
-                a.v[i] = (xi - a.u[i]) / a.h;
-                a.u[i] = xi;
-            } else {
-                a.v[i] = 0.0;
-                if (a.clamped[node]) a.u[i] = 0.0;
-            }
+            if (node >= 0 && comp < B) a.x[B * (int64_t)node + comp] = X[(sl * NR + c) * 32 + lane];
         }
     }
     if (threadIdx.x == 0 && (blockIdx.x == 0 || !ok)) {
@@ -547,6 +535,28 @@ __global__ void __launch_bounds__((CG_WARPS + CG_SUMS) * 32, 1) k_cg_solve(CgArg
             a.out->bb = bb;
         } else {
             a.out->failed = 1;
+            a.slots[CG_FAILED].epoch = a.epoch + 1;
+        }
+    }
+}
+
+// The solution of a solve that no CTA has given up to the caller (xout), or the state advanced: free
+// rows u = x, v = (x - u) / h; a clamped row is held at 0, a row without mass keeps u.
+__global__ void k_cg_finish(int64_t n3, const double *x, const CgSlot *slots, unsigned long long epoch,
+                            double *__restrict__ xout, double *__restrict__ u, double *__restrict__ v,
+                            const uint8_t *__restrict__ fr, const uint8_t *__restrict__ clamped, double h) {
+    dependency_wait();
+    if (slots[CG_FAILED].epoch == epoch) return;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n3;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        if (xout) {
+            xout[i] = x[i];
+        } else if (fr[i]) {
+            v[i] = (x[i] - u[i]) / h;
+            u[i] = x[i];
+        } else {
+            v[i] = 0.0;
+            if (clamped[i / 3]) u[i] = 0.0;
         }
     }
 }
@@ -749,9 +759,9 @@ int cg_alloc(Ctx *c) {
     c->cg_vec = nullptr;
     if (!vec_shared) STA_TRY(dev_alloc(c, &c->cg_vec, 5 * 32 * rows * slices));
     CgSlot *slots = nullptr;
-    STA_TRY(dev_alloc(c, &slots, CG_WORDS * CG_MAX_GRID));
+    STA_TRY(dev_alloc(c, &slots, CG_FAILED + 1));
     c->cg_slots = slots;
-    STA_CUDA_TRY(cudaMemset(slots, 0, sizeof(CgSlot) * CG_WORDS * CG_MAX_GRID));
+    STA_CUDA_TRY(cudaMemset(slots, 0, sizeof(CgSlot) * (CG_FAILED + 1)));
     if (!c->h_cg) {
         STA_CUDA_TRY(cudaHostAlloc((void **)&c->h_cg, sizeof(CgResult), cudaHostAllocMapped));
         STA_CUDA_TRY(cudaHostGetDevicePointer((void **)&c->d_cg, c->h_cg, 0));
@@ -779,9 +789,10 @@ int cg_alloc(Ctx *c) {
 }
 
 // Solves (h2 K(val) + mass) x = b on the rows with cg_free set, from the x, b and D^-1 in the
-// context's buffers; waits for the result.  mass null: none (h2 = 1).
+// context's buffers, into xout, or (null) into the state of the implicit-Euler loop, which it advances;
+// waits for the result.  A solve that fails changes neither.  mass null: none (h2 = 1).
 int launch_cg_solve(Ctx *c, const double *val, const double *mass, double h2, double tol,
-                    int32_t max_iter, bool stagnate, double *xout, bool advance, cudaStream_t s,
+                    int32_t max_iter, bool stagnate, double *xout, cudaStream_t s,
                     CgResult *res) {
     const int64_t n3 = c->nrows;
     *res = CgResult{};
@@ -807,14 +818,7 @@ int launch_cg_solve(Ctx *c, const double *val, const double *mass, double h2, do
     a.tol2 = tol * tol;
     a.max_iter = max_iter;
     a.stagnate = stagnate;
-    a.xout = xout;
-    if (advance) {
-        a.u = c->du;
-        a.v = c->dv;
-        a.fr = c->cg_free;
-        a.clamped = c->clamped;
-        a.h = c->dyn_h;
-    }
+    a.spins = c->cg_spins;
     *c->h_cg = CgResult{};
     if (scalar) {
         STA_TRY((c->cg_S == 1 ? launch_fill<1, 1>(c, val, mass, h2, s) : launch_fill<1, 4>(c, val, mass, h2, s)));
@@ -823,6 +827,9 @@ int launch_cg_solve(Ctx *c, const double *val, const double *mass, double h2, do
         STA_TRY((c->cg_S == 1 ? launch_fill<3, 1>(c, val, mass, h2, s) : launch_fill<3, 4>(c, val, mass, h2, s)));
         STA_TRY((c->cg_S == 1 ? launch_solve<3, 1>(c, a, s) : launch_solve<3, 4>(c, a, s)));
     }
+    const int64_t ctas = std::min<int64_t>((n3 + 255) / 256, 8 * (int64_t)c->num_sms);
+    STA_TRY(launch_overlapped(k_cg_finish, (unsigned)ctas, 256, 0, s, n3, (const double *)a.x, (const CgSlot *)a.slots,
+                              a.epoch + 1, xout, c->du, c->dv, c->cg_free, c->clamped, c->dyn_h));
     STA_CUDA_TRY(cudaStreamSynchronize(s));
     *res = *c->h_cg;
     if (res->failed) return fail(STA_ECUDA, "the solve's grid-wide sum did not complete");

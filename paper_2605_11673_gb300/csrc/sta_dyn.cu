@@ -368,7 +368,7 @@ extern "C" int sta_dyn_step(sta_ctx *x, double tol, int32_t max_iter, int32_t *i
                                                       c->cg + n3, c->cg + 2 * n3, c->cg_free);
         STA_CUDA_TRY(cudaGetLastError());
         STA_TRY(launch_cg_solve(c, c->val, c->mass, c->dyn_h * c->dyn_h, tol, max_iter, false, nullptr,
-                                true, s, &res));
+                                s, &res));
     }
     STA_TRY(check_values(c));  // (a rebuild that was still running before)
     if (iters) *iters = res.iters;
@@ -417,7 +417,7 @@ extern "C" int sta_solve(sta_ctx *x, const double *val, const double *b, const u
             k_cg_init_static<<<gv, DYN_TPB, 0, s>>>(n3, c->adj_ptr, c->adj, c->row_ptr, A, free, b,
                                                     xv, xw, bw, dinv, c->cg_free);
         STA_CUDA_TRY(cudaGetLastError());
-        STA_TRY(launch_cg_solve(c, A, nullptr, 1.0, tol, max_iter, true, xv, false, s, &res));
+        STA_TRY(launch_cg_solve(c, A, nullptr, 1.0, tol, max_iter, true, xv, s, &res));
     }
     STA_TRY(check_values(c));  // (a rebuild that was still running before)
     if (iters) *iters = res.iters;

@@ -218,13 +218,14 @@ struct Ctx {
     int32_t *dyn_perm = nullptr;  // n: sta_dyn_apply's node order (ascending row length)
 
     // conjugate gradients (sta_cg.cu), allocated by the first sta_dyn_setup or sta_solve
-    double *cg = nullptr;       // 4 x nrows: x, b, D^-1, z
+    double *cg = nullptr;       // x, b, D^-1 (nrows each), z (4 doubles a node of 3 DOFs, else 1)
     uint8_t *cg_free = nullptr; // nrows: DOF solved for
     int32_t *cg_snode = nullptr, *cg_sbase = nullptr, *cg_cta = nullptr, *cg_col = nullptr;  // slice plan
     double *cg_val = nullptr;   // the matrix of a solve in slice order
     double *cg_vec = nullptr;   // vectors in slice order when shared memory does not hold them
     void *cg_slots = nullptr;   // words of the grid-wide sums
     unsigned long long cg_epoch = 0;  // number of the last grid-wide sum given out
+    unsigned cg_spins = 1u << 22;     // polls of a grid-wide wait at most (seconds)
     int cg_grid = 0, cg_S = 1, cg_warps = 1;
     int64_t cg_slices = 0, cg_steps = 0;
     bool cg_resident = false;   // shared memory keeps the matrix,
@@ -365,7 +366,7 @@ int launch_dyn_mass_edited(Ctx *c, const int32_t *edited, int64_t m, const int64
                            int64_t cap, cudaStream_t s);
 int cg_alloc(Ctx *c);                              // sta_cg.cu
 int launch_cg_solve(Ctx *c, const double *val, const double *mass, double h2, double tol,
-                    int32_t max_iter, bool stagnate, double *xout, bool advance, cudaStream_t s,
+                    int32_t max_iter, bool stagnate, double *xout, cudaStream_t s,
                     CgResult *res);
 int build_proxy_maps(Ctx *c, const int32_t *tblk, cudaStream_t s);  // sta_proxy.cu
 int launch_proxy_rebuild(Ctx *c, cudaStream_t s);
