@@ -421,6 +421,9 @@ int sta_dyn_set_state(sta_ctx *ctx, const double *u, const double *v, int on_dev
  * reductions: deterministic).  Synchronises `stream`.  *iters and *rel_res (||r|| / ||b_f||
  * from the recurrence) may be NULL.  Both operators.  STA_ECUDA when a grid-wide wait of the solve
  * ran out: x is as it was.
+ * The first solve of a context (or sta_dyn_setup) allocates its working set: a copy of the matrix
+ * (76 bytes per node-pair block, 12 for the proxy operator; the rows of 32 or 8 nodes padded to the
+ * longest of them) and some vectors.
  *
  * sta_outer_grad -- the adjoint rule of such a solve: grad_val[k] = -lam[row(k)] u[col(k)]
  * for entries k between free DOFs, 0 elsewhere (lam, u: device nrows doubles; free: device

@@ -663,7 +663,22 @@ int cg_alloc(Ctx *c) {
     // with quads, 13,600 with lanes; 750 nodes an SM: 68,700 with quads, 62,400 with lanes
     // (scalar operator: 18,200 and 8,700).
     const int64_t per_sm = (n + c->num_sms - 1) / c->num_sms;
-    const int S = per_sm < 384 ? 4 : 1, per = 32 / S;
+    int S = per_sm < 384 ? 4 : 1;
+    // A warp works alone on a row far longer than the rest, 970 cycles a step (scalar: 110); where a lane's
+    // steps of it take longer than a CTA's whole product with quads (64 cycles an FP64 instruction of a
+    // quadrant), quads, which take a quarter of them.  Iterations, us, with lanes / quads, by the longest
+    // row: 453 nodes an SM, 30 blocks 33 / 35, 60: 42 / 40, 300: 152 / 66; 774 an SM, 60: 51 / 59, 100:
+    // 69 / 64, 300: 167 / 89; scalar, 774 an SM, 100: 16 / 22, 200: 24 / 24, 1000: 74 / 36.
+    if (S == 1) {
+        const int maxg = std::min(c->num_sms, CG_MAX_GRID);
+        int64_t longest = 0, quads = 0;
+        for (int64_t a = 0; a < n; ++a) {
+            longest = std::max<int64_t>(longest, ap[a + 1] - ap[a]);
+            quads += B * B * (int64_t)((ap[a + 1] - ap[a] + 3) / 4) + 10;
+        }
+        if (longest * (B == 3 ? 970 : 110) > quads / 8 / maxg / 4 * 64) S = 4;
+    }
+    const int per = 32 / S;
     const int64_t want = (n + per - 1) / per;
     const int maxg = std::min(c->num_sms, CG_MAX_GRID);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, maxg));

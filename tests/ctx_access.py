@@ -25,6 +25,11 @@ void ctx_delete(void *p) {
 void ctx_set_fault(void *p, unsigned int v) {
     *reinterpret_cast<volatile unsigned int *>(static_cast<sta_ctx *>(p)->c.h_fault) = v;
 }
+// lanes per node of the solve's plan (0: no plan yet)
+int ctx_plan_lanes(void *p) {
+    const sta::Ctx &c = static_cast<sta_ctx *>(p)->c;
+    return c.cg ? c.cg_S : 0;
+}
 // polls of a solve's grid-wide waits at most
 void ctx_set_spins(void *p, unsigned int n) { static_cast<sta_ctx *>(p)->c.cg_spins = n; }
 unsigned int ctx_fault(void *p) {
@@ -44,6 +49,7 @@ def load(directory):
     L.ctx_new.restype = C.c_void_p
     L.ctx_delete.argtypes = [C.c_void_p]
     L.ctx_set_fault.argtypes = [C.c_void_p, C.c_uint]
+    L.ctx_plan_lanes.argtypes = [C.c_void_p]
     L.ctx_set_spins.argtypes = [C.c_void_p, C.c_uint]
     L.ctx_fault.argtypes = [C.c_void_p]
     L.ctx_fault.restype = C.c_uint
