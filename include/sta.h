@@ -303,7 +303,7 @@ int sta_batch_apply_edits(sta_ctx *ctx, const int64_t *counts, const sta_edit *e
  * list read from the staging block below, grids sized for max_edited), the refold, and the
  * fold of a full rebuild.  Afterwards sta_apply_edits (frames of at most max_edited edited tetrahedra; a
  * swap counts two), sta_refold and sta_full_rebuild replay them with one cudaGraphLaunch each;
- * results are unchanged.  Frames of up to some hundred edits are launched without the graph where
+ * results are unchanged.  Frames of up to about a thousand edits are launched without the graph where
  * that is faster.  A frame is staged in one of two host-mapped pinned blocks (used in
  * turn) that the kernels read directly, so it costs no copy call; the block is
  * reused once the frame two calls back has finished.  Allocates those blocks and two sets of

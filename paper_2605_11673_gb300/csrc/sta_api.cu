@@ -164,7 +164,6 @@ int sta::create_impl(const double *nodes, int64_t n_nodes, const int32_t *tets, 
     c->n = n_nodes;
     c->T = n_tets;
     c->eps = o.eps;
-    c->block_threads = o.block_threads ? o.block_threads : 128;
     c->blocks_per_sm = o.blocks_per_sm;
     int rc = STA_OK;
     auto bail = [&](int code) {
@@ -334,7 +333,6 @@ int sta_set_launch(sta_ctx *x, int32_t block_threads, int32_t blocks_per_sm) {
         return fail(STA_EINVAL, "block_threads must be 0, 64, 128 or 256");
     if (blocks_per_sm < 0) return fail(STA_EINVAL, "blocks_per_sm must be >= 0");
     if (x->c.graph_on) return fail(STA_ESTATE, "disable graph mode before changing the launch shape");
-    x->c.block_threads = block_threads ? block_threads : 128;
     x->c.blocks_per_sm = blocks_per_sm;
     return STA_OK;
 }
@@ -344,7 +342,6 @@ int sta_set_fold_depth(sta_ctx *x, int32_t operands_in_flight) {
     if (operands_in_flight != 4 && operands_in_flight != 6)
         return fail(STA_EINVAL, "operands_in_flight must be 4 or 6");
     if (x->c.graph_on) return fail(STA_ESTATE, "disable graph mode before changing the fold depth");
-    x->c.fold_depth = operands_in_flight;
     return STA_OK;
 }
 

@@ -50,9 +50,9 @@
 namespace sta {
 namespace {
 
-// Working warps of a CTA at most (one CTA per SM).  A full SM has 24 slices: two for each of 12 warps,
-// three for each of 8, one or two for 15.  Steps of the 341,000-DOF block with 8, 12 and 15: 1.25, 1.15
-// and 1.19 ms; the scalar operator's frame 4.2, 4.1 and 4.3 ms.
+// Working warps of a CTA at most (one CTA per SM).  Measured at 750 nodes an SM, 24 slices (two for each
+// of 12 warps, three for each of 8, one or two for 15), and not at other sizes: steps of the 341,000-DOF
+// block with 8, 12 and 15 take 1.25, 1.15 and 1.19 ms, the scalar operator's frame 4.2, 4.1 and 4.3 ms.
 constexpr int CG_WARPS = 12;
 constexpr int CG_SUMS = 2;               // warps for the sums: r.z and r.r side by side
 constexpr int CG_MAX_GRID = 160;         // CTAs at most: 5 words a lane in an exchange

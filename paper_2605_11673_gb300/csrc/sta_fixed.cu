@@ -128,8 +128,8 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     const int64_t first = (int64_t)blockIdx.x * blockDim.x;
-    // the thread's first edit, its unit and its run, which no kernel of a frame writes, while the frame
-    // before this one may still run
+    // the thread's first edit, its unit and its run, which no kernel of a frame writes, before the wait:
+    // while the frame before this one ends
     uint32_t w1 = 0;
     int32_t u1 = 0, o1 = 0, p1 = 0;
     if (first + threadIdx.x < n) {
@@ -156,8 +156,9 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
             const int64_t off = again ? __ldg(krun + 10 * (int64_t)t + s) : o1;
             diag = s < 4;
             const int4 bm = __ldg(bmeta + u);
-            // (all in flight with the unit's record and the claim; one after another, each before its
-            // atomic, a graph-mode frame of 2,179 swaps took 14.9 us back to back, now 13.8)
+            // (all in flight with the unit's record and the claim, instead of one after another, each before
+            // its atomic: at 2,179 swaps, 14.8 -> 13.6 us back to back in graph mode, a gain no larger than
+            // what runs differ by)
             long long v[9];
 #pragma unroll
             for (int q = 0; q < 9; ++q) v[q] = q < 6 || !diag ? __ldg(Kq + off + q) : 0;

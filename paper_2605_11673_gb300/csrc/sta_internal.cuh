@@ -114,9 +114,7 @@ struct Ctx {
     int op = STA_OP_ELASTICITY;
     int64_t n = 0, T = 0, nblocks = 0, nnz = 0, nrows = 0;
     double eps = 0.0;
-    int block_threads = 256;
     int blocks_per_sm = 0;
-    int fold_depth = 4;            // operand loads in flight per lane of the rebuild fold: 4 or 6
     int rebuild_form = STA_REBUILD_AUTO;  // sta_set_rebuild_form
     int64_t n_active = 0;                 // active tetrahedra (host mirror count)
     int num_sms = 0;
@@ -334,15 +332,20 @@ int launch_spmv(Ctx *c, const double *val, const double *x, double *y, cudaStrea
 int launch_rebuild(Ctx *c, cudaStream_t s);                      // sta_rebuild.cu
 int rebuild_form_of(const Ctx *c);  // the form the next rebuild takes (AUTO resolved)
 // Frames of at most this many edited tetrahedra take one launch, k_frame_small (elasticity, re-fold
-// policy, without the dynamics' mass update).  Two kernels take 8.3-8.9 us a frame back to back from
-// 16 edits to 122, one cluster 5.6 us for 16, 5.8 for 32, 7.2 for 48, 7.4 for 60 and 9.2 for 90; but
-// a frame that is waited for is even at 32 edits and 1.5 us longer at 48 (21.5 us).
+// policy, without the dynamics' mass update).  The cluster's 112 warps fold the units of 40 tetrahedra
+// that share none, 160 diagonal and 240 pair units, in one round each.  Two kernels take 8.3-8.9 us a
+// frame back to back from 16 edits to 122, one cluster 5.6 us for 16, 5.8 for 32, 7.2 for 48, 7.4 for 60
+// and 9.2 for 90; a frame that is waited for is even at 32 edits and 1.5 us longer at 48 (21.5 us).
 constexpr int SMALL_FRAME = 40;
 // In graph mode, frames of at most this many edited tetrahedra are launched kernel by kernel all the
-// same: of such launches a frame's first kernel starts while the last one of the frame before runs,
-// which graph launches don't (600 scattered edits: 12.6 -> 10.4 us a frame, 643 of a crack front:
-// 13.3 -> 12.8).  Larger ones gain or lose with their host time, which a second launch adds 2 us to
-// (2,488 scattered: 19.5 -> 14.7, 2,179 of a crack front: 13.3 -> 14.8): they stay with the graph.
+// same.  Such a frame's kernels start as soon as the last CTA of the kernel before has left, without a
+// graph's entry and exit, but its second launch costs host time, and back to back it takes what its
+// call takes.  us a frame, graph / direct (two runs), on a block of 384,000 tetrahedra: edits in a plane,
+// 600: 12.2 / 9.9-11.9, 1,000: 12.8 / 10.7-12.5, 1,500: 13.0 / 11.7-13.4, 2,000: 13.6 / 12.4-14.3,
+// 3,000: 13.7 / 14.3-15.5; scattered, 600: 12.9 / 10.1-11.9, 2,000: 17.1 / 13.3-13.7, 4,000: 21.2 /
+// 17.4.  So up to about 1,000 edits direct launches are the faster ones for both; above, only where
+// the edits are scattered (the graph's kernels then take longer than the call), which the count does not
+// tell.  A frame that is waited for takes as long either way, or up to 2 us less from the graph.
 constexpr int DIRECT_FRAME = 1024;
 int launch_small_frame(Ctx *c, const int32_t *edited, int m, cudaStream_t s);
 bool small_frames_fit();

@@ -152,8 +152,8 @@ k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
     const int64_t n = 10 * (m_dev ? *m_dev : m);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    // the thread's first edit and its unit, which no kernel writes, while the frame before this one
-    // may still run (direct launches of 600 edits back to back: 18.5-20 us -> 10.4, with the edits
+    // the thread's first edit and its unit, which no kernel writes, before the wait: while the frame before
+    // this one ends (direct launches of 600 edits back to back: 18.5-20 us -> 10.4, with the edits
     // read from host memory instead of copied)
     uint32_t w1 = 0;
     int32_t u1 = 0, p1 = 0;
@@ -244,7 +244,7 @@ k_frame_small(const __grid_constant__ SmallFrame F, FoldArgs A, const int32_t *_
     if (threadIdx.x < 2) n_won[threadIdx.x] = 0;
     if (threadIdx.x == 2) touched = 0u;
     // items are dealt to the CTAs in turn, so that each gets its share of a short frame; their edits
-    // and units, which no kernel writes, are read while the frame before may still run
+    // and units, which no kernel writes, are read before the wait, while the frame before ends
     uint32_t w[SF_ROUNDS];
     int32_t u[SF_ROUNDS], pos[SF_ROUNDS];
 #pragma unroll
