@@ -15,13 +15,15 @@ program those captures run.  Measurement tooling beside bench.py, not part of th
         e.g. active tetrahedra, for per-unit figures) -- recorded as <key>_<workload> with the
         hash of the sources the kernels and their data layout are built from
         (KERNEL_SOURCES[key]): bench.py uses a record only while that hash matches
-    python ncu_summary.py run <workload> [--stream] [--proxy] [--elements]
+    python ncu_summary.py run <workload> [--stream] [--proxy] [--elements] [--dynamics]
         the program to capture: one context on the workload (prefractured, refinement,
         refinement_r040; --proxy: the graph-Laplacian proxy operator), sta_full_rebuild of
         the initial mask, 3 sta_refold calls after 256 MiB L2 flushes, (--elements) the
         element kernel over the active tetrahedra and the adjoint kernel for a seeded
-        gradient, 2 launches each after a flush, and (--stream) the 24-frame edit stream
-        through sta_apply_edits without CUDA graphs, each frame after a flush
+        gradient, 2 launches each after a flush, (--stream) the 24-frame edit stream
+        through sta_apply_edits without CUDA graphs, each frame after a flush, and (--dynamics) 4
+        frames of it with an implicit-Euler step each (bench.py's: bottom face clamped, a load on the
+        top face, tolerance 1e-8)
 """
 from __future__ import annotations
 
@@ -196,7 +198,8 @@ def record(rep: str, key: str, workload: str, out_json: str, kernels: str, units
     return rec
 
 
-def run(workload: str, stream: bool = False, proxy: bool = False, elements: bool = False) -> None:
+def run(workload: str, stream: bool = False, proxy: bool = False, elements: bool = False,
+        dynamics: bool = False) -> None:
     import torch
     sys.path.insert(0, str(ROOT))
     import paper_2605_11673_gb300 as P
@@ -219,6 +222,16 @@ def run(workload: str, stream: bool = False, proxy: bool = False, elements: bool
         for _ in range(2):
             flush.zero_()
             P.sta_adjoint(asm.h, gval)
+    if dynamics and not proxy:
+        import numpy as np
+        z, hm = wl.X[:, 2], 1.0 / (40 if workload == "prefractured" else 30)
+        top = z > z.max() - 0.5 * hm
+        load = np.zeros((wl.n_nodes, 3))
+        load[top, 2] = -1e3 / max(1, int(top.sum()))
+        asm.dyn_setup(1000.0, 1e-3, load.reshape(-1), z < z.min() + 0.5 * hm)
+        for ed in wl.frames[:4]:
+            asm.apply_edits(ed)
+            print("iterations, relative residual", asm.dyn_step(tol=1e-8))
     if stream:
         for ed in wl.frames:
             flush.zero_()
@@ -237,6 +250,7 @@ def main(argv) -> None:
     a.add_argument("--stream", action="store_true")
     a.add_argument("--proxy", action="store_true")
     a.add_argument("--elements", action="store_true")
+    a.add_argument("--dynamics", action="store_true")
     sub.add_parser("launches").add_argument("csv")
     sub.add_parser("full").add_argument("report")
     a = sub.add_parser("record")
@@ -247,7 +261,7 @@ def main(argv) -> None:
     a.add_argument("--command", default="")
     args = ap.parse_args(argv)
     if args.cmd == "run":
-        run(args.workload, args.stream, args.proxy, args.elements)
+        run(args.workload, args.stream, args.proxy, args.elements, args.dynamics)
     elif args.cmd == "launches":
         print(launches(args.csv))
     elif args.cmd == "full":
