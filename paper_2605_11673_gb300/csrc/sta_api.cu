@@ -411,8 +411,7 @@ static int grow_frames(Ctx *c, int64_t cap, cudaStream_t s) {
     return STA_OK;
 }
 
-// Whether the stream records a CUDA graph of the caller's.
-static bool capturing(cudaStream_t s) {
+bool sta::capturing(cudaStream_t s) {  // (40 ns)
     cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
     return st != cudaStreamCaptureStatusNone;
@@ -566,7 +565,7 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
     if (small) {
         c->last_counters = c->counters;
         c->count_on_host = true;
-        return launch_small_frame(c, stage, (int)m, s);
+        return launch_small_frame(c, stage, (int)m, capturing(s), s);
     }
 
     // the kernels read the host-mapped block itself: no copy call
@@ -580,7 +579,7 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
         c->last_counters = cnt;
         if (m > 0 && m <= DIRECT_FRAME && two_kernels && !capturing(s))
             STA_TRY(launch_stream_frame(c, frame_edited(d), m, nullptr, cnt, m, s,
-                                        c->d_gcnt + 4 * (gb ^ 1)));
+                                        c->d_gcnt + 4 * (gb ^ 1), false));
         else
             STA_CUDA_TRY(cudaGraphLaunch(c->g_streams[gb], s));
         STA_CUDA_TRY(cudaEventRecord(c->g_done[gb], s));
@@ -596,8 +595,9 @@ int sta::apply_frame(sta_ctx *x, const sta_edit *edits, int64_t n_edits, const i
     unsigned long long *cnt = c->f_cnt + 4 * gb;
     c->last_counters = cnt;
     // (a captured frame may be replayed without the other block's frame, which zeroes these, in between)
-    if (capturing(s)) STA_CUDA_TRY(cudaMemsetAsync(cnt, 0, 4 * sizeof(unsigned long long), s));
-    STA_TRY(launch_stream_frame(c, frame_edited(d), m, nullptr, cnt, m, s, c->f_cnt + 4 * (gb ^ 1)));
+    const bool replay = capturing(s);
+    if (replay) STA_CUDA_TRY(cudaMemsetAsync(cnt, 0, 4 * sizeof(unsigned long long), s));
+    STA_TRY(launch_stream_frame(c, frame_edited(d), m, nullptr, cnt, m, s, c->f_cnt + 4 * (gb ^ 1), replay));
     STA_CUDA_TRY(cudaEventRecord(c->f_done[gb], s));
     c->f_pending[gb] = true;
     c->f_next = gb ^ 1;

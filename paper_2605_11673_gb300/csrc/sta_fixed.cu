@@ -123,7 +123,7 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
                            uint32_t *__restrict__ uext, uint8_t *__restrict__ mask,
                            int32_t *__restrict__ list,
                            unsigned long long *counters, const int4 *__restrict__ bmeta,
-                           const long long *__restrict__ Kq, long long *__restrict__ S) {
+                           const long long *__restrict__ Kq, long long *__restrict__ S, bool replay) {
     const int64_t n = 10 * (m_dev ? *m_dev : m);
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -162,7 +162,8 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
             long long v[9];
 #pragma unroll
             for (int q = 0; q < 9; ++q) v[q] = q < 6 || !diag ? __ldg(Kq + off + q) : 0;
-            won = claim_unit(ustate, uext, u, again ? __ldg(tpos + 10 * (int64_t)t + s) : p1, on != 0u);
+            won = claim_unit(ustate, uext, u, again ? __ldg(tpos + 10 * (int64_t)t + s) : p1, on != 0u,
+                             replay);
 #pragma unroll
             for (int q = 0; q < 9; ++q)
                 if (q < 6 || !diag)
@@ -203,7 +204,7 @@ __global__ void k_fx_convert(FoldArgs A, const int32_t *list, const unsigned lon
         if (diag && q >= 6) continue;
         const int2 mir = diag ? make_int2(0, 0) : __ldg(A.bmirror + u);
         fx_write(A, e, bm, mir, diag, q, S[unit_key(bm, diag, q)]);
-        if (q == 0) ustate[u].claimed = 0;
+        if (q == 0) ustate[u].claims = 0;
     }
 }
 
@@ -239,11 +240,11 @@ int launch_fx_prepare(Ctx *c, cudaStream_t s) {
 
 int launch_fx_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_dev, int64_t cap,
                     int32_t *touched, unsigned long long *counters, cudaStream_t s,
-                    unsigned long long *next_cnt) {
+                    unsigned long long *next_cnt, bool replay) {
     const int threads = FX_CLAIM_THREADS;
     STA_TRY(launch_overlapped(k_fx_claim, grid_cap(c, 10 * cap, threads), threads, 0, s, edited, m, m_dev,
                               c->tunit, c->tpos, c->krun, c->ustate, c->uext, c->mask, touched, counters,
-                              c->bmeta, c->fx_q, c->fx_s));
+                              c->bmeta, c->fx_q, c->fx_s, replay));
     return launch_overlapped(k_fx_convert, grid_cap(c, (10 * (cap > 0 ? cap : 1) + 2) / 3 * 32, 128), 128, 0, s,
                              fold_args(c), touched, counters + 1, c->fx_e, c->fx_s, c->ustate,
                              next_cnt ? next_cnt + 1 : nullptr);

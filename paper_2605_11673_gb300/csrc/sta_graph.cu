@@ -104,7 +104,7 @@ extern "C" int sta_graph_enable(sta_ctx *x, int64_t max_edited, void *stream) {
         unsigned long long *cnt = c->d_gcnt + 4 * b, *next = c->d_gcnt + 4 * (b ^ 1);
         FrameHeader *fb = c->m_gframe[b];
         if ((rc = capture(cs, [&](cudaStream_t s) {
-                 return launch_stream_frame(c, frame_edited(fb), 0, &fb->m, cnt, c->gcap, s, next);
+                 return launch_stream_frame(c, frame_edited(fb), 0, &fb->m, cnt, c->gcap, s, next, false);
              }, &c->g_streams[b])))
             return bail(rc);
     }

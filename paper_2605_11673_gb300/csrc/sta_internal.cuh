@@ -61,11 +61,12 @@ __host__ __device__ inline int32_t contrib_code(int32_t t, int la, int lb) {
 __host__ __device__ inline int32_t code_tet(int32_t code) { return (code >> 4) & 0x07ffffff; }
 
 // Activity of a unit's contributors, kept equal to the mask by every call that changes it, and the
-// claim of the streaming frame in progress.  Contributor j's bit: w0 bit j (j < 32), w1 bit j - 32
-// (j < 64), else bit j % 32 of uext[xoff + j / 32 - 2].  claimed is 0 between frames.  Every change is
-// one that may be made again (a bit set or cleared, a claim marked), so a captured frame may be replayed.
+// claims of the streaming frame in progress.  Contributor j's bit: w0 bit j (j < 32), w1 bit j - 32
+// (j < 64), else bit j % 32 of uext[xoff + j / 32 - 2].  w0 and claims are one 64-bit word to the
+// claim kernels (claim_unit); the thread that finds no claim yet has won the unit.  claims is 0 between
+// frames.
 struct __align__(16) UnitState {
-    uint32_t w0, claimed, w1, xoff;  // xoff: UNIT_NARROW for at most 64 contributors
+    uint32_t w0, claims, w1, xoff;  // xoff: UNIT_NARROW for at most 64 contributors
 };
 constexpr uint32_t UNIT_NARROW = 0xffffffffu;
 
@@ -347,20 +348,21 @@ constexpr int SMALL_FRAME = 40;
 // the edits are scattered (the graph's kernels then take longer than the call), which the count does not
 // tell.  A frame that is waited for takes as long either way, or up to 2 us less from the graph.
 constexpr int DIRECT_FRAME = 1024;
-int launch_small_frame(Ctx *c, const int32_t *edited, int m, cudaStream_t s);
+int launch_small_frame(Ctx *c, const int32_t *edited, int m, bool replay, cudaStream_t s);
 bool small_frames_fit();
 // whether a streaming frame of this context stores its touched count into h_count_mapped
 bool frame_counts_to_host(const Ctx *c);
 // one streaming frame: the edited list, its count (*m_dev, or m) and the counters; cap: edited
 // tetrahedra the grids are sized for; next_cnt: the counters the frame's last kernel zeroes for the
-// next frame, or nullptr
+// next frame, or nullptr; replay: the caller captures the frame, and may replay it as it is
 int launch_stream_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_dev,
                         unsigned long long *cnt, int64_t cap, cudaStream_t s,
-                        unsigned long long *next_cnt);  // sta_stream.cu
+                        unsigned long long *next_cnt, bool replay);  // sta_stream.cu
+bool capturing(cudaStream_t s);  // whether the stream records a CUDA graph of the caller's
 int launch_fx_prepare(Ctx *c, cudaStream_t s);                   // sta_fixed.cu
 int launch_fx_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_dev, int64_t cap,
                     int32_t *touched, unsigned long long *counters, cudaStream_t s,
-                    unsigned long long *next_cnt);
+                    unsigned long long *next_cnt, bool replay);
 int launch_mask_bits(Ctx *c, cudaStream_t s);                    // activity bits <- mask
 int launch_values(Ctx *c, cudaStream_t s);  // the operator's rebuild (elasticity or proxy)
 int launch_dyn_qmass(Ctx *c, cudaStream_t s);     // sta_dyn.cu (no-ops unless set up)

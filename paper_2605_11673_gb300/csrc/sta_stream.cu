@@ -70,7 +70,7 @@ __device__ __forceinline__ void fold_units(const FoldArgs &A, UnitState *ustate,
     }
     if (!valid) return;
     // release the claim: all claims are done, and the other lanes of the unit do not read it
-    if (q == 0) ustate[u].claimed = 0;
+    if (q == 0) ustate[u].claims = 0;
     if (DIAG) {
         // 6-run entry q = (i, j), i <= j
         const int i = q < 3 ? 0 : (q < 5 ? 1 : 2), j = q < 3 ? q : (q < 5 ? q - 2 : 2);
@@ -145,7 +145,7 @@ k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
                                const int32_t *__restrict__ tpos, UnitState *__restrict__ ustate,
                                uint32_t *__restrict__ uext, uint8_t *__restrict__ mask,
                                int32_t *__restrict__ list, int64_t cap,
-                               unsigned long long *counters) {
+                               unsigned long long *counters, bool replay) {
     // per warp of the CTA: its packed winner counts, then its offset; the CTA's base
     __shared__ unsigned long long s_cnt[CLAIM_THREADS / 32];
     __shared__ unsigned long long s_base;
@@ -179,7 +179,8 @@ k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
             if (s == 0) mask[t] = (uint8_t)on;
             u = again ? __ldg(tunit + 10 * (int64_t)t + s) : u1;
             diag = s < 4;
-            won = claim_unit(ustate, uext, u, again ? __ldg(tpos + 10 * (int64_t)t + s) : p1, on != 0u);
+            won = claim_unit(ustate, uext, u, again ? __ldg(tpos + 10 * (int64_t)t + s) : p1, on != 0u,
+                             replay);
         }
         const unsigned dball = __ballot_sync(0xffffffffu, won && diag);
         const unsigned pball = __ballot_sync(0xffffffffu, won && !diag);
@@ -234,7 +235,7 @@ __global__ void __cluster_dims__(SF_CTAS, 1, 1) __launch_bounds__(SF_THREADS)
 k_frame_small(const __grid_constant__ SmallFrame F, FoldArgs A, const int32_t *__restrict__ tunit,
               const int32_t *__restrict__ tpos, UnitState *ustate, uint32_t *uext,
               uint8_t *__restrict__ mask, unsigned long long *counters,
-              unsigned long long *host_count) {  // (the folds read ustate's and uext's words through A)
+              unsigned long long *host_count, bool replay) {  // (the folds read ustate's and uext's words through A)
     constexpr int CAP = SF_ROUNDS * SF_THREADS;
     __shared__ double stage[SF_WARPS][ENT_DEPTH * 32];
     __shared__ int32_t won[CAP];
@@ -265,7 +266,7 @@ k_frame_small(const __grid_constant__ SmallFrame F, FoldArgs A, const int32_t *_
         if (i < 10 * F.m) {
             const int s = i % 10;
             if (s == 0) mask[w[r] & 0x7fffffffu] = (uint8_t)(w[r] >> 31);
-            if (claim_unit(ustate, uext, u[r], pos[r], (w[r] >> 31) != 0u)) {
+            if (claim_unit(ustate, uext, u[r], pos[r], (w[r] >> 31) != 0u, replay)) {
                 if (s < 4) won[atomicAdd(&n_won[0], 1)] = u[r];
                 else won[CAP - 1 - atomicAdd(&n_won[1], 1)] = u[r];
             }
@@ -403,14 +404,14 @@ int launch_values(Ctx *c, cudaStream_t s) {
 // One streaming frame: claim kernel, then the fold of the touched units.  The edited count is *m_dev
 // if given (a sequence captured once and replayed for any frame up to `cap`, for which the grids are
 // sized), else m.  `next_cnt`: the counters of the next frame, which the frame's last kernel zeroes,
-// or nullptr.
+// or nullptr.  `replay`: see claim_unit.
 int launch_stream_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_dev,
                         unsigned long long *cnt, int64_t cap, cudaStream_t s,
-                        unsigned long long *next_cnt) {
+                        unsigned long long *next_cnt, bool replay) {
     if (c->op == STA_OP_PROXY)
         return launch_proxy_frame(c, edited, m, m_dev, cap, c->plist, cnt, s, next_cnt);
     if (c->policy == STA_POLICY_FIXED) {
-        STA_TRY(launch_fx_frame(c, edited, m, m_dev, cap, c->touched, cnt, s, next_cnt));
+        STA_TRY(launch_fx_frame(c, edited, m, m_dev, cap, c->touched, cnt, s, next_cnt, replay));
         return launch_dyn_mass_edited(c, edited, m, m_dev, cap, s);
     }
     const int threads = CLAIM_THREADS;
@@ -418,7 +419,7 @@ int launch_stream_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t 
     const int64_t gmax = (int64_t)c->num_sms * 16;
     g = g < 1 ? 1 : (g > gmax ? gmax : g);
     STA_TRY(launch_overlapped(k_stream_claim, (unsigned)g, threads, 0, s, edited, m, m_dev, c->tunit,
-                              c->tpos, c->ustate, c->uext, c->mask, c->touched, c->nunits, cnt));
+                              c->tpos, c->ustate, c->uext, c->mask, c->touched, c->nunits, cnt, replay));
     STA_TRY(launch_fold_list(c, c->touched, c->nunits, cnt + 1, 10 * (cap > 0 ? cap : 1), s,
                              c->d_count_mapped, next_cnt ? next_cnt + 1 : nullptr));
     return launch_dyn_mass_edited(c, edited, m, m_dev, cap, s);
@@ -443,12 +444,12 @@ bool small_frames_fit() {
 }
 
 // A frame of m <= SMALL_FRAME edited tetrahedra (tet id | new state << 31, host memory) in one launch.
-int launch_small_frame(Ctx *c, const int32_t *edited, int m, cudaStream_t s) {
+int launch_small_frame(Ctx *c, const int32_t *edited, int m, bool replay, cudaStream_t s) {
     SmallFrame F;
     F.m = m;
     std::memcpy(F.edited, edited, sizeof(int32_t) * m);
     return launch_overlapped(k_frame_small, SF_CTAS, SF_THREADS, 0, s, F, fold_args(c), c->tunit, c->tpos,
-                             c->ustate, c->uext, c->mask, c->counters, c->d_count_mapped);
+                             c->ustate, c->uext, c->mask, c->counters, c->d_count_mapped, replay);
 }
 
 bool frame_counts_to_host(const Ctx *c) {
@@ -461,11 +462,12 @@ bool frame_counts_to_host(const Ctx *c) {
 // sta_last_touched reports them.
 int launch_stream_scratch(Ctx *c, int64_t m, const int32_t *d_edited, int32_t *touched,
                           unsigned long long *counters, cudaStream_t s) {
+    const bool replay = capturing(s);
     STA_CUDA_TRY(cudaMemsetAsync(counters + 1, 0, 3 * sizeof(unsigned long long), s));
     if (m > 0 && c->op == STA_OP_PROXY) {
         STA_TRY(launch_proxy_frame(c, d_edited, m, nullptr, m, touched, counters, s, nullptr));
     } else if (m > 0 && c->policy == STA_POLICY_FIXED) {
-        STA_TRY(launch_fx_frame(c, d_edited, m, nullptr, m, touched, counters, s, nullptr));
+        STA_TRY(launch_fx_frame(c, d_edited, m, nullptr, m, touched, counters, s, nullptr, replay));
     } else if (m > 0) {
         const int threads = CLAIM_THREADS;
         const int64_t g = (10 * m + threads - 1) / threads;
@@ -474,7 +476,7 @@ int launch_stream_scratch(Ctx *c, int64_t m, const int32_t *d_edited, int32_t *t
         // memset above, and a kernel that follows a memset starts when that is done)
         STA_TRY(launch_overlapped(k_stream_claim, (unsigned)g, threads, 0, s, d_edited, m, (const int64_t *)nullptr,
                                   c->tunit, c->tpos, c->ustate, c->uext, c->mask, touched, 10 * m,
-                                  counters));
+                                  counters, replay));
         STA_TRY(launch_fold_list(c, touched, 10 * m, counters + 1, 10 * m, s, nullptr, nullptr));
     }
     if (m > 0) STA_TRY(launch_dyn_mass_edited(c, d_edited, m, nullptr, m, s));
