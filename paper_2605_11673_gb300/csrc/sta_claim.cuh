@@ -13,18 +13,18 @@ namespace {
 // Contributor j of unit u becomes active (`on`) or inactive: moves its bit and claims the unit; true for
 // the thread that claims the unit first in its frame.  The bit holds the other state (edits are
 // validated), so for j < 32 one atomic adds or subtracts it and counts the claim.  A frame that the caller
-// captures (`replay`) may find the bit where it puts it: it sets or clears it and marks the claim,
-// two atomics that may be repeated (used for every frame, they cost the refinement hierarchy's cold
+// captures (REPLAY) may find the bit where it puts it: it sets or clears it and marks the claim, two
+// atomics that may be repeated (used for every frame, they cost the refinement hierarchy's cold
 // frames 5%: 21.3 -> 22.4 us at radius 0.15).
-__device__ __forceinline__ bool claim_unit(UnitState *ustate, uint32_t *uext, int32_t u, int32_t j, bool on,
-                                           bool replay) {
+template <bool REPLAY>
+__device__ __forceinline__ bool claim_unit(UnitState *ustate, uint32_t *uext, int32_t u, int32_t j, bool on) {
     uint32_t *w = j < 32 ? &ustate[u].w0 : (j < 64 ? &ustate[u].w1 : uext + ustate[u].xoff + (j / 32 - 2));
     const uint32_t bit = 1u << (j & 31);
-    if (replay || j >= 32) {
+    if (REPLAY || j >= 32) {
         if (on) atomicOr(w, bit);
         else atomicAnd(w, ~bit);
     }
-    if (replay) return atomicExch(&ustate[u].claims, 1u) == 0u;
+    if (REPLAY) return atomicExch(&ustate[u].claims, 1u) == 0u;
     unsigned long long step = 1ull << 32;  // one claim
     if (j < 32) step = on ? step + bit : step - bit;
     return (atomicAdd(reinterpret_cast<unsigned long long *>(ustate + u), step) >> 32) == 0ull;

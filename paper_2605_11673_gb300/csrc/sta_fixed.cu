@@ -115,6 +115,7 @@ __device__ __forceinline__ void fx_write(const FoldArgs &A, const int16_t *__res
 // to the unit's integer sums (+q on activation, -q on deactivation).
 constexpr int FX_CLAIM_THREADS = 256;
 
+template <bool REPLAY>
 __global__ void __launch_bounds__(FX_CLAIM_THREADS)
 k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
                            const int64_t *__restrict__ m_dev,
@@ -123,7 +124,7 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
                            uint32_t *__restrict__ uext, uint8_t *__restrict__ mask,
                            int32_t *__restrict__ list,
                            unsigned long long *counters, const int4 *__restrict__ bmeta,
-                           const long long *__restrict__ Kq, long long *__restrict__ S, bool replay) {
+                           const long long *__restrict__ Kq, long long *__restrict__ S) {
     const int64_t n = 10 * (m_dev ? *m_dev : m);
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -162,8 +163,7 @@ k_fx_claim(const int32_t *__restrict__ edited, int64_t m,
             long long v[9];
 #pragma unroll
             for (int q = 0; q < 9; ++q) v[q] = q < 6 || !diag ? __ldg(Kq + off + q) : 0;
-            won = claim_unit(ustate, uext, u, again ? __ldg(tpos + 10 * (int64_t)t + s) : p1, on != 0u,
-                             replay);
+            won = claim_unit<REPLAY>(ustate, uext, u, again ? __ldg(tpos + 10 * (int64_t)t + s) : p1, on != 0u);
 #pragma unroll
             for (int q = 0; q < 9; ++q)
                 if (q < 6 || !diag)
@@ -242,9 +242,9 @@ int launch_fx_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t *m_d
                     int32_t *touched, unsigned long long *counters, cudaStream_t s,
                     unsigned long long *next_cnt, bool replay) {
     const int threads = FX_CLAIM_THREADS;
-    STA_TRY(launch_overlapped(k_fx_claim, grid_cap(c, 10 * cap, threads), threads, 0, s, edited, m, m_dev,
+    STA_TRY(launch_overlapped(replay ? k_fx_claim<true> : k_fx_claim<false>, grid_cap(c, 10 * cap, threads), threads, 0, s, edited, m, m_dev,
                               c->tunit, c->tpos, c->krun, c->ustate, c->uext, c->mask, touched, counters,
-                              c->bmeta, c->fx_q, c->fx_s, replay));
+                              c->bmeta, c->fx_q, c->fx_s));
     return launch_overlapped(k_fx_convert, grid_cap(c, (10 * (cap > 0 ? cap : 1) + 2) / 3 * 32, 128), 128, 0, s,
                              fold_args(c), touched, counters + 1, c->fx_e, c->fx_s, c->ustate,
                              next_cnt ? next_cnt + 1 : nullptr);

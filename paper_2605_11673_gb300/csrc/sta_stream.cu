@@ -138,6 +138,7 @@ k_fold_entries(FoldArgs A, UnitState *ustate, const int32_t *list,
 // when cap >= min(10 m, units).
 constexpr int CLAIM_THREADS = 256;
 
+template <bool REPLAY>
 __global__ void __launch_bounds__(CLAIM_THREADS)
 k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
                                const int64_t *__restrict__ m_dev,
@@ -145,7 +146,7 @@ k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
                                const int32_t *__restrict__ tpos, UnitState *__restrict__ ustate,
                                uint32_t *__restrict__ uext, uint8_t *__restrict__ mask,
                                int32_t *__restrict__ list, int64_t cap,
-                               unsigned long long *counters, bool replay) {
+                               unsigned long long *counters) {
     // per warp of the CTA: its packed winner counts, then its offset; the CTA's base
     __shared__ unsigned long long s_cnt[CLAIM_THREADS / 32];
     __shared__ unsigned long long s_base;
@@ -179,8 +180,7 @@ k_stream_claim(const int32_t *__restrict__ edited, int64_t m,
             if (s == 0) mask[t] = (uint8_t)on;
             u = again ? __ldg(tunit + 10 * (int64_t)t + s) : u1;
             diag = s < 4;
-            won = claim_unit(ustate, uext, u, again ? __ldg(tpos + 10 * (int64_t)t + s) : p1, on != 0u,
-                             replay);
+            won = claim_unit<REPLAY>(ustate, uext, u, again ? __ldg(tpos + 10 * (int64_t)t + s) : p1, on != 0u);
         }
         const unsigned dball = __ballot_sync(0xffffffffu, won && diag);
         const unsigned pball = __ballot_sync(0xffffffffu, won && !diag);
@@ -231,11 +231,12 @@ struct SmallFrame {
     int32_t edited[SMALL_FRAME];
 };
 
+template <bool REPLAY>
 __global__ void __cluster_dims__(SF_CTAS, 1, 1) __launch_bounds__(SF_THREADS)
 k_frame_small(const __grid_constant__ SmallFrame F, FoldArgs A, const int32_t *__restrict__ tunit,
               const int32_t *__restrict__ tpos, UnitState *ustate, uint32_t *uext,
               uint8_t *__restrict__ mask, unsigned long long *counters,
-              unsigned long long *host_count, bool replay) {  // (the folds read ustate's and uext's words through A)
+              unsigned long long *host_count) {  // (the folds read ustate's and uext's words through A)
     constexpr int CAP = SF_ROUNDS * SF_THREADS;
     __shared__ double stage[SF_WARPS][ENT_DEPTH * 32];
     __shared__ int32_t won[CAP];
@@ -266,7 +267,7 @@ k_frame_small(const __grid_constant__ SmallFrame F, FoldArgs A, const int32_t *_
         if (i < 10 * F.m) {
             const int s = i % 10;
             if (s == 0) mask[w[r] & 0x7fffffffu] = (uint8_t)(w[r] >> 31);
-            if (claim_unit(ustate, uext, u[r], pos[r], (w[r] >> 31) != 0u, replay)) {
+            if (claim_unit<REPLAY>(ustate, uext, u[r], pos[r], (w[r] >> 31) != 0u)) {
                 if (s < 4) won[atomicAdd(&n_won[0], 1)] = u[r];
                 else won[CAP - 1 - atomicAdd(&n_won[1], 1)] = u[r];
             }
@@ -418,8 +419,9 @@ int launch_stream_frame(Ctx *c, const int32_t *edited, int64_t m, const int64_t 
     int64_t g = (10 * cap + threads - 1) / threads;
     const int64_t gmax = (int64_t)c->num_sms * 16;
     g = g < 1 ? 1 : (g > gmax ? gmax : g);
-    STA_TRY(launch_overlapped(k_stream_claim, (unsigned)g, threads, 0, s, edited, m, m_dev, c->tunit,
-                              c->tpos, c->ustate, c->uext, c->mask, c->touched, c->nunits, cnt, replay));
+    STA_TRY(launch_overlapped(replay ? k_stream_claim<true> : k_stream_claim<false>, (unsigned)g, threads, 0, s,
+                              edited, m, m_dev, c->tunit,
+                              c->tpos, c->ustate, c->uext, c->mask, c->touched, c->nunits, cnt));
     STA_TRY(launch_fold_list(c, c->touched, c->nunits, cnt + 1, 10 * (cap > 0 ? cap : 1), s,
                              c->d_count_mapped, next_cnt ? next_cnt + 1 : nullptr));
     return launch_dyn_mass_edited(c, edited, m, m_dev, cap, s);
@@ -437,8 +439,10 @@ bool small_frames_fit() {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int clusters = 0;
-    const bool fits = cudaFuncSetAttribute(k_frame_small, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-                      cudaOccupancyMaxActiveClusters(&clusters, k_frame_small, &cfg) == cudaSuccess && clusters > 0;
+    bool fits = true;
+    for (auto kern : {k_frame_small<false>, k_frame_small<true>})
+        fits = fits && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+               cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) == cudaSuccess && clusters > 0;
     if (!fits) cudaGetLastError();
     return fits;
 }
@@ -448,8 +452,8 @@ int launch_small_frame(Ctx *c, const int32_t *edited, int m, bool replay, cudaSt
     SmallFrame F;
     F.m = m;
     std::memcpy(F.edited, edited, sizeof(int32_t) * m);
-    return launch_overlapped(k_frame_small, SF_CTAS, SF_THREADS, 0, s, F, fold_args(c), c->tunit, c->tpos,
-                             c->ustate, c->uext, c->mask, c->counters, c->d_count_mapped, replay);
+    return launch_overlapped(replay ? k_frame_small<true> : k_frame_small<false>, SF_CTAS, SF_THREADS, 0, s, F, fold_args(c), c->tunit, c->tpos,
+                             c->ustate, c->uext, c->mask, c->counters, c->d_count_mapped);
 }
 
 bool frame_counts_to_host(const Ctx *c) {
@@ -474,9 +478,10 @@ int launch_stream_scratch(Ctx *c, int64_t m, const int32_t *d_edited, int32_t *t
         // the touched list holds 10 m units (at most 10 per edited tet)
         // (the claim reads d_edited before its dependency_wait: it was copied there before the
         // memset above, and a kernel that follows a memset starts when that is done)
-        STA_TRY(launch_overlapped(k_stream_claim, (unsigned)g, threads, 0, s, d_edited, m, (const int64_t *)nullptr,
+        STA_TRY(launch_overlapped(replay ? k_stream_claim<true> : k_stream_claim<false>, (unsigned)g, threads, 0, s,
+                                  d_edited, m, (const int64_t *)nullptr,
                                   c->tunit, c->tpos, c->ustate, c->uext, c->mask, touched, 10 * m,
-                                  counters, replay));
+                                  counters));
         STA_TRY(launch_fold_list(c, touched, 10 * m, counters + 1, 10 * m, s, nullptr, nullptr));
     }
     if (m > 0) STA_TRY(launch_dyn_mass_edited(c, d_edited, m, nullptr, m, s));
